@@ -115,6 +115,8 @@ struct TableSet {
     uint32_t* table16 = nullptr;
     void* ptable = nullptr;
     int64_t* d_pplane_off = nullptr;
+    uint32_t* pairs = nullptr;
+    int64_t* d_pair_off = nullptr;
     int64_t* d_plane_off = nullptr;
     int* d_support = nullptr;
     double* d_h = nullptr;
@@ -179,6 +181,10 @@ struct gw_plan_s {
     float table_inv = 1.f;        // 2^-table_exp2
     std::vector<int64_t> pplane_off;
     int64_t* d_pplane_off = nullptr;
+    // pair tables of the 16-bit gridder (tables and visibilities of one 16-bit kind)
+    uint32_t* pairs = nullptr;
+    std::vector<int64_t> pair_off;
+    int64_t* d_pair_off = nullptr;
     int64_t* d_plane_off = nullptr;
     int* d_support = nullptr;
     double* d_h = nullptr;
@@ -195,7 +201,10 @@ struct gw_plan_s {
 namespace {
 
 void free_tables(float2* table, uint32_t* table16, void* ptable, int64_t* d_pplane_off,
-                 int64_t* d_plane_off, int* d_support, double* d_h, float* d_hf) {
+                 uint32_t* pairs, int64_t* d_pair_off, int64_t* d_plane_off, int* d_support,
+                 double* d_h, float* d_hf) {
+    dev_free(pairs);
+    dev_free(d_pair_off);
     dev_free(table);
     dev_free(table16);
     dev_free(ptable);
@@ -240,13 +249,13 @@ void plan_free(gw_plan p) {
     if (p->tabs) {
         TableSet* t = p->tabs;
         if (t->refs.fetch_sub(1) == 1) {
-            free_tables(t->table, t->table16, t->ptable, t->d_pplane_off, t->d_plane_off,
-                        t->d_support, t->d_h, t->d_hf);
+            free_tables(t->table, t->table16, t->ptable, t->d_pplane_off, t->pairs, t->d_pair_off,
+                        t->d_plane_off, t->d_support, t->d_h, t->d_hf);
             delete t;
         }
     } else {   // a plan that failed before its tables were handed to a TableSet
-        free_tables(p->table, p->table16, p->ptable, p->d_pplane_off, p->d_plane_off,
-                    p->d_support, p->d_h, p->d_hf);
+        free_tables(p->table, p->table16, p->ptable, p->d_pplane_off, p->pairs, p->d_pair_off,
+                    p->d_plane_off, p->d_support, p->d_h, p->d_hf);
     }
     dev_free(p->sc.rec);
     dev_free(p->sc.count);
@@ -553,6 +562,13 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
         GW_ALLOC(pt, (size_t)p->pplane_off[P]);
         p->ptable = pt;
     }
+    if (desc->table_dtype != GW_C64 && desc->vis_dtype == desc->table_dtype) {
+        p->pair_off.assign(1, 1);
+        for (int q = 0; q < P; ++q)
+            p->pair_off.push_back(p->pair_off[q] + pair_table_pairs(p->support[q], beta));
+        GW_ALLOC(p->pairs, (size_t)(2 * p->pair_off[P]));
+        GW_ALLOC(p->d_pair_off, (size_t)P + 1);
+    }
     // the slack after the last slice reads as zeros
     e = cudaMemset(p->table + p->plane_off[P], 0, sizeof(float2) * kTableSlack);
     if (e == cudaSuccess && p->table16)
@@ -579,6 +595,9 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
                         cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(p->d_pplane_off, p->pplane_off.data(), sizeof(int64_t) * (P + 1),
+                            cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && p->pairs)
+        e = cudaMemcpyAsync(p->d_pair_off, p->pair_off.data(), sizeof(int64_t) * (P + 1),
                             cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(p->d_support, p->support.data(), sizeof(int) * P,
@@ -618,6 +637,9 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     else
         launch_pad_tables(p->table16, desc->table_dtype, p->d_plane_off, p->d_pplane_off,
                           p->d_support, P, beta, p->pad_stride, p->ptable, s);
+    if (p->pairs)
+        launch_pair_tables(p->table16, p->d_plane_off, p->d_pair_off, p->d_support, P, beta,
+                           p->pairs, s);
     e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { plan_free(p); return cuda_fail(e, "padding kernel tables"); }
@@ -627,6 +649,8 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     t->table16 = p->table16;
     t->ptable = p->ptable;
     t->d_pplane_off = p->d_pplane_off;
+    t->pairs = p->pairs;
+    t->d_pair_off = p->d_pair_off;
     t->d_plane_off = p->d_plane_off;
     t->d_support = p->d_support;
     t->d_h = p->d_h;
@@ -635,6 +659,8 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
                (int64_t)(p->grid_tk == kTabRealF32 ? sizeof(float) : dtype_bytes(desc->table_dtype)) *
                    p->pplane_off[P] +
                (p->table16 ? (int64_t)sizeof(uint32_t) * (p->plane_off[P] + kTableSlack) : 0) +
+               (p->pairs ? (int64_t)(2 * sizeof(uint32_t)) * p->pair_off[P] +
+                               (int64_t)sizeof(int64_t) * (P + 1) : 0) +
                (int64_t)(2 * sizeof(int64_t) + sizeof(int)) * (P + 1) +
                (int64_t)(sizeof(double) + sizeof(float)) * N;
     p->tabs = t;
@@ -694,6 +720,9 @@ gw_status gw_plan_clone(gw_plan src, int64_t max_vis_per_call, void* cuda_stream
     p->table_exp2 = src->table_exp2;
     p->table_inv = src->table_inv;
     p->d_pplane_off = src->d_pplane_off;
+    p->pairs = src->pairs;
+    p->pair_off = src->pair_off;
+    p->d_pair_off = src->d_pair_off;
     p->d_plane_off = src->d_plane_off;
     p->d_support = src->d_support;
     p->d_h = src->d_h;
@@ -817,6 +846,13 @@ static bool use_direct(gw_plan p, int64_t nvis) {
     return nvis <= kDirectMaxVis && nvis * smax * smax * p->desc.npol <= kDirectMaxTaps;
 }
 
+static void set_pairs(GridArgs& a, gw_plan p) {
+    if (!p->pairs) return;
+    a.pair_table = p->pairs;
+    a.pair_off = p->d_pair_off;
+    a.pair_count = p->pair_off.back();
+}
+
 static gw_status grid_impl(gw_plan p, const double* uvw_m, const double* freq_hz, int64_t nrow,
                            int32_t nchan, const void* vis, const float* weight, void* grid,
                            void* grid_err, int64_t* n_dropped, void* cuda_stream,
@@ -916,6 +952,7 @@ static gw_status grid_impl(gw_plan p, const double* uvw_m, const double* freq_hz
         a.ntiles_u = p->geom_grid.ntu;
         a.pad_stride = p->pad_stride;
         a.ptable_elems = p->pplane_off.back();
+        set_pairs(a, p);
         {
             StageTimer t(p, kStGrid, s);
             launch_grid(a, p->num_sms, s);
@@ -1171,6 +1208,7 @@ gw_status gw_grid_vis_compressed(gw_plan p, const double* uvw_m, const double* f
         a.ntiles_u = p->geom_grid.ntu;
         a.pad_stride = p->pad_stride;
         a.ptable_elems = p->pplane_off.back();
+        set_pairs(a, p);
         {
             StageTimer t(p, kStGrid, s);
             launch_grid(a, p->num_sms, s);
@@ -1296,6 +1334,7 @@ gw_status gw_grid_vis_wstack(gw_plan p, const double* uvw_m, const double* freq_
         a.ntiles_u = g.ntu;
         a.pad_stride = p->pad_stride;
         a.ptable_elems = p->pplane_off.back();
+        set_pairs(a, p);
         a.layer_tiles = g.layer_tiles;
         a.layer_stride = (int64_t)npol * p->desc.grid_n * p->desc.grid_n;
         {
@@ -1577,6 +1616,7 @@ gw_status gw_grid_vis_devcount(gw_plan p, const double* uvw_m, const double* fre
     a.ntiles_u = p->geom_grid.ntu;
     a.pad_stride = p->pad_stride;
     a.ptable_elems = p->pplane_off.back();
+    set_pairs(a, p);
     launch_grid(a, p->num_sms, s);
     e = cudaGetLastError();
     return e == cudaSuccess ? GW_OK : cuda_fail(e, "grid launch");
@@ -1657,6 +1697,7 @@ gw_status gw_grid_vis_devcount_readback(gw_plan p, const double* uvw_m, const do
     a.ntiles_u = ntu;
     a.pad_stride = p->pad_stride;
     a.ptable_elems = p->pplane_off.back();
+    set_pairs(a, p);
     // band b: tile rows [b ntv / nb, (b + 1) ntv / nb), its work items the
     // contiguous run item_off[first tile] .. item_off[first tile of the next
     // band]; its grid rows are final once its launch ends (no other band's

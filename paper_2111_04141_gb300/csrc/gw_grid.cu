@@ -52,6 +52,26 @@ __global__ void k_pad_tables_real(const float2* __restrict__ tab, const int64_t*
     }
 }
 
+// Pair tables (layout at pair_table_pairs).
+__global__ void k_pair_tables(const uint32_t* __restrict__ tab, const int64_t* __restrict__ plane_off,
+                              const int64_t* __restrict__ pair_off, const int* __restrict__ support,
+                              int beta, uint32_t* __restrict__ pairs) {
+    const int p = blockIdx.y;
+    const int S = support[p], W = S + 1;
+    const int64_t per = (int64_t)S * W;
+    const int64_t n = 2 * (int64_t)beta * beta * per;
+    const uint32_t* src = tab + plane_off[p];
+    uint32_t* dst = pairs + 2 * pair_off[p];
+    if (p == 0 && blockIdx.x == 0 && threadIdx.x < 2) pairs[threadIdx.x] = 0u;   // the zero pair
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t oc = e / per;                     // 2 x slice + copy
+        const int rem = (int)(e - oc * per);
+        const int row = rem / W, col = rem - row * W - (int)(oc & 1);
+        dst[e] = col >= 0 && col < S ? src[(oc >> 1) * S * S + (int64_t)row * S + col] : 0u;
+    }
+}
+
 __global__ void k_weight_vis(const void* __restrict__ vis, int kind, const float* __restrict__ w,
                              int64_t n, float2* __restrict__ out) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
@@ -263,6 +283,12 @@ void launch_pad_tables(const void* tab, int kind, const int64_t* plane_off,
         k_pad_tables<uint32_t><<<dim3(256, P), 256, 0, s>>>(
             static_cast<const uint32_t*>(tab), plane_off, pplane_off, support, P, beta, SP,
             static_cast<uint32_t*>(ptab));
+    note_launch();
+}
+
+void launch_pair_tables(const uint32_t* tab, const int64_t* plane_off, const int64_t* pair_off,
+                        const int* support, int P, int beta, uint32_t* pairs, cudaStream_t s) {
+    k_pair_tables<<<dim3(256, P), 256, 0, s>>>(tab, plane_off, pair_off, support, beta, pairs);
     note_launch();
 }
 

@@ -59,32 +59,43 @@
 //   visibilities of any kind are widened to FP32 when staged; all
 //   accumulation is FP32.  With an error grid the commit is compensated
 //   (commit_compensated).
+// * Where tables and visibilities are of one 16-bit kind and no weights are
+//   given, the compute warps are MmaWarp instead of FmaWarp: the same
+//   producers, tiles and hand-over, the products on the tensor cores.  An
+//   FP32 warp issues 32 packed FMAs (two issue slots each) and about 40 other
+//   instructions for an entry of 128 points and 4 polarisations; the tensor
+//   cores take 8 entries with 8 products and some 120 others.  3.13 M
+//   visibilities x 4 polarisations, 8192^2, 128 planes, support 7 -> 127,
+//   bfloat16: 5.24 -> 3.16 ms (2.9e12 -> 4.8e12 point updates x pol / s).
+//   FP32 operands split in two TF32 parts (three products a row) were slower
+//   than the FMAs (4096^2 batch: 11.1 against 8.25 ms): the split and the
+//   address arithmetic cost more than the FMAs they replace.
 #pragma once
 
 #include "gw_internal.cuh"
+
+// Kernel-value register sets in flight per FP32 compute warp (measured on the
+// 4-pol w-projection batch: 16 compute warps with ring 3 beat 8 compute warps
+// with rings of 2-10 entries at 168 registers).
+#ifndef GW_GRID_RING
+#define GW_GRID_RING 3
+#endif
 
 namespace gw {
 
 namespace {
 
-constexpr int kBlockU = kGridLanesU;                      // warp block: kBlockU (u) x kBlockV (v)
-constexpr int kBlockV = 4 * kGridLanesV;
-constexpr int kBlocksU = kGridTileU / kBlockU;            // blocks per tile row
-constexpr int kComputeWarps = kBlocksU * (kGridTileV / kBlockV);
+constexpr int kComputeWarps = 16;
 #ifndef GW_GRID_PRODUCER_WARPS
 #define GW_GRID_PRODUCER_WARPS 4
 #endif
 constexpr int kProducerWarps = GW_GRID_PRODUCER_WARPS;
 constexpr int kProducerThreads = kProducerWarps * 32;
 constexpr int kThreads = (kComputeWarps + kProducerWarps) * 32;
-constexpr int kBatch = 256;
-constexpr int kPerLane = kBatch / kProducerThreads;   // rows staged by each producer thread
+constexpr int kRows = 256;                             // staged rows of a buffer
+constexpr int kPerLane = kRows / kProducerThreads;     // rows staged by each producer thread
 constexpr int kProducerBar = 1;                        // named barrier of the producer warps
 
-// entry.y: record row in the batch (bits 0-8), conjugate kernel (bit 19),
-// mask of the slots the record's rows meet (bits 20-23)
-constexpr uint32_t kZeroRow = kBatch;   // staged visibility row that is always zero
-constexpr uint32_t kConjBit = 1u << 19;
 __device__ __forceinline__ gw_index_rec load_rec(const gw_index_rec* rec, uint32_t i) {
     int4 v = __ldg(reinterpret_cast<const int4*>(rec) + i);
     return *reinterpret_cast<gw_index_rec*>(&v);
@@ -141,6 +152,10 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src)
                  : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src)
+                 : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_all;" ::: "memory");
 }
@@ -167,21 +182,11 @@ __device__ __forceinline__ void commit_compensated(float2* g, float2* err, float
     if (e.x != 0.f || e.y != 0.f) atomicAdd(err, e);
 }
 
-template <int R>
-constexpr int list_cap() { return kBatch + 2 * R; }
-
-template <int NPOL, int B, int R>
-struct Smem {
-    float2 v[B][kBatch + 1][NPOL];          // weighted visibilities; row kBatch = 0
-    // per warp: list entries, padded to a multiple of R, then R null entries
-    uint2 list[B][kComputeWarps][list_cap<R>()];
-    int cnt[B][kComputeWarps];             // entries, padded to a multiple of R
-    int tile[B];                           // tile of the batch; -1 = end of work
-    int last[B];                           // batch ends its work item
-    Item item;                             // producers: the current work item
-    int done;                              // producers: no work item left
-    unsigned long long full[B], empty[B];  // mbarriers
-};
+// ---- compute warps: FP32 FMAs --------------------------------------------------
+// List entry: x = padded-table index of the tile origin relative to the record;
+// y = record row in the batch (bits 0-8), conjugate kernel (bit 19), mask of
+// the slots the record's rows meet (bits 20-23).
+constexpr uint32_t kConjBit = 1u << 19;
 
 // Packed FMAs of one entry into slots J0..J1 (compile-time range); A = V,
 // Bv = s (-V.im, V.re) (unused for a real kernel).
@@ -241,46 +246,371 @@ __device__ __forceinline__ void load_masked(const typename TE::T* __restrict__ t
     Kd[3] = (m & 8u) ? __ldg(p_ + 3 * kGridLanesV * SP) : z;
 }
 
-// Fills the ring with the first R entries of a list.
-template <int SP, int R, class TE>
-__device__ __forceinline__ void ring_fill(const uint2* lst, const typename TE::T* __restrict__ tab,
-                                          typename TE::T (&K)[R][4], uint32_t (&ey)[R]) {
-#pragma unroll
-    for (int d = 0; d < R; ++d) {
-        const uint2 en = lst[d];
-        ey[d] = en.y;
-        load_masked<SP, TE>(tab, en, K[d]);
-    }
-}
-
-// One ring pass: the FMAs of the R entries in the ring, each followed by the
-// loads of the entry R positions later, taken from `next`.  Every entry
-// updates all four slots; the slots outside its mask add zeros (spare FMA
-// issue, but one short loop body per ring position and no per-entry jump).
-template <int NPOL, int SP, int R, class TE>
-__device__ __forceinline__ void ring_pass(const uint2* next, const float2 (*vs)[NPOL],
-                                          const typename TE::T* __restrict__ tab,
-                                          typename TE::T (&K)[R][4], uint32_t (&ey)[R],
-                                          float2 (&acc)[4][NPOL]) {
-#pragma unroll
-    for (int d = 0; d < R; ++d) {
-        float2 A[NPOL], Bv[NPOL];
-        load_v<NPOL, TE::kReal>(A, Bv, vs, ey[d]);
-        slot_fma<NPOL, 0, 3, TE>(acc, K[d], A, Bv);
-        const uint2 en = next[d];
-        ey[d] = en.y;
-        load_masked<SP, TE>(tab, en, K[d]);
-    }
-}
-
-template <int NPOL, int SP, int TK, int B, int R>
-__global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
+template <int NPOL, int SP, int TK>
+struct FmaWarp {
     using TE = TabElem<TK>;
+    using T = typename TE::T;
+    using VT = float2;                         // staged visibility
+    static constexpr int kPol = NPOL, R = GW_GRID_RING;
+    static constexpr int kBlockU = kGridLanesU, kBlockV = 4 * kGridLanesV;
+    static constexpr int kBatch = kRows;       // records staged at a time
+    static constexpr uint32_t kZeroRow = kBatch;   // staged row that is always zero
+    static constexpr int kVisRows = kBatch + 1;
+    const T* __restrict__ tab;
+    float2 acc[4][NPOL];                       // (re, im)
+    // kernel-value ring, in the table's storage kind; finite values only
+    // (zero, then table values), so the null entries' zero visibility row
+    // contributes exact zeros
+    T K[R][4];
+    uint32_t ey[R];
+
+    __device__ __forceinline__ FmaWarp(const GridArgs& a, int warp, int lane) {
+        constexpr int blocks = kGridTileU / kBlockU;
+        const int bu = (warp % blocks) * kBlockU, bv = (warp / blocks) * kBlockV;
+        tab = reinterpret_cast<const T*>(a.ptable) + (bv + lane / kGridLanesU) * SP + bu +
+              lane % kGridLanesU;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) acc[j][p] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int d = 0; d < R; ++d)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) K[d][j] = T{};
+    }
+    // Fills the ring with the first R entries of a list.
+    __device__ __forceinline__ void fill(const uint2* lst, const VT (*)[NPOL]) {
+#pragma unroll
+        for (int d = 0; d < R; ++d) {
+            const uint2 en = lst[d];
+            ey[d] = en.y;
+            load_masked<SP, TE>(tab, en, K[d]);
+        }
+    }
+    // One ring pass: the FMAs of the R entries in the ring, each followed by the
+    // loads of the entry R positions later, taken from `next`.  Every entry
+    // updates all four slots; the slots outside its mask add zeros (spare FMA
+    // issue, but one short loop body per ring position and no per-entry jump).
+    __device__ __forceinline__ void pass(const uint2* next, const VT (*vs)[NPOL], const VT (*)[NPOL]) {
+#pragma unroll
+        for (int d = 0; d < R; ++d) {
+            float2 A[NPOL], Bv[NPOL];
+            load_v<NPOL, TE::kReal>(A, Bv, vs, ey[d]);
+            slot_fma<NPOL, 0, 3, TE>(acc, K[d], A, Bv);
+            const uint2 en = next[d];
+            ey[d] = en.y;
+            load_masked<SP, TE>(tab, en, K[d]);
+        }
+    }
+    // Commits the block's accumulators at (u0, v0) of `gbase` and clears them.
+    __device__ __forceinline__ void commit(const GridArgs& a, float2* gbase, int u0, int v0, int lane) {
+        const int N = a.N, u = u0 + lane % kGridLanesU;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int v = v0 + lane / kGridLanesU + kGridLanesV * j;
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) {
+                if (u < N && v < N && (acc[j][p].x != 0.f || acc[j][p].y != 0.f)) {
+                    const float2 val = make_float2(acc[j][p].x * a.table_inv,
+                                                   acc[j][p].y * a.table_inv);
+                    const int64_t off = ((int64_t)p * N + v) * N + u;
+                    if (a.grid_err) {
+                        commit_compensated(gbase + off, a.grid_err + off, val);
+                    } else {
+                        atomicAdd(gbase + off, val);
+                    }
+                }
+                acc[j][p] = make_float2(0.f, 0.f);
+            }
+        }
+    }
+    // Producer: visibility `id` (weighted) into a staged row.
+    static __device__ __forceinline__ void stage(const GridArgs& a, bool copy, VT (&row)[NPOL],
+                                                 uint32_t id) {
+        if (copy) {
+            const float2* src = reinterpret_cast<const float2*>(a.vis) + (int64_t)id * NPOL;
+            if (NPOL % 2 == 0) {
+#pragma unroll
+                for (int p = 0; p < NPOL; p += 2) cp_async16(&row[p], src + p);
+            } else {
+#pragma unroll
+                for (int p = 0; p < NPOL; ++p) cp_async8(&row[p], src + p);
+            }
+        } else {
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) {
+                float2 v = load_vis(a.vis, a.vis_kind, (int64_t)id * NPOL + p);
+                if (a.weight) {
+                    const float w = __ldg(a.weight + (int64_t)id * NPOL + p);
+                    v.x *= w;
+                    v.y *= w;
+                }
+                row[p] = v;
+            }
+        }
+    }
+    // visibilities copied as they are: FP32 pairs without weights, with
+    // the 16-byte alignment the 16-byte copies need (pairs of polarisations)
+    static __device__ __forceinline__ bool copies(const GridArgs& a) {
+        return a.vis_kind == GW_C64 && a.weight == nullptr &&
+               (NPOL % 2 == 1 || reinterpret_cast<uintptr_t>(a.vis) % 16 == 0);
+    }
+    // Producer: list entries of a record (staged row r, footprint lower corner
+    // (ulo, vlo) and upper corner relative to the tile).
+    struct Entries {
+        uint32_t base, ey;
+        __device__ __forceinline__ Entries(const GridArgs& a, const gw_index_rec& rc, int plane, int S,
+                                           int r, int ulo, int vlo) {
+            const int64_t slice = __ldg(a.pplane_off + plane) +
+                                  ((int64_t)(rc.ov + a.beta / 2) * a.beta + (rc.ou + a.beta / 2)) *
+                                      (int64_t)(S + 2 * kGridPadR) * SP;
+            // padded index of the tile origin relative to this record
+            base = (uint32_t)((int)slice + (kGridPadR - vlo) * SP + kGridPadC - ulo);
+            ey = (uint32_t)r | ((rc.flags & GW_FLAG_CONJ) ? kConjBit : 0u);
+        }
+        // entry of block (cu, cv), whose rows j0 .. j1 the footprint meets
+        __device__ __forceinline__ uint2 operator()(int, int, int j0, int j1) const {
+            const uint32_t mask = ((2u << (j1 / kGridLanesV)) - 1u) & ~((1u << (j0 / kGridLanesV)) - 1u);
+            return make_uint2(base, ey | (mask << 20));
+        }
+        // first and last table element the entry's loads touch
+        __device__ __forceinline__ void span(uint2, int cu, int cv, int j0, int j1, int64_t& lo,
+                                             int64_t& hi) const {
+            j0 = j0 / kGridLanesV * kGridLanesV;
+            j1 = j1 / kGridLanesV * kGridLanesV + kGridLanesV - 1;
+            lo = (int64_t)(int)base + (int64_t)(kBlockV * cv + j0) * SP + kBlockU * cu;
+            hi = (int64_t)(int)base + (int64_t)(kBlockV * cv + j1) * SP + kBlockU * cu + kBlockU - 1;
+        }
+    };
+};
+
+// ---- compute warps: 16-bit tensor cores -----------------------------------------
+// Tables and visibilities of one 16-bit kind: the products of 16-bit values
+// are exact in FP32, so a group of 8 records is one m16n8k16 product per
+// block row: rows of A the row's 16 points, K index the records' (re, im)
+// kernel values as stored, columns of B the components (re, im) of the
+// polarisations.  Its FP32 sums are added to the lane's accumulators with
+// ordinary (rounded) additions.  Lane (g, t) = (lane / 4, lane % 4) loads
+// column pair g of records t and t + 4 and holds polarisation t of points 2 g,
+// 2 g + 1; pairs come from the pair tables (layout at pair_table_pairs).
+//
+// List entry: x = pair index of the block's column 0, row 0 (modulo 2^32; only
+// columns and rows inside the footprint are loaded); y = record row in the
+// batch (bits 0-7), pairs per table row less one (8-14), conjugate kernel
+// (15), rows (16-23) and column pairs (24-31) that the footprint meets.
+constexpr uint32_t kMmaConj = 1u << 15;
+constexpr int kMmaRows = 16, kMmaCols = 24;
+
+template <int TK>
+__device__ __forceinline__ void mma_16(float (&d)[4], const uint32_t (&a)[4],
+                                       const uint32_t (&b)[2]) {
+    if constexpr (TK == GW_BF16X2)
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+            "{%8,%9}, {%10,%10,%10,%10};"
+            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.f));
+    else
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+            "{%8,%9}, {%10,%10,%10,%10};"
+            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.f));
+}
+
+template <int NPOL, int TK>
+struct MmaWarp {
+    using VT = uint32_t;                       // staged visibility, as stored
+    static constexpr int kPol = NPOL, R = 8;   // records per group, one group in flight
+    static constexpr int kBlockU = 16, kBlockV = 8;
+    static constexpr int kBatch = kRows - 1;   // rows 0 .. 254, and the zero row 255
+    static constexpr uint32_t kZeroRow = kBatch;
+    static constexpr int kVisRows = kRows;
+    float acc[8][4];                           // block row; point 2 g (re, im), point 2 g + 1
+    uint2 K[8][2];
+    uint32_t b[2];                             // operand B of the group in flight
+    const uint2* __restrict__ tab;
+    uint32_t g, t;
+
+    __device__ __forceinline__ MmaWarp(const GridArgs& a, int, int lane) {
+        tab = reinterpret_cast<const uint2*>(a.pair_table);
+        g = lane >> 2;
+        t = lane & 3;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[j][i] = 0.f;
+    }
+    // position, row step and row mask of the lane's two records
+    struct Cursor {
+        uint32_t off[2], q[2], m[2];
+    };
+    __device__ __forceinline__ Cursor start(const uint2* lst, const VT (*vs)[NPOL]) {
+        Cursor c;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint2 en = lst[4 * k + t];
+            c.off[k] = en.x + g;
+            c.q[k] = ((en.y >> 8) & 0x7fu) + 1u;
+            c.m[k] = (en.y >> (kMmaCols + g)) & 1u ? en.y >> kMmaRows : 0u;
+            // column g of B: component (re, im) g & 1 of polarisation g / 2;
+            // (K.re, K.im) multiply (V.re, -s V.im) or (V.im, s V.re), s = -1 for
+            // the conjugate kernel
+            uint32_t w = 0u;
+            if (NPOL == 4 || (int)(g >> 1) < NPOL) {
+                w = vs[en.y & 0xffu][g >> 1];
+                w = __byte_perm(w, 0, (g & 1) ? 0x1032 : 0x3210) ^
+                    ((~g << 31) ^ ((en.y & kMmaConj) << 16));
+            }
+            b[k] = w;
+        }
+        return c;
+    }
+    // lanes outside the footprint read a zero pair (a select of the address:
+    // 16 predicated loads with zeroed destinations do not fit the registers)
+    __device__ __forceinline__ void load(int j, Cursor& c) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            K[j][k] = __ldg(tab + (c.m[k] & (1u << j) ? c.off[k] : 0u));
+            c.off[k] += c.q[k];
+        }
+    }
+    __device__ __forceinline__ void fill(const uint2* lst, const VT (*vs)[NPOL]) {
+        Cursor c = start(lst, vs);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) load(j, c);
+    }
+    // one pass: the products of the group in flight, each row followed by its
+    // loads for the next group
+    __device__ __forceinline__ void pass(const uint2* next, const VT (*)[NPOL], const VT (*nvs)[NPOL]) {
+        const uint32_t bc[2] = {b[0], b[1]};
+        Cursor c = start(next, nvs);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t a[4] = {K[j][0].x, K[j][0].y, K[j][1].x, K[j][1].y};
+            float d[4];
+            mma_16<TK>(d, a, bc);
+#pragma unroll
+            for (int i = 0; i < 4; i += 2) {
+                const float2 q = __fadd2_rn(make_float2(acc[j][i], acc[j][i + 1]),
+                                            make_float2(d[i], d[i + 1]));
+                acc[j][i] = q.x;
+                acc[j][i + 1] = q.y;
+            }
+            load(j, c);
+        }
+    }
+    // Commits the block's accumulators; both points of a pair in one 16-byte
+    // reduction where the grid's alignment allows (N and the blocks are even).
+    // Lanes of polarisations beyond NPOL hold zeros.
+    __device__ __forceinline__ void commit(const GridArgs& a, float2* gbase, int u0, int v0, int) {
+        const int N = a.N, u = u0 + 2 * (int)g;
+        const bool vec = (reinterpret_cast<uintptr_t>(gbase) & 15u) == 0 && a.grid_err == nullptr;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int v = v0 + j;
+            const float4 q = make_float4(acc[j][0] * a.table_inv, acc[j][1] * a.table_inv,
+                                         acc[j][2] * a.table_inv, acc[j][3] * a.table_inv);
+            const bool n0 = q.x != 0.f || q.y != 0.f, n1 = q.z != 0.f || q.w != 0.f;
+            if ((int)t < NPOL && u < N && v < N && (n0 || n1)) {
+                const int64_t off = ((int64_t)t * N + v) * N + u;
+                const float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
+                if (vec) {
+                    atomicAdd(reinterpret_cast<float4*>(gbase + off), q);
+                } else if (a.grid_err) {
+                    if (n0) commit_compensated(gbase + off, a.grid_err + off, q0);
+                    if (n1) commit_compensated(gbase + off + 1, a.grid_err + off + 1, q1);
+                } else {
+                    if (n0) atomicAdd(gbase + off, q0);
+                    if (n1) atomicAdd(gbase + off + 1, q1);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[j][i] = 0.f;
+        }
+    }
+    static __device__ __forceinline__ bool copies(const GridArgs& a) {
+        return NPOL % 2 == 1 || reinterpret_cast<uintptr_t>(a.vis) % (4 * NPOL) == 0;
+    }
+    // Producer: visibility `id` into a staged row, with the widest copies its
+    // alignment allows.
+    static __device__ __forceinline__ void stage(const GridArgs& a, bool copy, VT (&row)[NPOL],
+                                                 uint32_t id) {
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(a.vis) + (int64_t)id * NPOL;
+        if (copy && NPOL == 4) {
+            cp_async16(&row[0], src);
+        } else if (copy && NPOL == 2) {
+            cp_async8(&row[0], src);
+        } else if (copy) {
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) cp_async4(&row[p], src + p);
+        } else {
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) row[p] = __ldg(src + p);
+        }
+    }
+    struct Entries {
+        uint32_t base, ey;
+        int Q, pc0;
+        __device__ __forceinline__ Entries(const GridArgs& a, const gw_index_rec& rc, int plane, int S,
+                                           int r, int ulo, int vlo) {
+            Q = (S + 1) / 2;                       // pairs per table row
+            // the copy of the slice whose pairs line up with the tile's even
+            // columns, and the pair column of the tile's column 0
+            const int odd = ulo & 1;
+            pc0 = (odd - ulo) / 2;
+            const int64_t slice =
+                __ldg(a.pair_off + plane) +
+                (2 * ((int64_t)(rc.ov + a.beta / 2) * a.beta + (rc.ou + a.beta / 2)) + odd) *
+                    (int64_t)(S * Q);
+            base = (uint32_t)slice + (uint32_t)(pc0 - vlo * Q);
+            ey = (uint32_t)r | (uint32_t)(Q - 1) << 8 | ((rc.flags & GW_FLAG_CONJ) ? kMmaConj : 0u);
+        }
+        __device__ __forceinline__ uint2 operator()(int cu, int cv, int j0, int j1) const {
+            const int pc = pc0 + kBlockU / 2 * cu;
+            const int lo = max(0, -pc), hi = min(kBlockU / 2 - 1, Q - 1 - pc);
+            const uint32_t rows = ((2u << j1) - 1u) & ~((1u << j0) - 1u);
+            const uint32_t cols = (2u << hi) - (1u << lo);
+            return make_uint2(base + (uint32_t)(kBlockV * cv * Q + kBlockU / 2 * cu),
+                              ey | rows << kMmaRows | cols << kMmaCols);
+        }
+        // first and last pair the entry's loads touch
+        __device__ __forceinline__ void span(uint2 e, int cu, int, int j0, int j1, int64_t& lo,
+                                             int64_t& hi) const {
+            const int pc = pc0 + kBlockU / 2 * cu;
+            lo = (int64_t)(uint32_t)(e.x + (uint32_t)(j0 * Q + max(0, -pc)));
+            hi = (int64_t)(uint32_t)(e.x + (uint32_t)(j1 * Q + min(kBlockU / 2 - 1, Q - 1 - pc)));
+        }
+    };
+};
+
+template <int NPOL, int SP, int TK, bool NAT>
+struct PickWarp { using W = FmaWarp<NPOL, SP, TK>; };
+template <int NPOL, int SP, int TK>
+struct PickWarp<NPOL, SP, TK, true> { using W = MmaWarp<NPOL, TK>; };
+
+template <class W, int B>
+struct Smem {
+    typename W::VT v[B][W::kVisRows][W::kPol];   // staged visibilities; row kZeroRow = 0
+    // per warp: list entries, padded to a multiple of R, then R null entries
+    uint2 list[B][kComputeWarps][kRows + 2 * W::R];
+    int cnt[B][kComputeWarps];             // entries, padded to a multiple of R
+    int tile[B];                           // tile of the batch; -1 = end of work
+    int last[B];                           // batch ends its work item
+    Item item;                             // producers: the current work item
+    int done;                              // producers: no work item left
+    unsigned long long full[B], empty[B];  // mbarriers
+};
+
+template <int NPOL, int SP, int TK, bool NAT, int B>
+__global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
+    using W = typename PickWarp<NPOL, SP, TK, NAT>::W;
+    using VT = typename W::VT;
+    constexpr int R = W::R, kBatch = W::kBatch, kBlockU = W::kBlockU, kBlockV = W::kBlockV;
+    constexpr int kBlocksU = kGridTileU / kBlockU;
+    constexpr uint32_t kZeroRow = W::kZeroRow;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    Smem<NPOL, B, R>& sm = *reinterpret_cast<Smem<NPOL, B, R>*>(smem_raw);
+    Smem<W, B>& sm = *reinterpret_cast<Smem<W, B>*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int side = a.ntiles_u;
-    const int hb = a.beta / 2;
 
     // one-time set-up: barriers, the zero visibility row
     if (threadIdx.x == 0) {
@@ -290,7 +620,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
         }
     }
     for (int t = threadIdx.x; t < B * NPOL; t += kThreads)
-        sm.v[t / NPOL][kZeroRow][t % NPOL] = make_float2(0.f, 0.f);
+        sm.v[t / NPOL][kZeroRow][t % NPOL] = VT{};
     __syncthreads();
 
     if (warp >= kComputeWarps) {
@@ -303,10 +633,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
         // items [i0, *item_count): a band of tile rows, or all of them
         const uint32_t i0 = a.item_first ? *a.item_first : 0u;
         const uint32_t nitems = *a.item_count - i0;
-        // visibilities copied as they are: FP32 pairs without weights, with
-        // the 16-byte alignment the 16-byte copies need (pairs of polarisations)
-        const bool copy_vis = a.vis_kind == GW_C64 && a.weight == nullptr &&
-                              (NPOL % 2 == 1 || reinterpret_cast<uintptr_t>(a.vis) % 16 == 0);
+        const bool copy_vis = W::copies(a);
         uint32_t nbatch = 0;
         for (;;) {
             int b = 0, nb_total = 1;
@@ -359,62 +686,28 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
                         if (r >= nb) break;
                         const uint32_t id = ids[k];
                         const gw_index_rec rc = rcs[k];
-                        if (copy_vis) {
-                            const float2* src = reinterpret_cast<const float2*>(a.vis) +
-                                                (int64_t)id * NPOL;
-                            if (NPOL % 2 == 0) {
-#pragma unroll
-                                for (int p = 0; p < NPOL; p += 2)
-                                    cp_async16(&sm.v[buf][r][p], src + p);
-                            } else {
-#pragma unroll
-                                for (int p = 0; p < NPOL; ++p) cp_async8(&sm.v[buf][r][p], src + p);
-                            }
-                        } else {
-#pragma unroll
-                            for (int p = 0; p < NPOL; ++p) {
-                                float2 v = load_vis(a.vis, a.vis_kind, (int64_t)id * NPOL + p);
-                                if (a.weight) {
-                                    const float w = __ldg(a.weight + (int64_t)id * NPOL + p);
-                                    v.x *= w;
-                                    v.y *= w;
-                                }
-                                sm.v[buf][r][p] = v;
-                            }
-                        }
+                        W::stage(a, copy_vis, sm.v[buf][r], id);
                         // w-stacking records carry their layer in `plane`; the
                         // kernel is the plan's single (w = 0) plane
                         const int plane = (a.layer_tiles && !a.plane_groups) ? 0 : rc.plane;
                         const int S = __ldg(a.support + plane), h = S >> 1;
-                        const int64_t slice = __ldg(a.pplane_off + plane) +
-                                              ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) *
-                                                  (int64_t)(S + 2 * kGridPadR) * SP;
-                        // padded index of the tile origin relative to this record
-                        const int base = (int)slice + (tv0 - rc.kv + h + kGridPadR) * SP +
-                                         (tu0 - rc.ku + h + kGridPadC);
-                        const uint32_t conj = (rc.flags & GW_FLAG_CONJ) ? kConjBit : 0u;
                         // footprint relative to the tile: [ulo, uhi] x [vlo, vhi]
                         const int ulo = rc.ku - h - tu0, uhi = rc.ku + h - tu0;
                         const int vlo = rc.kv - h - tv0, vhi = rc.kv + h - tv0;
+                        const typename W::Entries entry(a, rc, plane, S, r, ulo, vlo);
                         const int cu0 = max(0, ulo) / kBlockU, cu1 = min(kGridTileU - 1, uhi) / kBlockU;
                         const int cv0 = max(0, vlo) / kBlockV, cv1 = min(kGridTileV - 1, vhi) / kBlockV;
                         for (int cv = cv0; cv <= cv1; ++cv) {
-                            const int j0 = max(0, vlo - kBlockV * cv) / kGridLanesV;
-                            const int j1 = min(kBlockV - 1, vhi - kBlockV * cv) / kGridLanesV;
-                            const uint32_t mask = ((2u << j1) - 1u) & ~((1u << j0) - 1u);
-                            const uint2 e = make_uint2((uint32_t)base,
-                                                       (uint32_t)r | (mask << 20) | conj);
+                            const int j0 = max(0, vlo - kBlockV * cv);
+                            const int j1 = min(kBlockV - 1, vhi - kBlockV * cv);
                             for (int cu = cu0; cu <= cu1; ++cu) {
                                 const int w = cv * kBlocksU + cu;
+                                const uint2 e = entry(cu, cv, j0, j1);
 #ifdef GW_DEBUG_BOUNDS
-                                // the entry's loads: slots j0..j1 of the warp's block
-                                const int64_t lo = (int64_t)base + (int64_t)(kBlockV * cv + kGridLanesV * j0) * SP +
-                                                   kBlockU * cu;
-                                const int64_t hi = (int64_t)base +
-                                                   (int64_t)(kBlockV * cv + kGridLanesV * j1 + kGridLanesV - 1) * SP +
-                                                   kBlockU * cu + kBlockU - 1;
-                                if (!gw_in_bounds(a.ptable_elems == 0 || (lo >= 0 && hi < a.ptable_elems),
-                                                  a.queue + 1))
+                                int64_t lo, hi;
+                                entry.span(e, cu, cv, j0, j1, lo, hi);
+                                const int64_t n = NAT ? a.pair_count : a.ptable_elems;
+                                if (!gw_in_bounds(n == 0 || (lo >= 0 && lo <= hi && hi < n), a.queue + 1))
                                     continue;
 #endif
                                 const int pos = atomicAdd(&sm.cnt[buf][w], 1);
@@ -456,24 +749,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(GW_GRID_SETMAXNREG) : "memory");
 #endif
     const int bu = (warp % kBlocksU) * kBlockU, bv = (warp / kBlocksU) * kBlockV;
-    const int lu = lane % kGridLanesU, lv = lane / kGridLanesU;
-    const typename TE::T* __restrict__ tab =
-        reinterpret_cast<const typename TE::T*>(a.ptable) + (bv + lv) * SP + bu + lu;
-    const int N = a.N;
-    float2 acc[4][NPOL];   // (re, im)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int p = 0; p < NPOL; ++p) acc[j][p] = make_float2(0.f, 0.f);
-    // kernel-value ring, in the table's storage kind; finite values only
-    // (zero, then table values), so the null entries' zero visibility row
-    // contributes exact zeros
-    typename TE::T K[R][4];
-    uint32_t ey[R];
-#pragma unroll
-    for (int d = 0; d < R; ++d)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) K[d][j] = typename TE::T{};
+    W cw(a, warp, lane);
 
     // The ring runs across batches: the last pass over a batch's list loads
     // the first R entries of the next batch, so no batch starts with an empty
@@ -483,7 +759,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
         if (lane == 0) atomicOr(a.queue + 1, 1u);
         return;
     }
-    ring_fill<SP, R, TE>(sm.list[0][warp], tab, K, ey);
+    cw.fill(sm.list[0][warp], sm.v[0]);
     uint32_t nbatch = 0;
     for (;;) {
         const int buf = nbatch % B;
@@ -501,10 +777,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
                 return;
             }
             if (n == 0) {   // nothing of this batch for this warp
-                ring_fill<SP, R, TE>(nlst, tab, K, ey);
+                cw.fill(nlst, sm.v[nbuf]);
                 break;
             }
-            ring_pass<NPOL, SP, R, TE>(tail ? nlst : lst + i + R, sm.v[buf], tab, K, ey, acc);
+            cw.pass(tail ? nlst : lst + i + R, sm.v[buf], sm.v[tail ? nbuf : buf]);
             if (tail) break;
         }
         mbar_arrive(&sm.empty[buf]);  // buffer free (every lane, after its reads)
@@ -514,75 +790,53 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
             const int ltile = a.layer_tiles ? tile % a.layer_tiles : tile;
             float2* const gbase = a.grid + (a.layer_tiles ? (int64_t)(tile / a.layer_tiles) *
                                                                  a.layer_stride : 0);
-            const int u = (ltile % a.ntiles_u) * kGridTileU + bu + lu;
-            const int v0 = (ltile / a.ntiles_u) * kGridTileV + bv + lv;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int v = v0 + kGridLanesV * j;
-#pragma unroll
-                for (int p = 0; p < NPOL; ++p) {
-                    if (u < N && v < N && (acc[j][p].x != 0.f || acc[j][p].y != 0.f)) {
-                        const float2 val = make_float2(acc[j][p].x * a.table_inv,
-                                                       acc[j][p].y * a.table_inv);
-                        const int64_t off = ((int64_t)p * N + v) * N + u;
-                        if (a.grid_err) {
-                            commit_compensated(gbase + off, a.grid_err + off, val);
-                        } else {
-                            atomicAdd(gbase + off, val);
-                        }
-                    }
-                    acc[j][p] = make_float2(0.f, 0.f);
-                }
-            }
+            cw.commit(a, gbase, (ltile % a.ntiles_u) * kGridTileU + bu,
+                      (ltile / a.ntiles_u) * kGridTileV + bv, lane);
         }
     }
 }
 
-template <int NPOL, int SP, int TK, int B, int R>
-void launch_v(const GridArgs& a, int num_sms, cudaStream_t s) {
-    const size_t smem = sizeof(Smem<NPOL, B, R>);
-    cudaFuncSetAttribute(k_grid<NPOL, SP, TK, B, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grid<NPOL, SP, TK, B, R>, kThreads,
-                                                  smem);
-    if (per_sm < 1) per_sm = 1;
-    k_grid<NPOL, SP, TK, B, R><<<num_sms * per_sm, kThreads, smem, s>>>(a);
-    note_launch();
-}
-
-// GW_GRID_BUFS staging buffers of 256 records and a ring of GW_GRID_RING
-// kernel-value register sets per compute warp (measured on the 4-pol
-// w-projection batch: 16 compute warps with ring 3 beat 8 compute warps with
-// rings of 2-10 entries at 168 registers).
-#ifndef GW_GRID_RING
-#define GW_GRID_RING 3
-#endif
+// GW_GRID_BUFS staging buffers of 256 records.
 #ifndef GW_GRID_BUFS
 #define GW_GRID_BUFS 4
 #endif
-template <int NPOL, int SP, int TK>
+template <int NPOL, int SP, int TK, bool NAT>
 void launch_sp(const GridArgs& a, int num_sms, cudaStream_t s) {
-    launch_v<NPOL, SP, TK, GW_GRID_BUFS, GW_GRID_RING>(a, num_sms, s);
+    constexpr int B = GW_GRID_BUFS;
+    const size_t smem = sizeof(Smem<typename PickWarp<NPOL, SP, TK, NAT>::W, B>);
+    cudaFuncSetAttribute(k_grid<NPOL, SP, TK, NAT, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grid<NPOL, SP, TK, NAT, B>, kThreads,
+                                                  smem);
+    if (per_sm < 1) per_sm = 1;
+    k_grid<NPOL, SP, TK, NAT, B><<<num_sms * per_sm, kThreads, smem, s>>>(a);
+    note_launch();
 }
 
 template <int NPOL, int TK>
 void launch_t(const GridArgs& a, int num_sms, cudaStream_t s) {
+    if constexpr (TK == GW_BF16X2 || TK == GW_F16X2) {
+        if (a.pair_table && a.vis_kind == TK && !a.weight) {
+            launch_sp<NPOL, 0, TK, true>(a, num_sms, s);
+            return;
+        }
+    }
     switch (a.pad_stride) {
 #if GW_GRID_LANES_U == 16
-        case 32: launch_sp<NPOL, 32, TK>(a, num_sms, s); break;
-        case 48: launch_sp<NPOL, 48, TK>(a, num_sms, s); break;
-        case 64: launch_sp<NPOL, 64, TK>(a, num_sms, s); break;
-        case 96: launch_sp<NPOL, 96, TK>(a, num_sms, s); break;
-        case 160: launch_sp<NPOL, 160, TK>(a, num_sms, s); break;
-        default: launch_sp<NPOL, 288, TK>(a, num_sms, s); break;
+        case 32: launch_sp<NPOL, 32, TK, false>(a, num_sms, s); break;
+        case 48: launch_sp<NPOL, 48, TK, false>(a, num_sms, s); break;
+        case 64: launch_sp<NPOL, 64, TK, false>(a, num_sms, s); break;
+        case 96: launch_sp<NPOL, 96, TK, false>(a, num_sms, s); break;
+        case 160: launch_sp<NPOL, 160, TK, false>(a, num_sms, s); break;
+        default: launch_sp<NPOL, 288, TK, false>(a, num_sms, s); break;
 #else
-        case 24: launch_sp<NPOL, 24, TK>(a, num_sms, s); break;
-        case 32: launch_sp<NPOL, 32, TK>(a, num_sms, s); break;
-        case 48: launch_sp<NPOL, 48, TK>(a, num_sms, s); break;
-        case 80: launch_sp<NPOL, 80, TK>(a, num_sms, s); break;
-        case 144: launch_sp<NPOL, 144, TK>(a, num_sms, s); break;
-        default: launch_sp<NPOL, 272, TK>(a, num_sms, s); break;
+        case 24: launch_sp<NPOL, 24, TK, false>(a, num_sms, s); break;
+        case 32: launch_sp<NPOL, 32, TK, false>(a, num_sms, s); break;
+        case 48: launch_sp<NPOL, 48, TK, false>(a, num_sms, s); break;
+        case 80: launch_sp<NPOL, 80, TK, false>(a, num_sms, s); break;
+        case 144: launch_sp<NPOL, 144, TK, false>(a, num_sms, s); break;
+        default: launch_sp<NPOL, 272, TK, false>(a, num_sms, s); break;
 #endif
     }
 }

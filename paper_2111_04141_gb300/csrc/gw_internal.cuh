@@ -319,6 +319,10 @@ struct GridArgs {
     const gw_index_rec* rec;
     const void* ptable;          // zero-padded tables of kind table_kind (launch_pad_tables)
     const int64_t* pplane_off;   // device [P]: padded plane offsets
+    // pair tables (launch_pair_tables; null: none): gridding by 16-bit tensor cores
+    const void* pair_table = nullptr;
+    const int64_t* pair_off = nullptr;   // device [P]: plane offsets, in pairs
+    int64_t pair_count = 0;              // pairs of pair_table (debug bounds checks)
     const void* vis;           // [nvis][npol] of kind vis_kind
     const float* weight;       // [nvis][npol] or null
     const int64_t* plane_off;  // device [P]
@@ -391,6 +395,18 @@ int64_t padded_table_elems(int S, int beta, int SP);
 void launch_pad_tables(const void* tab, int kind, const int64_t* plane_off,
                        const int64_t* pplane_off, const int* support, int P, int beta, int SP,
                        void* ptab, cudaStream_t s);
+
+// Pair tables of the 16-bit gridder: every S x S slice twice, each row extended
+// to S + 1 entries by a zero, after the row in the first copy and before it
+// in the second.  Whatever the parity of a footprint's first column, one of
+// the copies puts the points (2 x, 2 x + 1) of the grid into one aligned
+// pair.  Pairs of a plane: beta^2 slices x 2 copies x S rows x (S + 1) / 2.
+// The planes follow a zero pair, which lanes outside a footprint read.
+inline int64_t pair_table_pairs(int S, int beta) {
+    return (int64_t)beta * beta * S * (S + 1);
+}
+void launch_pair_tables(const uint32_t* tab, const int64_t* plane_off, const int64_t* pair_off,
+                        const int* support, int P, int beta, uint32_t* pairs, cudaStream_t s);
 
 struct DegridArgs {
     const gw_index_rec* rec;
