@@ -9,8 +9,8 @@
 //                   degridder reads a record's whole footprint).
 // Steps: histogram (atomics; per-CTA shared histograms when the tile count
 // allows) -> exclusive scan -> scatter (atomic cursors),
-// then the footprint bins are cut into work items of at most item_max
-// entries.  Order within a bin is unspecified.
+// and the scan cuts the bins into work items of at most item_max entries.
+// Order within a bin is unspecified.
 #include "gw_internal.cuh"
 
 namespace gw {
@@ -70,61 +70,18 @@ __global__ void k_count(const gw_index_rec* __restrict__ rec, int64_t nvis, DevC
     }
 }
 
-// Exclusive scans of count[] -> offsets[], and of ceil(count / item_max) ->
-// item_off[], in one block.  n may exceed the block size; each thread scans
-// a contiguous run, then the run totals are scanned across the block.
-__global__ void k_scan(const uint32_t* __restrict__ count, int n, int item_max,
-                       uint32_t* __restrict__ offsets, uint32_t* __restrict__ item_off,
-                       uint32_t* __restrict__ cursor) {
-    __shared__ uint32_t s_a[1024];
-    __shared__ uint32_t s_b[1024];
-    const int tid = threadIdx.x;
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int lo = min(n, tid * per), hi = min(n, lo + per);
-    uint32_t sa = 0, sb = 0;
-    for (int i = lo; i < hi; ++i) {
-        const uint32_t c = count[i];
-        sa += c;
-        sb += (c + item_max - 1) / item_max;
-    }
-    s_a[tid] = sa;
-    s_b[tid] = sb;
-    __syncthreads();
-    // Hillis-Steele inclusive scan over the run totals
-    for (int d = 1; d < (int)blockDim.x; d <<= 1) {
-        uint32_t xa = 0, xb = 0;
-        if (tid >= d) {
-            xa = s_a[tid - d];
-            xb = s_b[tid - d];
-        }
-        __syncthreads();
-        s_a[tid] += xa;
-        s_b[tid] += xb;
-        __syncthreads();
-    }
-    uint32_t ra = s_a[tid] - sa, rb = s_b[tid] - sb;
-    for (int i = lo; i < hi; ++i) {
-        const uint32_t c = count[i];
-        offsets[i] = ra;
-        item_off[i] = rb;
-        cursor[i] = 0;
-        ra += c;
-        rb += (c + item_max - 1) / item_max;
-    }
-    if (tid == blockDim.x - 1) {
-        offsets[n] = s_a[tid];
-        item_off[n] = s_b[tid];
-    }
-}
-
-// Segmented scans for many bins: segments of kScanSeg bins, one CTA each.
-// Pass 0 writes each segment's totals (bins and work items); k_scan_top scans
-// the totals in one CTA; pass 1 writes offsets, item offsets and zeroed
-// cursors with the segment's base.
+// Exclusive scans of count[] -> offsets[] and of ceil(count / item_max) ->
+// item_off[], with zeroed cursors and the work items, in segments of kScanSeg
+// bins, one CTA each.
+// Up to kScanSingleMax bins one kernel does it: every CTA first sums the bins
+// before its segment (at most 1 MB of counts, read from L2 by 1,024 threads),
+// so no CTA waits for another (65,536 bins: bin stage 424 -> 242 us, the scan
+// having been one CTA with 64 bins a thread).  Beyond, pass 0 writes each
+// segment's totals, k_scan_top scans the totals in one CTA, and pass 1 finishes.
 constexpr int kScanThreads = 1024;
 constexpr int kScanPer = 8;
 constexpr int kScanSeg = kScanThreads * kScanPer;
-constexpr int kScanSingleMax = 65536;
+constexpr int kScanSingleMax = 262144;
 
 __device__ __forceinline__ void block_excl_scan2(uint32_t& a, uint32_t& b, uint32_t* sa,
                                                  uint32_t* sb) {
@@ -154,12 +111,28 @@ __device__ __forceinline__ void block_excl_scan2(uint32_t& a, uint32_t& b, uint3
     b = bb + ib - b;
 }
 
+// Work items of a bin: runs of at most item_max entries.
+__device__ __forceinline__ void write_items(Item* items, uint32_t o, int tile, uint32_t start,
+                                            uint32_t n, uint32_t item_max) {
+    for (uint32_t s = 0; s < n; s += item_max, ++o) {
+        Item it;
+        it.tile = tile;
+        it.start = (int32_t)(start + s);
+        it.len = (int32_t)min(item_max, n - s);
+        it.pad = 0;
+        items[o] = it;
+    }
+}
+
+// pass 0: segment totals; pass 1: the rest, from scanned totals; pass 2: all in
+// one kernel.
 __global__ void __launch_bounds__(kScanThreads) k_scan_seg(
     const uint32_t* __restrict__ count, int n, int item_max, int pass,
     uint32_t* __restrict__ seg_tot, uint32_t* __restrict__ offsets,
-    uint32_t* __restrict__ item_off, uint32_t* __restrict__ cursor) {
+    uint32_t* __restrict__ item_off, uint32_t* __restrict__ cursor, Item* __restrict__ items) {
     __shared__ uint32_t sa[32], sb[32];
-    const int64_t i0 = (int64_t)blockIdx.x * kScanSeg + (int64_t)threadIdx.x * kScanPer;
+    const int64_t s0 = (int64_t)blockIdx.x * kScanSeg;
+    const int64_t i0 = s0 + (int64_t)threadIdx.x * kScanPer;
     uint32_t c[kScanPer];
     uint32_t ta = 0, tb = 0;
 #pragma unroll
@@ -167,6 +140,26 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_seg(
         c[k] = i0 + k < n ? count[i0 + k] : 0u;
         ta += c[k];
         tb += (c[k] + item_max - 1) / item_max;
+    }
+    uint32_t ra = 0, rb = 0;
+    if (pass == 2 && s0 > 0) {
+        uint32_t pa = 0, pb = 0;                     // bins before this segment
+        for (int64_t i = threadIdx.x; i < s0 / 4; i += kScanThreads) {
+            const uint4 q = __ldg(reinterpret_cast<const uint4*>(count) + i);
+            pa += q.x + q.y + q.z + q.w;
+            pb += (q.x + item_max - 1) / item_max + (q.y + item_max - 1) / item_max +
+                  (q.z + item_max - 1) / item_max + (q.w + item_max - 1) / item_max;
+        }
+        pa = __reduce_add_sync(0xffffffffu, pa);
+        pb = __reduce_add_sync(0xffffffffu, pb);
+        if ((threadIdx.x & 31) == 0) {
+            sa[threadIdx.x >> 5] = pa;
+            sb[threadIdx.x >> 5] = pb;
+        }
+        __syncthreads();
+        ra = __reduce_add_sync(0xffffffffu, sa[threadIdx.x & 31]);
+        rb = __reduce_add_sync(0xffffffffu, sb[threadIdx.x & 31]);
+        __syncthreads();
     }
     uint32_t ea = ta, eb = tb;
     block_excl_scan2(ea, eb, sa, sb);
@@ -177,16 +170,27 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_seg(
         }
         return;
     }
-    uint32_t ra = seg_tot[2 * blockIdx.x] + ea, rb = seg_tot[2 * blockIdx.x + 1] + eb;
+    if (pass == 1) {
+        ra = seg_tot[2 * blockIdx.x];
+        rb = seg_tot[2 * blockIdx.x + 1];
+    }
+    ra += ea;
+    rb += eb;
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) {
         if (i0 + k < n) {
             offsets[i0 + k] = ra;
             item_off[i0 + k] = rb;
             cursor[i0 + k] = 0;
+            // (the allocation-free degrid path has no items)
+            if (items) write_items(items, rb, (int)(i0 + k), ra, c[k], (uint32_t)item_max);
         }
         ra += c[k];
         rb += (c[k] + item_max - 1) / item_max;
+    }
+    if (pass == 2 && blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1) {
+        offsets[n] = ra;
+        item_off[n] = rb;
     }
 }
 
@@ -246,6 +250,11 @@ __global__ void k_scatter(const gw_index_rec* __restrict__ rec, int64_t nvis, De
 // the entries with shared-memory cursors that start at the run bases.
 constexpr int kBinSmThreads = 512;
 constexpr int kBinSmTilesMax = 49152;     // 192 KB of u32 counters
+// Fewest CTAs worth it, at one CTA per ntiles records.  255 k records over
+// 16,384 tiles (15 CTAs) bin in 115 us with shared histograms and 55 us with
+// global atomics, 1.03 M over 32,768 (31 CTAs) in 290 and 120; 3.1 M over
+// 32,768 (95 CTAs) in 300 and 500, 30 k over 512 (59 CTAs) in 24 and 39.
+constexpr int kBinSmBlocksMin = 48;
 
 __global__ void __launch_bounds__(kBinSmThreads) k_count_sm(
     const gw_index_rec* __restrict__ rec, int64_t nvis, DevCount dc, BinGeom g, int P, int smin,
@@ -319,23 +328,6 @@ __global__ void __launch_bounds__(kBinSmThreads) k_scatter_sm(
     }
 }
 
-__global__ void k_items(const uint32_t* __restrict__ count, const uint32_t* __restrict__ offsets,
-                        const uint32_t* __restrict__ item_off, int ntiles, int item_max,
-                        Item* __restrict__ items) {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x) {
-        const uint32_t c = count[t];
-        uint32_t o = item_off[t];
-        for (uint32_t s = 0; s < c; s += (uint32_t)item_max, ++o) {
-            Item it;
-            it.tile = t;
-            it.start = (int32_t)(offsets[t] + s);
-            it.len = (int32_t)min((uint32_t)item_max, c - s);
-            it.pad = 0;
-            items[o] = it;
-        }
-    }
-}
-
 }  // namespace
 
 void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, int smin, int smax,
@@ -344,11 +336,11 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
     cudaMemsetAsync(sc.count, 0, sizeof(uint32_t) * ntiles, s);
     // per-CTA shared histograms when the bins fit and every CTA has at
     // least ntiles records (zeroing and flushing its histogram stays a small
-    // part of its work); small inputs keep the global-atomic kernels, which
-    // also leave the GPU to concurrent work on other streams
+    // part of its work) with enough of them for kBinSmBlocksMin CTAs; smaller
+    // inputs keep the global-atomic kernels, which spread over all SMs
     int sm_blocks = 0;
     const size_t hsm = sizeof(uint32_t) * (size_t)ntiles;
-    if (ntiles <= kBinSmTilesMax && nvis >= 2LL * ntiles) {
+    if (ntiles <= kBinSmTilesMax && nvis >= (int64_t)kBinSmBlocksMin * ntiles) {
         int dev = 0, nsm = 0, c_sm = 0, s_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -372,18 +364,17 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
                                                          sc.work);
         note_launch();
     }
-    // one CTA scans up to 64 bins per thread quickly; beyond that, segments
+    const int nseg = (ntiles + kScanSeg - 1) / kScanSeg;
     if (ntiles <= kScanSingleMax || !sc.scan_tmp || ntiles > sc.scan_tmp_bins) {
-        k_scan<<<1, 1024, 0, s>>>(sc.count, ntiles, g.item_max, sc.offsets, sc.item_off,
-                                  sc.cursor);
+        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, g.item_max, 2, nullptr, sc.offsets,
+                                                 sc.item_off, sc.cursor, sc.items);
         note_launch();
     } else {
-        const int nseg = (ntiles + kScanSeg - 1) / kScanSeg;
         k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, g.item_max, 0, sc.scan_tmp,
-                                                 sc.offsets, sc.item_off, sc.cursor);
+                                                 sc.offsets, sc.item_off, sc.cursor, sc.items);
         k_scan_top<<<1, kScanThreads, 0, s>>>(sc.scan_tmp, nseg, ntiles, sc.offsets, sc.item_off);
         k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, g.item_max, 1, sc.scan_tmp,
-                                                 sc.offsets, sc.item_off, sc.cursor);
+                                                 sc.offsets, sc.item_off, sc.cursor, sc.items);
         note_launch(3);
     }
     if (nvis > 0) {
@@ -396,21 +387,14 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
                                                            sc.offsets, sc.cursor, sc.entries);
         note_launch();
     }
-    if (sc.items) {   // work items (the allocation-free degrid path has none)
-        const int tb = (ntiles + 255) / 256;
-        k_items<<<tb, 256, 0, s>>>(sc.count, sc.offsets, sc.item_off, ntiles, g.item_max, sc.items);
-        note_launch();
-    }
 }
 
 cudaError_t preload_bin_kernels() {
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, k_count);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k_count_sm);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k_scan);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k_scatter);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k_scatter_sm);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k_items);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k_scan_seg);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, k_scan_top);
     return e;

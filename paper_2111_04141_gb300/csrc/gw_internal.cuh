@@ -43,8 +43,10 @@ constexpr double kQLimit = 1073741824.0;  // 2^30: |q| bound for a representable
 // evaluated exactly in integers.
 __host__ __device__ inline int plane_support(int p, int P, int smin, int smax) {
     if (P <= 1) return smin;
-    long long Y = (long long)smin * (P - 1) + (long long)(smax - smin) * p;
-    return (int)(2 * (Y / (2LL * (P - 1))) + 1);
+    // at most 255 x 4095 + 254 x 4095: 32 bits hold it (a 64-bit division costs
+    // about 100 instructions a record)
+    const unsigned Y = (unsigned)(smin * (P - 1) + (smax - smin) * p);
+    return (int)(2u * (Y / (2u * (unsigned)(P - 1))) + 1u);
 }
 
 __host__ __device__ inline long long floor_div(long long a, long long b) {
@@ -229,7 +231,7 @@ struct Scratch {
     unsigned long long* work = nullptr;     // [2]: valid visibilities, sum of S_p^2
     float2* wvis = nullptr;                 // [chunk * npol] weighted visibilities (lazy)
     uint32_t* scan_tmp = nullptr;           // [scan_tmp_words(scan_tmp_bins)] segment totals,
-                                            // or null (single-CTA scan)
+                                            // or null (one-kernel scan)
     int64_t scan_tmp_bins = 0;              // bins scan_tmp is sized for
     int64_t entries_cap = 0;
     int64_t items_cap = 0;
