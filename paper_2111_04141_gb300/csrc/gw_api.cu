@@ -538,6 +538,9 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     p->ip.wmax = desc->w_max_lambda;
     p->ip.N = N;
     p->ip.beta = beta;
+    p->ip.beta_shift = -1;
+    for (int b = 1; b <= 8; ++b)
+        if (beta == 1 << b) p->ip.beta_shift = b;
     p->ip.P = P;
     p->ip.smin = desc->support_min;
     p->ip.smax = desc->support_max;

@@ -36,7 +36,6 @@ constexpr int kGridPadR = kGridLanesV - 1;
 constexpr int kGridPadC = kGridLanesU - 1;
 constexpr int kItemMax = 1024;        // default max bin entries per work item
 constexpr int kItemMin = 64;          // smallest work-item size a plan may be tuned to
-constexpr double kQLimit = 1073741824.0;  // 2^30: |q| bound for a representable record
 
 // Support of plane p: the odd integer nearest
 // y = S_min + (S_max - S_min) p / (P - 1), ties upward: S = 2 floor(y/2) + 1,
@@ -127,6 +126,7 @@ struct IndexParams {
     double Pm1_d;    // P - 1 as double
     double wmax;     // w_max (wavelengths)
     int N, beta, P, smin, smax;
+    int beta_shift;  // log2(beta), or -1 if beta is no power of two
     // w-stacking (2-D plans only): layer = clamp(floor((w - wmin) / dw + 1/2), 0, nlayers - 1)
     // stored in the record's `plane` field; nlayers = 0: off
     int nlayers = 0;
@@ -141,20 +141,33 @@ struct IndexParams {
 // ((j + 1/2) / (P - 1))^2 w_max as int64 bit patterns (non-negative finite
 // doubles order like their bits).  Returns false (and an all-zero record)
 // for a dropped visibility.
+//
+// floor and the conversion to an integer are one FP64 addition rounded
+// towards minus infinity: y + 1.5 x 2^52 has a unit of 1 in the last place,
+// so its low word is floor(y) modulo 2^32.  The range test |y| < 2^30 (false
+// for infinities and NaN) compares the high word: it admits one value more
+// than |floor(y)| < 2^30, y in (-2^30, 1 - 2^30), whose pixel is off the grid.
 struct IndexAxis {
-    long long k, o;
+    int k, o;
     bool ok;
 };
 __device__ __forceinline__ IndexAxis index_axis(double coord_m, double f_c, const IndexParams& p) {
     // u_lambda = u * (f / c0) ; x = u_lambda * L + N/2 ; q = floor(beta * x + 0.5)
     const double lam = __dmul_rn(coord_m, f_c);
     const double x = __dadd_rn(__dmul_rn(lam, p.L), p.halfN);
-    const double q = floor(__dadd_rn(__dmul_rn(p.beta_d, x), 0.5));
+    const double y = __dadd_rn(__dmul_rn(p.beta_d, x), 0.5);
     IndexAxis r;
-    r.ok = isfinite(q) && fabs(q) < kQLimit;
-    const long long qi = r.ok ? (long long)q : 0LL;
-    r.k = floor_div(qi + p.beta / 2, p.beta);
-    r.o = qi - r.k * p.beta;
+    r.ok = (__double2hiint(y) & 0x7fffffff) < 0x41d00000;      // |y| < 2^30
+    const int q = r.ok ? __double2loint(__dadd_rd(y, 6755399441055744.0)) : 0;
+    // k = floor((q + beta / 2) / beta), o = q - k beta
+    const int m = q + p.beta / 2;
+    if (p.beta_shift >= 0) {
+        r.k = m >> p.beta_shift;
+    } else {
+        r.k = m / p.beta;
+        r.k -= m - r.k * p.beta < 0;
+    }
+    r.o = q - r.k * p.beta;
     return r;
 }
 __device__ __forceinline__ bool index_record(double u, double v, double w, double f_c,
@@ -190,8 +203,8 @@ __device__ __forceinline__ bool index_record(double u, double v, double w, doubl
                         (av.k - h >= 0) && (av.k + h <= p.N - 1);
     const bool valid = au.ok && av.ok && okw && inside;
     if (valid) {
-        r.ku = (int32_t)au.k;
-        r.kv = (int32_t)av.k;
+        r.ku = au.k;
+        r.kv = av.k;
         r.ou = (int16_t)au.o;
         r.ov = (int16_t)av.o;
         r.plane = (int16_t)plane;
