@@ -840,13 +840,16 @@ gw_status gw_plan_info_get(gw_plan p, gw_plan_info* out) {
     return GW_OK;
 }
 
-// Direct (unbinned) gridding of a chunk of nvis visibilities: forced by the
-// tuning, or automatic for inputs small enough that launches dominate.
-static bool use_direct(gw_plan p, int64_t nvis) {
-    if (p->tuning.grid_kernel == 1) return false;
-    if (p->tuning.grid_kernel == 2) return true;
+// Inputs small enough that launches dominate: gridded and degridded directly.
+static bool direct_size(gw_plan p, int64_t nvis) {
     const int64_t smax = p->support.empty() ? 1 : p->support.back();
     return nvis <= kDirectMaxVis && nvis * smax * smax * p->desc.npol <= kDirectMaxTaps;
+}
+// Direct (unbinned) gridding of a chunk of nvis visibilities: forced by the
+// tuning, or automatic for small inputs.
+static bool use_direct(gw_plan p, int64_t nvis) {
+    if (p->tuning.grid_kernel == 1) return false;
+    return p->tuning.grid_kernel == 2 || direct_size(p, nvis);
 }
 
 static void set_pairs(GridArgs& a, gw_plan p) {
@@ -1527,14 +1530,7 @@ gw_status gw_degrid_vis(gw_plan p, const double* uvw_m, const double* freq_hz, i
         const int64_t nr = std::min(rpc, nrow - r0);
         const int64_t v0 = r0 * nchan;
         void* out = static_cast<char*>(vis_out) + (size_t)v0 * npol * vb;
-        e = cudaMemsetAsync(out, 0, vb * nr * nchan * npol, s);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-        const bool staged = p->tuning.degrid_kernel != 2 && degrid_staged_fits(p->hmax, npol);
-        const BinGeom& geom = staged ? p->geom_staged : p->geom_degrid;
-        st = index_and_bin(p, uvw_m + 3 * r0, freq_hz, nr, nchan, geom, s);
-        if (st != GW_OK) return st;
         DegridArgs a;
-        a.rec = p->sc.rec;
         a.grid = reinterpret_cast<const float2*>(grid);
         a.table = p->table16 ? (const void*)p->table16 : (const void*)p->table;
         a.table_kind = p->desc.table_dtype;
@@ -1543,18 +1539,30 @@ gw_status gw_degrid_vis(gw_plan p, const double* uvw_m, const double* freq_hz, i
         a.table_elems = p->plane_off.back() + kTableSlack;
         a.plane_off = p->d_plane_off;
         a.support = p->d_support;
-        a.entries = p->sc.entries;
-        a.n_entries = p->sc.offsets + geom.ntu * geom.ntv;
         a.vis_out = out;
         a.vis_count = nr * (int64_t)nchan;
         a.N = p->desc.grid_n;
         a.npol = npol;
         a.beta = p->desc.oversample;
-        a.items = p->sc.items;
-        a.item_count = p->sc.item_off + geom.ntu * geom.ntv;
         a.queue = p->sc.counters;
-        a.ntiles_u = geom.ntu;
-        {
+        if (p->tuning.degrid_kernel == 0 && direct_size(p, nr * nchan)) {
+            // small input: one launch that indexes and degrids
+            StageTimer t(p, kStDegrid, s);
+            const DirectIndex di{uvw_m + 3 * r0, freq_hz, nr, nchan, p->ip, p->sc.dropped};
+            launch_degrid_direct(a, di, p->sc.work, s);
+        } else {
+            e = cudaMemsetAsync(out, 0, vb * nr * nchan * npol, s);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+            const bool staged = p->tuning.degrid_kernel != 2 && degrid_staged_fits(p->hmax, npol);
+            const BinGeom& geom = staged ? p->geom_staged : p->geom_degrid;
+            st = index_and_bin(p, uvw_m + 3 * r0, freq_hz, nr, nchan, geom, s);
+            if (st != GW_OK) return st;
+            a.rec = p->sc.rec;
+            a.entries = p->sc.entries;
+            a.n_entries = p->sc.offsets + geom.ntu * geom.ntv;
+            a.items = p->sc.items;
+            a.item_count = p->sc.item_off + geom.ntu * geom.ntv;
+            a.ntiles_u = geom.ntu;
             StageTimer t(p, kStDegrid, s);
             if (!(staged && launch_degrid_staged(a, p->hmax, p->num_sms, s)))
                 launch_degrid(a, nr * nchan, p->num_sms, s);

@@ -100,6 +100,138 @@ void launch_t(const DegridArgs& a, int64_t nvis, int num_sms, cudaStream_t s) {
     note_launch();
 }
 
+// Direct degridding for small inputs, the counterpart of the direct gridder:
+// one launch and no bins.  A warp per visibility, whose lane 0 computes the
+// index record (the same bit-exact FP64 sequence as the index stage) and
+// broadcasts it; lanes over the flattened S x S taps read the grid through
+// L1/L2.  Dropped visibilities are written as zeros, and the work counters
+// accumulate as the binner's would.
+constexpr int kDirectChanCache = 256;   // channel factors kept in shared memory
+
+template <int NPOL, int TK>
+__global__ void __launch_bounds__(kThreads) k_degrid_direct(DegridArgs a, DirectIndex di,
+                                                            unsigned long long* __restrict__ work) {
+    using TE = TabElem<TK>;
+    extern __shared__ long long sh_idx[];
+    __shared__ unsigned long long s_cnt[3];   // the block's valid, taps, dropped
+    const int nthr = di.p.P > 1 ? di.p.P - 1 : 0;
+    const int nc = min(di.nchan, kDirectChanCache);
+    long long* thr = sh_idx;
+    double* fc = reinterpret_cast<double*>(sh_idx + nthr);
+    for (int j = threadIdx.x; j < nthr; j += blockDim.x) thr[j] = wplane_threshold(j, di.p);
+    for (int c = threadIdx.x; c < nc; c += blockDim.x) fc[c] = __ddiv_rn(__ldg(di.freq + c), kC0);
+    if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int hb = a.beta / 2, N = a.N;
+    const int64_t nvis = di.nrow * (int64_t)di.nchan;
+    unsigned long long n_valid = 0, n_taps = 0, n_drop = 0;
+    for (int64_t i = warp0; i < nvis; i += nwarps) {
+        int4 rv = make_int4(0, 0, 0, 0);
+        if (lane == 0) {
+            const int64_t row = i / di.nchan;
+            const int chan = (int)(i - row * di.nchan);
+            const double f_c = chan < nc ? fc[chan] : __ddiv_rn(__ldg(di.freq + chan), kC0);
+            gw_index_rec r;
+            index_record(__ldg(di.uvw + 3 * row + 0), __ldg(di.uvw + 3 * row + 1),
+                         __ldg(di.uvw + 3 * row + 2), f_c, di.p, thr, r);
+            rv = *reinterpret_cast<const int4*>(&r);
+        }
+        rv.x = __shfl_sync(0xffffffffu, rv.x, 0);
+        rv.y = __shfl_sync(0xffffffffu, rv.y, 0);
+        rv.z = __shfl_sync(0xffffffffu, rv.z, 0);
+        rv.w = __shfl_sync(0xffffffffu, rv.w, 0);
+        const gw_index_rec rc = *reinterpret_cast<const gw_index_rec*>(&rv);
+        float acc[NPOL][2];
+#pragma unroll
+        for (int p = 0; p < NPOL; ++p) acc[p][0] = acc[p][1] = 0.f;
+        bool valid = (rc.flags & GW_FLAG_VALID) != 0;
+        const int S = valid ? __ldg(a.support + rc.plane) : 0, h = S >> 1;
+        const int64_t kofs = valid ? __ldg(a.plane_off + rc.plane) +
+                                         ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * S * S : 0;
+        if (lane == 0) {
+            n_valid += valid;
+            n_drop += !valid;
+            n_taps += (unsigned long long)(S * S);
+        }
+#ifdef GW_DEBUG_BOUNDS
+        // the slice, the footprint's pixels and the output row
+        if (valid && !gw_in_bounds((a.table_elems == 0 || (kofs >= 0 && kofs + (int64_t)S * S <= a.table_elems)) &&
+                                       rc.ku - h >= 0 && rc.ku + h < N && rc.kv - h >= 0 && rc.kv + h < N &&
+                                       (a.vis_count == 0 || i < a.vis_count),
+                                   a.queue ? a.queue + 1 : nullptr))
+            continue;
+#endif
+        const typename TE::T* K = reinterpret_cast<const typename TE::T*>(a.table) + kofs;
+        const float s = (rc.flags & GW_FLAG_CONJ) ? -1.f : 1.f;
+        for (int t = lane; t < S * S; t += 32) {
+            const int tv = t / S, tu = t - tv * S;
+            const float2 k = TE::load(K + t);
+            const float ki = s * k.y;
+            const int64_t pix = (int64_t)(rc.kv - h + tv) * N + (rc.ku - h + tu);
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) {
+                const float2 g = __ldg(a.grid + (int64_t)p * N * N + pix);
+                // (k.x - j ki) * (g.x + j g.y)
+                acc[p][0] = fmaf(k.x, g.x, acc[p][0]);
+                acc[p][0] = fmaf(ki, g.y, acc[p][0]);
+                acc[p][1] = fmaf(k.x, g.y, acc[p][1]);
+                acc[p][1] = fmaf(-ki, g.x, acc[p][1]);
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < NPOL; ++p)
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) {
+                acc[p][0] += __shfl_xor_sync(0xffffffffu, acc[p][0], d);
+                acc[p][1] += __shfl_xor_sync(0xffffffffu, acc[p][1], d);
+            }
+        if (lane < NPOL) {
+            float re = acc[0][0], im = acc[0][1];
+#pragma unroll
+            for (int p = 1; p < NPOL; ++p)
+                if (lane == p) { re = acc[p][0]; im = acc[p][1]; }
+            store_vis(a.vis_out, a.vis_kind, i * NPOL + lane, re * a.table_inv, im * a.table_inv);
+        }
+    }
+    // counts are held by lane 0 of each warp: one global atomic per block
+    if (lane == 0) {
+        if (n_valid) {
+            atomicAdd(&s_cnt[0], n_valid);
+            atomicAdd(&s_cnt[1], n_taps);
+        }
+        if (n_drop) atomicAdd(&s_cnt[2], n_drop);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s_cnt[0]) {
+            atomicAdd(work, s_cnt[0]);
+            atomicAdd(work + 1, s_cnt[1]);
+        }
+        if (s_cnt[2]) atomicAdd(di.dropped, s_cnt[2]);
+    }
+}
+
+template <int TK>
+void launch_direct_k(const DegridArgs& a, const DirectIndex& di, unsigned long long* work,
+                     cudaStream_t s) {
+    const int64_t nvis = di.nrow * (int64_t)di.nchan;
+    int64_t blocks = (nvis * 32 + kThreads - 1) / kThreads;
+    if (blocks > current_sm_count() * 8) blocks = current_sm_count() * 8;
+    const size_t smem = sizeof(long long) * (size_t)(di.p.P > 1 ? di.p.P - 1 : 0) +
+                        sizeof(double) * (size_t)std::min(di.nchan, kDirectChanCache);
+    const unsigned b = (unsigned)blocks;
+    switch (a.npol) {
+        case 1: k_degrid_direct<1, TK><<<b, kThreads, smem, s>>>(a, di, work); break;
+        case 2: k_degrid_direct<2, TK><<<b, kThreads, smem, s>>>(a, di, work); break;
+        case 3: k_degrid_direct<3, TK><<<b, kThreads, smem, s>>>(a, di, work); break;
+        default: k_degrid_direct<4, TK><<<b, kThreads, smem, s>>>(a, di, work); break;
+    }
+    note_launch();
+}
+
 #ifndef GW_DEGRID_THREADS
 #define GW_DEGRID_THREADS 768
 #endif
@@ -525,6 +657,16 @@ bool launch_degrid_staged(const DegridArgs& a, int hmax, int num_sms, cudaStream
         case GW_BF16X2: return launch_staged_k<GW_BF16X2>(a, hmax, num_sms, s);
         case GW_F16X2: return launch_staged_k<GW_F16X2>(a, hmax, num_sms, s);
         default: return launch_staged_k<GW_C64>(a, hmax, num_sms, s);
+    }
+}
+
+void launch_degrid_direct(const DegridArgs& a, const DirectIndex& di, unsigned long long* work,
+                          cudaStream_t s) {
+    if (di.nrow <= 0 || di.nchan <= 0) return;
+    switch (a.table_kind) {
+        case GW_BF16X2: launch_direct_k<GW_BF16X2>(a, di, work, s); break;
+        case GW_F16X2: launch_direct_k<GW_F16X2>(a, di, work, s); break;
+        default: launch_direct_k<GW_C64>(a, di, work, s); break;
     }
 }
 

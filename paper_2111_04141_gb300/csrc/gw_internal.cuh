@@ -445,6 +445,12 @@ struct DegridArgs {
     int64_t vis_count = 0;      // visibilities of vis_out
 };
 void launch_degrid(const DegridArgs& a, int64_t nvis_upper, int num_sms, cudaStream_t s);
+// Direct degridding (no bins) of nrow x nchan visibilities, each warp
+// computing its visibility's index record: dropped visibilities are written
+// as zeros and counted in di.dropped, and work[0], work[1] accumulate as in
+// launch_grid_direct.
+void launch_degrid_direct(const DegridArgs& a, const DirectIndex& di, unsigned long long* work,
+                          cudaStream_t s);
 // Staged-degrid region budget (bytes): the 227 KB a CTA may hold, less two
 // buffers of 1,024 records' metadata and the static shared memory.
 constexpr size_t kStagedSmemMax = 232448 - 2 * 1024 * 16 - 512;
