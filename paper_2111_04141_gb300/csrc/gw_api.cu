@@ -128,7 +128,7 @@ struct gw_plan_s {
     gw_plan_desc desc{};
     int device = -1;
     int num_sms = 0;
-    BinGeom geom_grid{}, geom_degrid{}, geom_staged{};
+    BinGeom geom_grid{}, geom_degrid{}, geom_staged{}, geom_staged64{};
     int hmax = 0;        // largest half-support over the planes
     int ntiles = 0;      // bins allocated (max over the geometries and plane groups)
     int max_groups = 1;  // plane groups the bins are allocated for (gw_tuning.plane_groups)
@@ -347,6 +347,7 @@ void apply_tuning(gw_plan p) {
     p->geom_grid.item_max = im;
     p->geom_degrid.item_max = im;
     p->geom_staged.item_max = im;
+    p->geom_staged64.item_max = im;
 }
 
 enum Stage { kStIndex = 0, kStBin = 1, kStGrid = 2, kStDegrid = 3 };
@@ -482,10 +483,8 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     p->geom_grid = BinGeom{0, kGridTileShiftU, 5, (N + kGridTileU - 1) / kGridTileU,
                            (N + kGridTileV - 1) / kGridTileV};
     p->geom_degrid = BinGeom{1, 5, 5, (N + kTile - 1) / kTile, (N + kTile - 1) / kTile};
-    {
-        const int st = degrid_staged_tile();
-        p->geom_staged = BinGeom{1, 4, 4, (N + st - 1) / st, (N + st - 1) / st};
-    }
+    p->geom_staged = BinGeom{1, 4, 4, (N + 15) / 16, (N + 15) / 16};
+    p->geom_staged64 = BinGeom{1, 6, 6, (N + 63) / 64, (N + 63) / 64};
     p->ntiles = std::max({p->geom_grid.ntu * p->geom_grid.ntv,
                           p->geom_degrid.ntu * p->geom_degrid.ntv,
                           p->geom_staged.ntu * p->geom_staged.ntv});
@@ -694,6 +693,7 @@ gw_status gw_plan_clone(gw_plan src, int64_t max_vis_per_call, void* cuda_stream
     p->geom_grid = src->geom_grid;
     p->geom_degrid = src->geom_degrid;
     p->geom_staged = src->geom_staged;
+    p->geom_staged64 = src->geom_staged64;
     p->hmax = src->hmax;
     p->ntiles = src->ntiles;
     p->max_groups = src->max_groups;
@@ -838,6 +838,22 @@ gw_status gw_plan_info_get(gw_plan p, gw_plan_info* out) {
     out->table_bytes = p->tabs ? p->tabs->bytes : 0;
     out->scratch_bytes = p->scratch_bytes;
     return GW_OK;
+}
+
+// Bins of the staged degridder for nvis visibilities.  A tile's grid region is
+// staged once for the records centred in it, so sparse inputs take larger
+// tiles.  By visibilities per 16 x 16 points (kernel times):
+//   16 (255 k x 4, 2048^2, support 7-41): 16 / 32 / 64-point tiles 380 / 260 / 331 us
+//   4  (1.04 M x 4, 8192^2, support 7-127): 32 / 64 / 128 4.88 / 3.63 / 3.52 ms
+//   63 (1.04 M x 4, 2048^2, support 7-127): 16 / 64 4.53 / 4.03 ms
+//   126 (8.3 M x 4, 4096^2, support 7-63): 16 / 32 / 64 9.52 / 9.89 / 10.7 ms
+// Where the region of 16-point tiles does not fit and is served in bands, 32
+// points are taken at any density.
+static const BinGeom& staged_geom(gw_plan p, int64_t nvis) {
+    const double n = (double)p->desc.grid_n, per = (double)nvis * 256.0;
+    if (per < kStagedSparse64 * n * n) return p->geom_staged64;
+    return per < kStagedSparse32 * n * n || staged_banded(p->hmax, p->desc.npol) ? p->geom_degrid
+                                                                               : p->geom_staged;
 }
 
 // Inputs small enough that launches dominate: gridded and degridded directly.
@@ -1553,8 +1569,8 @@ gw_status gw_degrid_vis(gw_plan p, const double* uvw_m, const double* freq_hz, i
         } else {
             e = cudaMemsetAsync(out, 0, vb * nr * nchan * npol, s);
             if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-            const bool staged = p->tuning.degrid_kernel != 2 && degrid_staged_fits(p->hmax, npol);
-            const BinGeom& geom = staged ? p->geom_staged : p->geom_degrid;
+            const bool staged = p->tuning.degrid_kernel != 2;
+            const BinGeom& geom = staged ? staged_geom(p, nr * nchan) : p->geom_degrid;
             st = index_and_bin(p, uvw_m + 3 * r0, freq_hz, nr, nchan, geom, s);
             if (st != GW_OK) return st;
             a.rec = p->sc.rec;
@@ -1563,8 +1579,11 @@ gw_status gw_degrid_vis(gw_plan p, const double* uvw_m, const double* freq_hz, i
             a.items = p->sc.items;
             a.item_count = p->sc.item_off + geom.ntu * geom.ntv;
             a.ntiles_u = geom.ntu;
+            a.tile_shift = geom.su;
             StageTimer t(p, kStDegrid, s);
-            if (!(staged && launch_degrid_staged(a, p->hmax, p->num_sms, s)))
+            if (staged)
+                launch_degrid_staged(a, p->hmax, p->num_sms, s);
+            else
                 launch_degrid(a, nr * nchan, p->num_sms, s);
         }
         e = cudaGetLastError();
@@ -1747,7 +1766,7 @@ gw_status gw_degrid_vis_devcount(gw_plan p, const double* uvw_m, const double* f
     const DevCount dc{d_nrow, nchan};
     const int64_t nmax = max_nrow * (int64_t)nchan;
     launch_zero_vis(vis_out, vk, nmax, npol, dc, s);
-    const bool staged = p->tuning.degrid_kernel != 2 && degrid_staged_fits(p->hmax, npol);
+    const bool staged = p->tuning.degrid_kernel != 2;
     const BinGeom& geom = staged ? p->geom_staged : p->geom_degrid;
     launch_index(uvw_m, freq_hz, max_nrow, nchan, p->ip, p->sc.rec, p->sc.dropped, s, d_nrow);
     launch_bin(p->sc.rec, nmax, geom, p->desc.n_wplanes, p->desc.support_min,
@@ -1773,7 +1792,10 @@ gw_status gw_degrid_vis_devcount(gw_plan p, const double* uvw_m, const double* f
     a.item_count = p->sc.item_off + geom.ntu * geom.ntv;
     a.queue = p->sc.counters;
     a.ntiles_u = geom.ntu;
-    if (!(staged && launch_degrid_staged(a, p->hmax, p->num_sms, s)))
+    a.tile_shift = geom.su;
+    if (staged)
+        launch_degrid_staged(a, p->hmax, p->num_sms, s);
+    else
         launch_degrid(a, nmax, p->num_sms, s);
     e = cudaGetLastError();
     return e == cudaSuccess ? GW_OK : cuda_fail(e, "degrid launch");

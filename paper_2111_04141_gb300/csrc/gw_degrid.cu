@@ -5,10 +5,10 @@
 // Tables of any storage kind are widened to FP32 on load, the sum is FP32,
 // and the result is written in the plan's visibility kind.
 //
-// Two kernels:
-// * k_degrid_staged (used by gw_degrid_vis): one CTA of 24 warps per SM
-//   serves chunks of work items (at most 1,024 records centred in one 16 x 16
-//   tile).  Warps 0-3 load the records' metadata (id, kernel slice, centre,
+// Three kernels:
+// * k_degrid_staged (used by gw_degrid_vis): one CTA of 32 warps per SM
+//   serves chunks of work items (at most 1,024 records centred in one tile of
+//   16 x 16 points, or 32 x 32 or 64 x 64 for sparse inputs).  Warps 0-3 load the records' metadata (id, kernel slice, centre,
 //   support) into one of two shared buffers, the next chunk's while all
 //   warps compute the current one.  The CTA stages the tile's grid region
 //   (the tile plus the chunk's largest half-support on every side) in
@@ -20,9 +20,19 @@
 //   consecutive taps of the S x S footprint (flattened, so every lane is
 //   busy), with kernel values loaded four steps ahead, packed FP32x2 FMAs
 //   into K.re G and K.im G sums, and a reduce-scatter over the lanes.
-// * k_degrid (the fallback when the region does not fit in shared memory,
-//   and the allocation-free entry point): the same per-record warp, reading
-//   the grid through L1/L2, records visited in 32 x 32 centre-tile order.
+//   A region larger than the shared memory is served in bands of rows: every
+//   record sums the tap rows in the band, and its sums wait in shared memory
+//   for the next one.  (Read through L1/L2 instead, 32 B a tap, 1.04 M
+//   visibilities x 4 polarisations with supports to 127 on an 8192^2 grid took
+//   13.2 ms; in bands they take 3.3, the same items read in place where few
+//   taps share a region 5.2.)  The L1 data pipe bounds it (87 % on the 4-pol
+//   w-projection batch: 16-byte loads of staged points); 32 warps of 64
+//   registers beat 24 of 80 there, 9.34 against 9.52 ms, and 3.28 against 3.63
+//   in bands.
+// * k_degrid_direct (small calls): one launch, index records included.
+// * k_degrid (the allocation-free entry point): the same per-record warp,
+//   reading the grid through L1/L2, records visited in 32 x 32 centre-tile
+//   order.
 #include "gw_internal.cuh"
 
 namespace gw {
@@ -233,10 +243,9 @@ void launch_direct_k(const DegridArgs& a, const DirectIndex& di, unsigned long l
 }
 
 #ifndef GW_DEGRID_THREADS
-#define GW_DEGRID_THREADS 768
+#define GW_DEGRID_THREADS 1024
 #endif
 constexpr int kStagedThreads = GW_DEGRID_THREADS;
-constexpr int kStagedTile = 16;
 constexpr int kStagedMeta = 1024;   // records whose metadata a CTA stages at once
 constexpr int kStagedPad = 4;       // zero elements after each staged plane
 #ifndef GW_DEGRID_DEPTH
@@ -264,27 +273,33 @@ __device__ __forceinline__ void loader_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(kLoaderThreads) : "memory");
 }
 
-template <int NPOL, int TK>
-__global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, int hmax) {
+// GEN: any tile size, regions in bands; otherwise 16 x 16 tiles whose largest
+// region fits (a tap loop without the band's bounds: 3.11 against 3.31 ms on
+// 4.2 M visibilities of one polarisation, support 31).
+template <int NPOL, int TK, bool GEN>
+__global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, int hmax, int cap) {
     using TE = TabElem<TK>;
-    using T = typename TE::T;
+    using TT = typename TE::T;
     constexpr int D = kStagedDepth;
     // grid region as polarisation pairs [NPOL / 2][RS][RS] of (G_p, G_p+1),
-    // then [RS][RS] of the last polarisation if NPOL is odd; two chunks'
-    // record metadata after the largest region (RS = 16 + 2 h_max)
+    // then [RS][RS] of the last polarisation if NPOL is odd (`cap` grid points
+    // at most: larger regions are served in bands of rows); then two chunks'
+    // record metadata, and the partial sums of records that span bands
     constexpr int NPR = NPOL / 2;
     extern __shared__ __align__(16) float4 reg[];
     __shared__ StagedChunk s_ch[2];
     uint4* meta0;
     {
-        const int RSM = kStagedTile + 2 * hmax, pm = RSM * RSM + kStagedPad;
+        const int pm = cap + kStagedPad;
         meta0 = reinterpret_cast<uint4*>(reinterpret_cast<float2*>(reg + (size_t)NPR * pm) +
                                          (NPOL % 2 ? pm : 0));
     }
+    float2* part = reinterpret_cast<float2*>(meta0 + 2 * kStagedMeta);   // [kStagedMeta][NPOL]
+    const int T = GEN ? 1 << a.tile_shift : 16;
     const int lane = threadIdx.x & 31;
     const int N = a.N, hb = a.beta / 2;
     const uint32_t nitems = *a.item_count;
-    const T* __restrict__ tab = reinterpret_cast<const T*>(a.table);
+    const TT* __restrict__ tab = reinterpret_cast<const TT*>(a.table);
     // thread 0: the item being served and the next chunk's first record
     Item cur{};
     int next_c0 = 0;
@@ -322,8 +337,8 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
         if (c.done) return;
         const Item item = c.item;
         const int c0 = c.c0, nc = c.nc;
-        const int tx0 = (item.tile % a.ntiles_u) * kStagedTile;
-        const int ty0 = (item.tile / a.ntiles_u) * kStagedTile;
+        const int tx0 = (item.tile % a.ntiles_u) * T;
+        const int ty0 = (item.tile / a.ntiles_u) * T;
         uint4* meta = meta0 + buf * kStagedMeta;
         int hw = 0;
         for (int k0 = 0; k0 < kMetaPerLoader; k0 += kLoaderBatch) {
@@ -358,8 +373,8 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                     // table's start, centred in the tile
                     const bool ok =
                         (a.table_elems == 0 || (kofs >= 0 && kofs + (int64_t)S * S <= a.table_elems)) &&
-                        rc.ku - tx0 >= 0 && rc.ku - tx0 < kStagedTile && rc.kv - ty0 >= 0 &&
-                        rc.kv - ty0 < kStagedTile && h <= hmax &&
+                        rc.ku - tx0 >= 0 && rc.ku - tx0 < T && rc.kv - ty0 >= 0 &&
+                        rc.kv - ty0 < T && h <= hmax &&
                         (a.vis_count == 0 || ids[k] < (uint64_t)a.vis_count);
                     if (!gw_in_bounds(ok, a.queue + 1)) {
                         rel = 8u | 8u << 8;
@@ -386,6 +401,24 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
         if (lane == 0 && hw > 0) atomicMax(&c.h, hw);
     };
 
+    // sum of a record's polarisation over one band: stored, or added to the
+    // bands before and kept for the bands after
+    auto finish = [&](int r, int p, uint32_t id, int before, bool more, float re, float im) {
+        if constexpr (GEN) {
+            float2* w = part + r * NPOL + p;
+            if (before > 0) {
+                re += w->x;
+                im += w->y;
+            }
+            if (more) {
+                *w = make_float2(re, im);
+                return;
+            }
+        }
+        store_vis(a.vis_out, a.vis_kind, (int64_t)id * NPOL + p, re * a.table_inv,
+                  im * a.table_inv);
+    };
+
     if (threadIdx.x < kLoaderThreads) load_chunk(0);
     __syncthreads();
     for (int kc = 0;; ++kc) {
@@ -394,10 +427,10 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
         if (c.done) break;
         const Item item = c.item;
         const int c0 = c.c0, nc = c.nc;
-        const int tx0 = (item.tile % a.ntiles_u) * kStagedTile;
-        const int ty0 = (item.tile / a.ntiles_u) * kStagedTile;
+        const int tx0 = (item.tile % a.ntiles_u) * T;
+        const int ty0 = (item.tile / a.ntiles_u) * T;
         const uint4* meta = meta0 + buf * kStagedMeta;
-        // the region: rows and columns [t0 - hi, t0 + 16 + hi) of the tile,
+        // the region: rows and columns [t0 - hi, t0 + T + hi) of the tile,
         // RS x RS values at row pitch RSP; each plane holds RS x RSP elements
         // and kStagedPad zeros (element RS * RSP is read by lanes without a
         // tap in a record's last step).  A quarter-warp's 8 flattened taps
@@ -408,7 +441,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
         // several chunks keep RSP = RS).  RS is even, so every part stays
         // 16-byte aligned.
         const int hi = c.h;
-        const int RS = kStagedTile + 2 * hi;
+        const int RS = T + 2 * hi;
         int RSP = RS;
         if (item.len <= kStagedMeta) {
             int best = 0, bt = -1;
@@ -419,196 +452,216 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                     best = k;
                 }
             const int rsp = RS + ((best - RS) & 7);
-            const int RSM = kStagedTile + 2 * hmax;
-            if (RS * rsp <= RSM * RSM) RSP = rsp;
+            if (RS * rsp <= cap || (GEN && RS * RS > cap)) RSP = rsp;
         }
-        const int plane = RS * RSP + kStagedPad;
-        const int zoff = RS * RSP;
+        // bands of BR region rows, of equal height
+        const int nb = !GEN || RS * RSP <= cap ? 1 : (RS + cap / RSP - 1) / (cap / RSP);
+        const int BR = (RS + nb - 1) / nb;
+        const int plane = BR * RSP + kStagedPad;
+        const int zoff = BR * RSP;
         float2* single = reinterpret_cast<float2*>(reg + (size_t)NPR * plane);
-        if (c0 == 0) {
-            const int rx0 = tx0 - hi, ry0 = ty0 - hi;
-            if (threadIdx.x < kStagedPad) {
+        for (int band = 0; band < nb; ++band) {
+            const int yb = GEN ? band * BR : 0, nrows = GEN ? min(BR, RS - yb) : RS;
+            if (c0 == 0 || nb > 1) {
+                const int rx0 = tx0 - hi, ry0 = ty0 - hi + yb;
+                if (band > 0 && threadIdx.x == 0) s_ch[buf].next = 0;
+                if (threadIdx.x < kStagedPad) {
 #pragma unroll
-                for (int q = 0; q < NPR; ++q)
-                    reg[(size_t)q * plane + zoff + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (NPOL % 2) single[zoff + threadIdx.x] = make_float2(0.f, 0.f);
+                    for (int q = 0; q < NPR; ++q)
+                        reg[(size_t)q * plane + zoff + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (NPOL % 2) single[zoff + threadIdx.x] = make_float2(0.f, 0.f);
+                }
+                for (int e0 = threadIdx.x; e0 < nrows * RS; e0 += kStagedThreads) {
+                    const int y = e0 / RS, x = e0 - y * RS;
+                    const int e = y * RSP + x;
+                    const int gy = ry0 + y, gx = rx0 + x;
+                    const bool in = gx >= 0 && gx < N && gy >= 0 && gy < N;
+                    float2 g[NPOL];
+#pragma unroll
+                    for (int p = 0; p < NPOL; ++p)
+                        g[p] = in ? __ldg(a.grid + ((int64_t)p * N + gy) * N + gx) : make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int q = 0; q < NPR; ++q)
+                        reg[(size_t)q * plane + e] = make_float4(g[2 * q].x, g[2 * q].y, g[2 * q + 1].x,
+                                                                 g[2 * q + 1].y);
+                    if (NPOL % 2) single[e] = g[NPOL - 1];
+                }
+                __syncthreads();
             }
-            for (int e0 = threadIdx.x; e0 < RS * RS; e0 += kStagedThreads) {
-                const int y = e0 / RS, x = e0 - y * RS;
-                const int e = y * RSP + x;
-                const int gy = ry0 + y, gx = rx0 + x;
-                const bool in = gx >= 0 && gx < N && gy >= 0 && gy < N;
-                float2 g[NPOL];
+            // the loaders prepare the next chunk, then join the record claims
+            if (band == nb - 1 && threadIdx.x < kLoaderThreads) load_chunk(buf ^ 1);
+            for (;;) {
+                int r = 0;
+                if (lane == 0) r = atomicAdd(&s_ch[buf].next, 1);
+                r = __shfl_sync(0xffffffffu, r, 0);
+                if (r >= nc) break;
+                const uint4 m = meta[r];
+                const uint32_t id = m.x;
+                const int S = (int)(m.w & 0xffffu);
+                const float sg = (m.w >> 16) ? -1.f : 1.f;
+                // region row and column of tap (0, 0): centre - h + hi; the tap rows
+                // [tv0, tv1) lie in this band
+                const int ry = (int)(m.z >> 8) - (S >> 1) + hi, rx = (int)(m.z & 0xffu) - (S >> 1) + hi;
+                const int tv0 = GEN ? max(0, yb - ry) : 0;
+                const int tv1 = GEN ? min(S, yb + nrows - ry) : S;
+                if (GEN && tv1 <= tv0) continue;
+                const TT* K = tab + m.y + tv0 * S;
+                const int n = (tv1 - tv0) * S;
+                // flattened taps t = lane + 32 i; the region index advances by
+                // `step` per 32 taps, plus `wrap` when the tap column wraps
+                const int dq = 32 / S, dr = 32 - dq * S;
+                const int step = dq * RSP + dr, wrap = RSP - S;
+                int tu = lane % S;
+                const int base = (ry + tv0 - yb) * RSP + rx;
+                int off = base + (lane / S) * RSP + tu;
+                // a1 = sum K.re G, a2 = sum K.im G (packed FP32x2 FMAs); the
+                // conjugation sign is applied once at the end
+                float2 a1[NPOL], a2[NPOL];
 #pragma unroll
-                for (int p = 0; p < NPOL; ++p)
-                    g[p] = in ? __ldg(a.grid + ((int64_t)p * N + gy) * N + gx) : make_float2(0.f, 0.f);
+                for (int p = 0; p < NPOL; ++p) a1[p] = a2[p] = make_float2(0.f, 0.f);
+                auto tap = [&](const float2 k, const int o) {
+                    const float2 kxx = make_float2(k.x, k.x), kyy = make_float2(k.y, k.y);
 #pragma unroll
-                for (int q = 0; q < NPR; ++q)
-                    reg[(size_t)q * plane + e] = make_float4(g[2 * q].x, g[2 * q].y, g[2 * q + 1].x,
-                                                             g[2 * q + 1].y);
-                if (NPOL % 2) single[e] = g[NPOL - 1];
-            }
-            __syncthreads();
-        }
-        // the loaders prepare the next chunk, then join the record claims
-        if (threadIdx.x < kLoaderThreads) load_chunk(buf ^ 1);
-        for (;;) {
-            int r = 0;
-            if (lane == 0) r = atomicAdd(&s_ch[buf].next, 1);
-            r = __shfl_sync(0xffffffffu, r, 0);
-            if (r >= nc) break;
-            const uint4 m = meta[r];
-            const uint32_t id = m.x;
-            const T* K = tab + m.y;
-            const int S = (int)(m.w & 0xffffu);
-            const float sg = (m.w >> 16) ? -1.f : 1.f;
-            const int n = S * S;
-            // flattened taps t = lane + 32 i; the region index advances by
-            // `step` per 32 taps, plus `wrap` when the tap column wraps
-            const int dq = 32 / S, dr = 32 - dq * S;
-            const int step = dq * RSP + dr, wrap = RSP - S;
-            int tu = lane % S;
-            // region index of tap (0, 0): centre - h + hi on both axes
-            const int base = ((int)(m.z >> 8) - (S >> 1) + hi) * RSP + ((int)(m.z & 0xffu) - (S >> 1) + hi);
-            int off = base + (lane / S) * RSP + tu;
-            // a1 = sum K.re G, a2 = sum K.im G (packed FP32x2 FMAs); the
-            // conjugation sign is applied once at the end
-            float2 a1[NPOL], a2[NPOL];
-#pragma unroll
-            for (int p = 0; p < NPOL; ++p) a1[p] = a2[p] = make_float2(0.f, 0.f);
-            auto tap = [&](const float2 k, const int o) {
-                const float2 kxx = make_float2(k.x, k.x), kyy = make_float2(k.y, k.y);
-#pragma unroll
-                for (int q = 0; q < NPR; ++q) {
-                    const float4 g = reg[(size_t)q * plane + o];
-                    const float2 g0 = make_float2(g.x, g.y), g1 = make_float2(g.z, g.w);
-                    a1[2 * q] = __ffma2_rn(kxx, g0, a1[2 * q]);
-                    a2[2 * q] = __ffma2_rn(kyy, g0, a2[2 * q]);
-                    a1[2 * q + 1] = __ffma2_rn(kxx, g1, a1[2 * q + 1]);
-                    a2[2 * q + 1] = __ffma2_rn(kyy, g1, a2[2 * q + 1]);
-                }
-                if (NPOL % 2) {
-                    const float2 g = single[o];
-                    a1[NPOL - 1] = __ffma2_rn(kxx, g, a1[NPOL - 1]);
-                    a2[NPOL - 1] = __ffma2_rn(kyy, g, a2[NPOL - 1]);
-                }
-            };
-            auto advance = [&]() {
-                off += step;
-                tu += dr;
-                if (tu >= S) {
-                    tu -= S;
-                    off += wrap;
-                }
-            };
-            // steps 0 .. nfull - 1 have a tap on every lane, step nfull on
-            // the lanes below n - 32 nfull.  Kernel values are loaded D steps
-            // ahead, unconditionally: past the slice they read the next
-            // slice or the table's zero slack, never used.
-            const int nfull = (n - 1) >> 5;
-            const T* kp = K + lane;
-            T kq[D];
-#pragma unroll
-            for (int d = 0; d < D; ++d) kq[d] = __ldg(kp + 32 * d);
-            kp += 32 * D;
-            int i = 0;
-            for (; i + D <= nfull; i += D) {
-#pragma unroll
-                for (int d = 0; d < D; ++d) {
-                    const float2 k = TE::cvt(kq[d]);
-                    kq[d] = __ldg(kp + 32 * d);
-                    tap(k, off);
-                    advance();
-                }
-                kp += 32 * D;
-            }
-            // the last (< D) full steps and the partial one, from the front
-            // of the ring
-            for (; i <= nfull; ++i) {
-                const bool live = i < nfull || lane + 32 * nfull < n;
-                tap(live ? TE::cvt(kq[0]) : make_float2(0.f, 0.f), live ? off : zoff);
-                advance();
-#pragma unroll
-                for (int d = 0; d + 1 < D; ++d) kq[d] = kq[d + 1];
-            }
-            // conj(K_i) G with K_i = K (w >= 0) or conj K (w < 0):
-            // re = sum K.re G.re + s K.im G.im, im = sum K.re G.im - s K.im G.re
-            float acc[NPOL][2];
-#pragma unroll
-            for (int p = 0; p < NPOL; ++p) {
-                acc[p][0] = fmaf(sg, a2[p].y, a1[p].x);
-                acc[p][1] = fmaf(-sg, a2[p].x, a1[p].y);
-            }
-            if constexpr (NPOL == 4) {
-                // reduce-scatter butterfly: lanes with bit 4 set keep pols 2, 3,
-                // then bit 3 picks one of the two; 12 shuffles instead of 40
-                const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0;
-                const float k0r = (b4 ? acc[2][0] : acc[0][0]) +
-                                  __shfl_xor_sync(0xffffffffu, b4 ? acc[0][0] : acc[2][0], 16);
-                const float k0i = (b4 ? acc[2][1] : acc[0][1]) +
-                                  __shfl_xor_sync(0xffffffffu, b4 ? acc[0][1] : acc[2][1], 16);
-                const float k1r = (b4 ? acc[3][0] : acc[1][0]) +
-                                  __shfl_xor_sync(0xffffffffu, b4 ? acc[1][0] : acc[3][0], 16);
-                const float k1i = (b4 ? acc[3][1] : acc[1][1]) +
-                                  __shfl_xor_sync(0xffffffffu, b4 ? acc[1][1] : acc[3][1], 16);
-                float re = (b3 ? k1r : k0r) + __shfl_xor_sync(0xffffffffu, b3 ? k0r : k1r, 8);
-                float im = (b3 ? k1i : k0i) + __shfl_xor_sync(0xffffffffu, b3 ? k0i : k1i, 8);
-#pragma unroll
-                for (int d = 4; d > 0; d >>= 1) {
-                    re += __shfl_xor_sync(0xffffffffu, re, d);
-                    im += __shfl_xor_sync(0xffffffffu, im, d);
-                }
-                if ((lane & 7) == 0) {
-                    const int p = (b4 ? 2 : 0) + (b3 ? 1 : 0);
-                    store_vis(a.vis_out, a.vis_kind, (int64_t)id * NPOL + p, re * a.table_inv,
-                              im * a.table_inv);
-                }
-            } else {
-#pragma unroll
-                for (int p = 0; p < NPOL; ++p)
-#pragma unroll
-                    for (int d = 16; d > 0; d >>= 1) {
-                        acc[p][0] += __shfl_xor_sync(0xffffffffu, acc[p][0], d);
-                        acc[p][1] += __shfl_xor_sync(0xffffffffu, acc[p][1], d);
+                    for (int q = 0; q < NPR; ++q) {
+                        const float4 g = reg[(size_t)q * plane + o];
+                        const float2 g0 = make_float2(g.x, g.y), g1 = make_float2(g.z, g.w);
+                        a1[2 * q] = __ffma2_rn(kxx, g0, a1[2 * q]);
+                        a2[2 * q] = __ffma2_rn(kyy, g0, a2[2 * q]);
+                        a1[2 * q + 1] = __ffma2_rn(kxx, g1, a1[2 * q + 1]);
+                        a2[2 * q + 1] = __ffma2_rn(kyy, g1, a2[2 * q + 1]);
                     }
-                if (lane < NPOL) {
-                    float re = acc[0][0], im = acc[0][1];
+                    if (NPOL % 2) {
+                        const float2 g = single[o];
+                        a1[NPOL - 1] = __ffma2_rn(kxx, g, a1[NPOL - 1]);
+                        a2[NPOL - 1] = __ffma2_rn(kyy, g, a2[NPOL - 1]);
+                    }
+                };
+                auto advance = [&]() {
+                    off += step;
+                    tu += dr;
+                    if (tu >= S) {
+                        tu -= S;
+                        off += wrap;
+                    }
+                };
+                // steps 0 .. nfull - 1 have a tap on every lane, step nfull on
+                // the lanes below n - 32 nfull.  Kernel values are loaded D steps
+                // ahead, unconditionally: past the slice they read the next
+                // slice or the table's zero slack, never used.
+                const int nfull = (n - 1) >> 5;
+                const TT* kp = K + lane;
+                TT kq[D];
 #pragma unroll
-                    for (int p = 1; p < NPOL; ++p)
-                        if (lane == p) { re = acc[p][0]; im = acc[p][1]; }
-                    store_vis(a.vis_out, a.vis_kind, (int64_t)id * NPOL + lane, re * a.table_inv,
-                              im * a.table_inv);
+                for (int d = 0; d < D; ++d) kq[d] = __ldg(kp + 32 * d);
+                kp += 32 * D;
+                int i = 0;
+                for (; i + D <= nfull; i += D) {
+#pragma unroll
+                    for (int d = 0; d < D; ++d) {
+                        const float2 k = TE::cvt(kq[d]);
+                        kq[d] = __ldg(kp + 32 * d);
+                        tap(k, off);
+                        advance();
+                    }
+                    kp += 32 * D;
+                }
+                // the last (< D) full steps and the partial one, from the front
+                // of the ring
+                for (; i <= nfull; ++i) {
+                    const bool live = i < nfull || lane + 32 * nfull < n;
+                    tap(live ? TE::cvt(kq[0]) : make_float2(0.f, 0.f), live ? off : zoff);
+                    advance();
+#pragma unroll
+                    for (int d = 0; d + 1 < D; ++d) kq[d] = kq[d + 1];
+                }
+                // conj(K_i) G with K_i = K (w >= 0) or conj K (w < 0):
+                // re = sum K.re G.re + s K.im G.im, im = sum K.re G.im - s K.im G.re
+                float acc[NPOL][2];
+#pragma unroll
+                for (int p = 0; p < NPOL; ++p) {
+                    acc[p][0] = fmaf(sg, a2[p].y, a1[p].x);
+                    acc[p][1] = fmaf(-sg, a2[p].x, a1[p].y);
+                }
+                if constexpr (NPOL == 4) {
+                    // reduce-scatter butterfly: lanes with bit 4 set keep pols 2, 3,
+                    // then bit 3 picks one of the two; 12 shuffles instead of 40
+                    const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0;
+                    const float k0r = (b4 ? acc[2][0] : acc[0][0]) +
+                                      __shfl_xor_sync(0xffffffffu, b4 ? acc[0][0] : acc[2][0], 16);
+                    const float k0i = (b4 ? acc[2][1] : acc[0][1]) +
+                                      __shfl_xor_sync(0xffffffffu, b4 ? acc[0][1] : acc[2][1], 16);
+                    const float k1r = (b4 ? acc[3][0] : acc[1][0]) +
+                                      __shfl_xor_sync(0xffffffffu, b4 ? acc[1][0] : acc[3][0], 16);
+                    const float k1i = (b4 ? acc[3][1] : acc[1][1]) +
+                                      __shfl_xor_sync(0xffffffffu, b4 ? acc[1][1] : acc[3][1], 16);
+                    float re = (b3 ? k1r : k0r) + __shfl_xor_sync(0xffffffffu, b3 ? k0r : k1r, 8);
+                    float im = (b3 ? k1i : k0i) + __shfl_xor_sync(0xffffffffu, b3 ? k0i : k1i, 8);
+#pragma unroll
+                    for (int d = 4; d > 0; d >>= 1) {
+                        re += __shfl_xor_sync(0xffffffffu, re, d);
+                        im += __shfl_xor_sync(0xffffffffu, im, d);
+                    }
+                    if ((lane & 7) == 0) {
+                        const int p = (b4 ? 2 : 0) + (b3 ? 1 : 0);
+                        finish(r, p, id, tv0, tv1 < S, re, im);
+                    }
+                } else {
+#pragma unroll
+                    for (int p = 0; p < NPOL; ++p)
+#pragma unroll
+                        for (int d = 16; d > 0; d >>= 1) {
+                            acc[p][0] += __shfl_xor_sync(0xffffffffu, acc[p][0], d);
+                            acc[p][1] += __shfl_xor_sync(0xffffffffu, acc[p][1], d);
+                        }
+                    if (lane < NPOL) {
+                        float re = acc[0][0], im = acc[0][1];
+#pragma unroll
+                        for (int p = 1; p < NPOL; ++p)
+                            if (lane == p) { re = acc[p][0]; im = acc[p][1]; }
+                        finish(r, lane, id, tv0, tv1 < S, re, im);
+                    }
                 }
             }
+            __syncthreads();   // band consumed; after the last, the next chunk's metadata is in place
         }
-        __syncthreads();   // chunk consumed, the next chunk's metadata in place
     }
 }
 
-template <int NPOL, int TK>
-bool launch_staged_t(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s) {
-    const int RS = kStagedTile + 2 * hmax;
-    if ((size_t)RS * RS * NPOL * sizeof(float2) > kStagedSmemMax) return false;
-    const size_t smem = (size_t)(RS * RS + kStagedPad) * NPOL * sizeof(float2) +
-                        2 * kStagedMeta * sizeof(uint4);
-    cudaFuncSetAttribute(k_degrid_staged<NPOL, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_degrid_staged<NPOL, TK>,
-                                                  kStagedThreads, smem);
-    if (per_sm < 1) return false;
-    k_degrid_staged<NPOL, TK><<<num_sms * per_sm, kStagedThreads, smem, s>>>(a, hmax);
+template <int NPOL, int TK, bool GEN>
+void launch_staged_g(const DegridArgs& a, int hmax, size_t cap, size_t part, int num_sms,
+                     cudaStream_t s) {
+    const size_t smem = (cap + kStagedPad) * NPOL * sizeof(float2) +
+                        2 * kStagedMeta * sizeof(uint4) + part;
+    cudaFuncSetAttribute(k_degrid_staged<NPOL, TK, GEN>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_degrid_staged<NPOL, TK, GEN><<<num_sms, kStagedThreads, smem, s>>>(a, hmax, (int)cap);
     note_launch();
-    return true;
+}
+
+template <int NPOL, int TK>
+void launch_staged_t(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s) {
+    // grid points of the largest region where it fits, else as many as fit
+    // beside the partial sums of a chunk
+    const int RS = (1 << a.tile_shift) + 2 * hmax;
+    constexpr size_t point = NPOL * sizeof(float2);
+    size_t cap = (size_t)RS * RS, part = 0;
+    if (cap * point > kStagedSmemMax) {
+        part = kStagedMeta * point;
+        cap = (kStagedSmemMax - part) / point / 4 * 4;
+    }
+    if (part || a.tile_shift != 4)
+        launch_staged_g<NPOL, TK, true>(a, hmax, cap, part, num_sms, s);
+    else
+        launch_staged_g<NPOL, TK, false>(a, hmax, cap, part, num_sms, s);
 }
 
 template <int TK>
-bool launch_staged_k(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s) {
+void launch_staged_k(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s) {
     switch (a.npol) {
-        case 1: return launch_staged_t<1, TK>(a, hmax, num_sms, s);
-        case 2: return launch_staged_t<2, TK>(a, hmax, num_sms, s);
-        case 3: return launch_staged_t<3, TK>(a, hmax, num_sms, s);
-        default: return launch_staged_t<4, TK>(a, hmax, num_sms, s);
+        case 1: launch_staged_t<1, TK>(a, hmax, num_sms, s); break;
+        case 2: launch_staged_t<2, TK>(a, hmax, num_sms, s); break;
+        case 3: launch_staged_t<3, TK>(a, hmax, num_sms, s); break;
+        default: launch_staged_t<4, TK>(a, hmax, num_sms, s); break;
     }
 }
 
@@ -623,8 +676,6 @@ void launch_k(const DegridArgs& a, int64_t nvis, int num_sms, cudaStream_t s) {
 }
 
 }  // namespace
-
-int degrid_staged_tile() { return kStagedTile; }
 
 cudaError_t preload_degrid_kernel(int npol, int table_kind) {
     cudaFuncAttributes attr;
@@ -646,17 +697,12 @@ cudaError_t preload_degrid_kernel(int npol, int table_kind) {
     }
 }
 
-bool degrid_staged_fits(int hmax, int npol) {
-    const int RS = kStagedTile + 2 * hmax;
-    return (size_t)RS * RS * npol * sizeof(float2) <= kStagedSmemMax;
-}
-
-bool launch_degrid_staged(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s) {
+void launch_degrid_staged(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s) {
     cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), s);
     switch (a.table_kind) {
-        case GW_BF16X2: return launch_staged_k<GW_BF16X2>(a, hmax, num_sms, s);
-        case GW_F16X2: return launch_staged_k<GW_F16X2>(a, hmax, num_sms, s);
-        default: return launch_staged_k<GW_C64>(a, hmax, num_sms, s);
+        case GW_BF16X2: launch_staged_k<GW_BF16X2>(a, hmax, num_sms, s); break;
+        case GW_F16X2: launch_staged_k<GW_F16X2>(a, hmax, num_sms, s); break;
+        default: launch_staged_k<GW_C64>(a, hmax, num_sms, s); break;
     }
 }
 

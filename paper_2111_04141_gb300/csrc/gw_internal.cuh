@@ -393,6 +393,10 @@ constexpr int64_t kGroupTargetBytes = 64ll << 20;
 // Bands of tile rows a banded read-back may use (gw_grid_vis_devcount_readback).
 constexpr int kReadbackBandsMax = 64;
 constexpr int64_t kDirectMaxTaps = (int64_t)1 << 22;
+// Staged degridding takes 32 x 32 and 64 x 64 centre tiles instead of 16 x 16
+// below this many visibilities per 16 x 16 points on average.
+constexpr double kStagedSparse32 = 48.0;
+constexpr double kStagedSparse64 = 6.0;
 // One instantiation set per table kind (gw_grid_c64.cu, gw_grid_bf16.cu, gw_grid_f16.cu,
 // gw_grid_r32.cu).
 void launch_grid_c64(const GridArgs& a, int num_sms, cudaStream_t s);
@@ -435,11 +439,12 @@ struct DegridArgs {
     int N, npol, beta;
     int vis_kind = GW_C64, table_kind = GW_C64;
     float table_inv = 1.f;      // 2^-exp2: undoes the table storage scale
-    // staged kernel only: work items over 16 x 16 centre tiles
+    // staged kernel only: work items over centre tiles
     const Item* items = nullptr;
     const uint32_t* item_count = nullptr;
     uint32_t* queue = nullptr;
     int ntiles_u = 0;
+    int tile_shift = 4;         // centre tiles of 2^tile_shift points a side
     // debug bounds checks (0: unknown, not checked)
     int64_t table_elems = 0;    // elements of `table`, slack included
     int64_t vis_count = 0;      // visibilities of vis_out
@@ -454,6 +459,11 @@ void launch_degrid_direct(const DegridArgs& a, const DirectIndex& di, unsigned l
 // Staged-degrid region budget (bytes): the 227 KB a CTA may hold, less two
 // buffers of 1,024 records' metadata and the static shared memory.
 constexpr size_t kStagedSmemMax = 232448 - 2 * 1024 * 16 - 512;
+// Whether the largest region of 16 x 16 tiles is served in bands of rows.
+inline bool staged_banded(int hmax, int npol) {
+    const size_t RS = 16 + 2 * (size_t)hmax;
+    return RS * RS * npol * sizeof(float2) > kStagedSmemMax;
+}
 // Device status word bits (the word after the work-queue head): a bounded
 // wait gave up; a bounds check of the debug build failed.
 constexpr uint32_t kStatusTimeout = 1u;
@@ -473,10 +483,7 @@ __device__ __forceinline__ constexpr bool gw_in_bounds(bool, uint32_t*) { return
 // Zeroed elements after the last kernel slice of the unpadded tables: the
 // staged degridder loads kernel values up to this many elements past a slice.
 constexpr int64_t kTableSlack = 256;
-int degrid_staged_tile();
-bool degrid_staged_fits(int hmax, int npol);
-// Returns false (nothing launched) if the region does not fit.
-bool launch_degrid_staged(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s);
+void launch_degrid_staged(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s);
 
 // ---- full compression (gw_compress.cu) --------------------------------------
 struct CompressScratch {
