@@ -115,7 +115,7 @@ struct TableSet {
     uint32_t* table16 = nullptr;
     void* ptable = nullptr;
     int64_t* d_pplane_off = nullptr;
-    uint32_t* pairs = nullptr;
+    void* pairs = nullptr;
     int64_t* d_pair_off = nullptr;
     int64_t* d_plane_off = nullptr;
     int* d_support = nullptr;
@@ -181,8 +181,9 @@ struct gw_plan_s {
     float table_inv = 1.f;        // 2^-table_exp2
     std::vector<int64_t> pplane_off;
     int64_t* d_pplane_off = nullptr;
-    // pair tables of the 16-bit gridder (tables and visibilities of one 16-bit kind)
-    uint32_t* pairs = nullptr;
+    // pair tables: FP32 complex kernels of at most kPairPolMax polarisations
+    // (instead of ptable), or tables and visibilities of one 16-bit kind
+    void* pairs = nullptr;
     std::vector<int64_t> pair_off;
     int64_t* d_pair_off = nullptr;
     int64_t* d_plane_off = nullptr;
@@ -201,7 +202,7 @@ struct gw_plan_s {
 namespace {
 
 void free_tables(float2* table, uint32_t* table16, void* ptable, int64_t* d_pplane_off,
-                 uint32_t* pairs, int64_t* d_pair_off, int64_t* d_plane_off, int* d_support,
+                 void* pairs, int64_t* d_pair_off, int64_t* d_plane_off, int* d_support,
                  double* d_h, float* d_hf) {
     dev_free(pairs);
     dev_free(d_pair_off);
@@ -550,25 +551,30 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     // 2-D plans (P = 1) grid with the real w = 0 kernel: its imaginary parts
     // are exactly zero, so the gridder's padded table keeps the real parts
     p->grid_tk = desc->table_dtype == GW_C64 && P == 1 ? kTabRealF32 : desc->table_dtype;
+    const bool pairs_only = p->grid_tk == GW_C64 && desc->npol <= kPairPolMax;
     if (p->grid_tk == kTabRealF32) {
         float* pt = nullptr;
         GW_ALLOC(pt, (size_t)p->pplane_off[P]);
         p->ptable = pt;
     } else if (desc->table_dtype == GW_C64) {
-        float2* pt = nullptr;
-        GW_ALLOC(pt, (size_t)p->pplane_off[P]);
-        p->ptable = pt;
+        if (!pairs_only) {
+            float2* pt = nullptr;
+            GW_ALLOC(pt, (size_t)p->pplane_off[P]);
+            p->ptable = pt;
+        }
     } else {
         uint32_t* pt = nullptr;
         GW_ALLOC(p->table16, (size_t)(p->plane_off[P] + kTableSlack));
         GW_ALLOC(pt, (size_t)p->pplane_off[P]);
         p->ptable = pt;
     }
-    if (desc->table_dtype != GW_C64 && desc->vis_dtype == desc->table_dtype) {
+    if (pairs_only || (desc->table_dtype != GW_C64 && desc->vis_dtype == desc->table_dtype)) {
         p->pair_off.assign(1, 1);
         for (int q = 0; q < P; ++q)
             p->pair_off.push_back(p->pair_off[q] + pair_table_pairs(p->support[q], beta));
-        GW_ALLOC(p->pairs, (size_t)(2 * p->pair_off[P]));
+        char* pt = nullptr;
+        GW_ALLOC(pt, (size_t)(2 * p->pair_off[P]) * dtype_bytes(desc->table_dtype));
+        p->pairs = pt;
         GW_ALLOC(p->d_pair_off, (size_t)P + 1);
     }
     // the slack after the last slice reads as zeros
@@ -633,14 +639,17 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
         p->c1_norm = nrm;
     }
     p->table_inv = std::ldexp(1.0f, -p->table_exp2);
-    if (desc->table_dtype == GW_C64)
+    if (!p->ptable)
+        ;   // the pair tables alone
+    else if (desc->table_dtype == GW_C64)
         launch_pad_tables(p->table, p->grid_tk, p->d_plane_off, p->d_pplane_off, p->d_support, P,
                           beta, p->pad_stride, p->ptable, s);
     else
         launch_pad_tables(p->table16, desc->table_dtype, p->d_plane_off, p->d_pplane_off,
                           p->d_support, P, beta, p->pad_stride, p->ptable, s);
     if (p->pairs)
-        launch_pair_tables(p->table16, p->d_plane_off, p->d_pair_off, p->d_support, P, beta,
+        launch_pair_tables(p->table16 ? (const void*)p->table16 : (const void*)p->table,
+                           desc->table_dtype, p->d_plane_off, p->d_pair_off, p->d_support, P, beta,
                            p->pairs, s);
     e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -658,10 +667,11 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     t->d_h = p->d_h;
     t->d_hf = p->d_hf;
     t->bytes = (int64_t)sizeof(float2) * (p->plane_off[P] + kTableSlack) +
-               (int64_t)(p->grid_tk == kTabRealF32 ? sizeof(float) : dtype_bytes(desc->table_dtype)) *
-                   p->pplane_off[P] +
+               (p->ptable ? (int64_t)(p->grid_tk == kTabRealF32 ? sizeof(float)
+                                                                : dtype_bytes(desc->table_dtype)) *
+                                p->pplane_off[P] : 0) +
                (p->table16 ? (int64_t)sizeof(uint32_t) * (p->plane_off[P] + kTableSlack) : 0) +
-               (p->pairs ? (int64_t)(2 * sizeof(uint32_t)) * p->pair_off[P] +
+               (p->pairs ? (int64_t)(2 * dtype_bytes(desc->table_dtype)) * p->pair_off[P] +
                                (int64_t)sizeof(int64_t) * (P + 1) : 0) +
                (int64_t)(2 * sizeof(int64_t) + sizeof(int)) * (P + 1) +
                (int64_t)(sizeof(double) + sizeof(float)) * N;

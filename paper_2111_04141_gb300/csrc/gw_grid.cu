@@ -53,22 +53,23 @@ __global__ void k_pad_tables_real(const float2* __restrict__ tab, const int64_t*
 }
 
 // Pair tables (layout at pair_table_pairs).
-__global__ void k_pair_tables(const uint32_t* __restrict__ tab, const int64_t* __restrict__ plane_off,
+template <class T>
+__global__ void k_pair_tables(const T* __restrict__ tab, const int64_t* __restrict__ plane_off,
                               const int64_t* __restrict__ pair_off, const int* __restrict__ support,
-                              int beta, uint32_t* __restrict__ pairs) {
+                              int beta, T* __restrict__ pairs) {
     const int p = blockIdx.y;
     const int S = support[p], W = S + 1;
     const int64_t per = (int64_t)S * W;
     const int64_t n = 2 * (int64_t)beta * beta * per;
-    const uint32_t* src = tab + plane_off[p];
-    uint32_t* dst = pairs + 2 * pair_off[p];
-    if (p == 0 && blockIdx.x == 0 && threadIdx.x < 2) pairs[threadIdx.x] = 0u;   // the zero pair
+    const T* src = tab + plane_off[p];
+    T* dst = pairs + 2 * pair_off[p];
+    if (p == 0 && blockIdx.x == 0 && threadIdx.x < 2) pairs[threadIdx.x] = T{};   // the zero pair
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t oc = e / per;                     // 2 x slice + copy
         const int rem = (int)(e - oc * per);
         const int row = rem / W, col = rem - row * W - (int)(oc & 1);
-        dst[e] = col >= 0 && col < S ? src[(oc >> 1) * S * S + (int64_t)row * S + col] : 0u;
+        dst[e] = col >= 0 && col < S ? src[(oc >> 1) * S * S + (int64_t)row * S + col] : T{};
     }
 }
 
@@ -286,9 +287,16 @@ void launch_pad_tables(const void* tab, int kind, const int64_t* plane_off,
     note_launch();
 }
 
-void launch_pair_tables(const uint32_t* tab, const int64_t* plane_off, const int64_t* pair_off,
-                        const int* support, int P, int beta, uint32_t* pairs, cudaStream_t s) {
-    k_pair_tables<<<dim3(256, P), 256, 0, s>>>(tab, plane_off, pair_off, support, beta, pairs);
+void launch_pair_tables(const void* tab, int kind, const int64_t* plane_off,
+                        const int64_t* pair_off, const int* support, int P, int beta, void* pairs,
+                        cudaStream_t s) {
+    const dim3 grid(256, P);
+    if (kind == GW_C64)
+        k_pair_tables<<<grid, 256, 0, s>>>(static_cast<const float2*>(tab), plane_off, pair_off,
+                                           support, beta, static_cast<float2*>(pairs));
+    else
+        k_pair_tables<<<grid, 256, 0, s>>>(static_cast<const uint32_t*>(tab), plane_off, pair_off,
+                                           support, beta, static_cast<uint32_t*>(pairs));
     note_launch();
 }
 

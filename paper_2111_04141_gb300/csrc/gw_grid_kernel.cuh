@@ -72,6 +72,8 @@
 //   address arithmetic cost more than the FMAs they replace.
 #pragma once
 
+#include <type_traits>
+
 #include "gw_internal.cuh"
 
 // Kernel-value register sets in flight per FP32 compute warp (measured on the
@@ -384,6 +386,169 @@ struct FmaWarp {
     };
 };
 
+// Commits the sums s0, s1 of points (u, v) and (u + 1, v), u even, of
+// polarisation p: both in one 16-byte reduction where the grid's alignment
+// allows (N is even).
+__device__ __forceinline__ void commit_pair(const GridArgs& a, float2* gbase, int u, int v, int p,
+                                            float2 s0, float2 s1) {
+    const int N = a.N;
+    const float4 q = make_float4(s0.x * a.table_inv, s0.y * a.table_inv, s1.x * a.table_inv,
+                                 s1.y * a.table_inv);
+    const bool n0 = q.x != 0.f || q.y != 0.f, n1 = q.z != 0.f || q.w != 0.f;
+    if (u >= N || v >= N || !(n0 || n1)) return;
+    const int64_t off = ((int64_t)p * N + v) * N + u;
+    const float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
+    if (a.grid_err) {
+        if (n0) commit_compensated(gbase + off, a.grid_err + off, q0);
+        if (n1) commit_compensated(gbase + off + 1, a.grid_err + off + 1, q1);
+    } else if ((reinterpret_cast<uintptr_t>(gbase) & 15u) == 0) {
+        atomicAdd(reinterpret_cast<float4*>(gbase + off), q);
+    } else {
+        if (n0) atomicAdd(gbase + off, q0);
+        if (n1) atomicAdd(gbase + off + 1, q1);
+    }
+}
+
+// ---- compute warps over pair tables ---------------------------------------------
+// Blocks of 16 (u) x 8 (v) points, kernel values in aligned pairs of horizontally
+// adjacent points (layout at pair_table_pairs).  List entry: x = pair index of
+// the block's column 0, row 0 (modulo 2^32; only columns and rows inside the
+// footprint are loaded); y = record row in the batch (bits 0-7), pairs per
+// table row less one (8-14), conjugate kernel (15), rows (16-23) and column
+// pairs (24-31) that the footprint meets.
+constexpr uint32_t kPairConj = 1u << 15;
+constexpr int kPairRows = 16, kPairCols = 24;
+
+// Producer: list entries of a record over the pair tables.
+struct PairEntries {
+    static constexpr int kBlockU = 16, kBlockV = 8;
+    uint32_t base, ey;
+    int Q, pc0;
+    __device__ __forceinline__ PairEntries(const GridArgs& a, const gw_index_rec& rc, int plane, int S,
+                                       int r, int ulo, int vlo) {
+        Q = (S + 1) / 2;                       // pairs per table row
+        // the copy of the slice whose pairs line up with the tile's even
+        // columns, and the pair column of the tile's column 0
+        const int odd = ulo & 1;
+        pc0 = (odd - ulo) / 2;
+        const int64_t slice =
+            __ldg(a.pair_off + plane) +
+            (2 * ((int64_t)(rc.ov + a.beta / 2) * a.beta + (rc.ou + a.beta / 2)) + odd) *
+                (int64_t)(S * Q);
+        base = (uint32_t)slice + (uint32_t)(pc0 - vlo * Q);
+        ey = (uint32_t)r | (uint32_t)(Q - 1) << 8 | ((rc.flags & GW_FLAG_CONJ) ? kPairConj : 0u);
+    }
+    __device__ __forceinline__ uint2 operator()(int cu, int cv, int j0, int j1) const {
+        const int pc = pc0 + kBlockU / 2 * cu;
+        const int lo = max(0, -pc), hi = min(kBlockU / 2 - 1, Q - 1 - pc);
+        const uint32_t rows = ((2u << j1) - 1u) & ~((1u << j0) - 1u);
+        const uint32_t cols = (2u << hi) - (1u << lo);
+        return make_uint2(base + (uint32_t)(kBlockV * cv * Q + kBlockU / 2 * cu),
+                          ey | rows << kPairRows | cols << kPairCols);
+    }
+    // first and last pair the entry's loads touch
+    __device__ __forceinline__ void span(uint2 e, int cu, int, int j0, int j1, int64_t& lo,
+                                         int64_t& hi) const {
+        const int pc = pc0 + kBlockU / 2 * cu;
+        lo = (int64_t)(uint32_t)(e.x + (uint32_t)(j0 * Q + max(0, -pc)));
+        hi = (int64_t)(uint32_t)(e.x + (uint32_t)(j1 * Q + min(kBlockU / 2 - 1, Q - 1 - pc)));
+    }
+};;
+
+// FP32 tables with one or two polarisations.  With so few FMAs an entry the
+// gathers bound the kernel (each a quarter-warp's cache lines), and a 16-byte
+// load of a pair takes 8 lanes through one 128-byte row: about 7.5 lines for
+// 64 points against 11.5 for two 8-byte loads of 8 x 4 points.  4.2 M
+// visibilities, 1 polarisation, support 31, 2048^2: 3.65 ms with FmaWarp; here
+// 3.30 / 3.23 / 2.98 / 2.90 with 3 / 4 / 5 / 6 entries in flight.  With more
+// polarisations the FMAs share the bound and the 8 x 16 blocks of FmaWarp
+// stay ahead (4: 8.2 against 9.2 ms on the 4096^2 batch).
+// Lane (g, r) = (lane % 8, lane / 8): points 2 g, 2 g + 1 of rows r and r + 4.
+template <int NPOL>
+struct PairWarp {
+    using VT = float2;                         // staged visibility
+    static constexpr int kPol = NPOL, R = NPOL == 1 ? 6 : 5;   // entries in flight
+    static constexpr int kBlockU = 16, kBlockV = 8;
+    static constexpr int kBatch = kRows - 1;   // rows 0 .. 254, and the zero row 255
+    static constexpr uint32_t kZeroRow = kBatch;
+    static constexpr int kVisRows = kRows;
+    float2 acc[4][NPOL];                       // (row slot, point of the pair), (re, im)
+    float4 K[R][2];
+    uint32_t ey[R];
+    const float4* __restrict__ tab;
+    uint32_t g, r;
+
+    __device__ __forceinline__ PairWarp(const GridArgs& a, int, int lane) {
+        tab = reinterpret_cast<const float4*>(a.pair_table);
+        g = lane & 7;
+        r = lane >> 3;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) acc[j][p] = make_float2(0.f, 0.f);
+    }
+    // kernel values of an entry, zero outside its footprint
+    __device__ __forceinline__ void load(int d, const uint2 en) {
+        const uint32_t q = ((en.y >> 8) & 0x7fu) + 1u, off = en.x + g + r * q;
+        const uint32_t c = 1u << (kPairCols + g);
+        const uint32_t m0 = c | 1u << (kPairRows + r), m1 = c | 1u << (kPairRows + 4 + r);
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        ey[d] = en.y;
+        K[d][0] = (en.y & m0) == m0 ? __ldg(tab + off) : z;
+        K[d][1] = (en.y & m1) == m1 ? __ldg(tab + (off + 4 * q)) : z;
+    }
+    __device__ __forceinline__ void fill(const uint2* lst, const VT (*)[NPOL]) {
+#pragma unroll
+        for (int d = 0; d < R; ++d) load(d, lst[d]);
+    }
+    // one ring pass: the FMAs of the R entries in the ring, each followed by
+    // the loads of the entry R positions later
+    __device__ __forceinline__ void pass(const uint2* next, const VT (*vs)[NPOL], const VT (*)[NPOL]) {
+#pragma unroll
+        for (int d = 0; d < R; ++d) {
+            const float2* row = vs[ey[d] & 0xffu];
+            const float s = (ey[d] & kPairConj) ? -1.f : 1.f;
+            float2 A[NPOL], Bv[NPOL];
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) {
+                A[p] = row[p];
+                Bv[p] = make_float2(-s * A[p].y, s * A[p].x);
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float kr = i ? K[d][j].z : K[d][j].x, ki = i ? K[d][j].w : K[d][j].y;
+#pragma unroll
+                    for (int p = 0; p < NPOL; ++p) {
+                        float2& c = acc[2 * j + i][p];
+                        c = __ffma2_rn(make_float2(kr, kr), A[p], c);
+                        c = __ffma2_rn(make_float2(ki, ki), Bv[p], c);
+                    }
+                }
+            load(d, next[d]);
+        }
+    }
+    __device__ __forceinline__ void commit(const GridArgs& a, float2* gbase, int u0, int v0, int) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) {
+                commit_pair(a, gbase, u0 + 2 * (int)g, v0 + (int)r + 4 * j, p, acc[2 * j][p],
+                            acc[2 * j + 1][p]);
+                acc[2 * j][p] = acc[2 * j + 1][p] = make_float2(0.f, 0.f);
+            }
+    }
+    static __device__ __forceinline__ bool copies(const GridArgs& a) {
+        return FmaWarp<NPOL, 0, GW_C64>::copies(a);
+    }
+    static __device__ __forceinline__ void stage(const GridArgs& a, bool copy, VT (&row)[NPOL],
+                                                 uint32_t id) {
+        FmaWarp<NPOL, 0, GW_C64>::stage(a, copy, row, id);
+    }
+    using Entries = PairEntries;
+};
+
 // ---- compute warps: 16-bit tensor cores -----------------------------------------
 // Tables and visibilities of one 16-bit kind: the products of 16-bit values
 // are exact in FP32, so a group of 8 records is one m16n8k16 product per
@@ -393,14 +558,6 @@ struct FmaWarp {
 // ordinary (rounded) additions.  Lane (g, t) = (lane / 4, lane % 4) loads
 // column pair g of records t and t + 4 and holds polarisation t of points 2 g,
 // 2 g + 1; pairs come from the pair tables (layout at pair_table_pairs).
-//
-// List entry: x = pair index of the block's column 0, row 0 (modulo 2^32; only
-// columns and rows inside the footprint are loaded); y = record row in the
-// batch (bits 0-7), pairs per table row less one (8-14), conjugate kernel
-// (15), rows (16-23) and column pairs (24-31) that the footprint meets.
-constexpr uint32_t kMmaConj = 1u << 15;
-constexpr int kMmaRows = 16, kMmaCols = 24;
-
 template <int TK>
 __device__ __forceinline__ void mma_16(float (&d)[4], const uint32_t (&a)[4],
                                        const uint32_t (&b)[2]) {
@@ -450,7 +607,7 @@ struct MmaWarp {
             const uint2 en = lst[4 * k + t];
             c.off[k] = en.x + g;
             c.q[k] = ((en.y >> 8) & 0x7fu) + 1u;
-            c.m[k] = (en.y >> (kMmaCols + g)) & 1u ? en.y >> kMmaRows : 0u;
+            c.m[k] = (en.y >> (kPairCols + g)) & 1u ? en.y >> kPairRows : 0u;
             // column g of B: component (re, im) g & 1 of polarisation g / 2;
             // (K.re, K.im) multiply (V.re, -s V.im) or (V.im, s V.re), s = -1 for
             // the conjugate kernel
@@ -458,7 +615,7 @@ struct MmaWarp {
             if (NPOL == 4 || (int)(g >> 1) < NPOL) {
                 w = vs[en.y & 0xffu][g >> 1];
                 w = __byte_perm(w, 0, (g & 1) ? 0x1032 : 0x3210) ^
-                    ((~g << 31) ^ ((en.y & kMmaConj) << 16));
+                    ((~g << 31) ^ ((en.y & kPairConj) << 16));
             }
             b[k] = w;
         }
@@ -498,31 +655,13 @@ struct MmaWarp {
             load(j, c);
         }
     }
-    // Commits the block's accumulators; both points of a pair in one 16-byte
-    // reduction where the grid's alignment allows (N and the blocks are even).
-    // Lanes of polarisations beyond NPOL hold zeros.
+    // Commits the block's accumulators (polarisations beyond NPOL hold zeros,
+    // which are not committed).
     __device__ __forceinline__ void commit(const GridArgs& a, float2* gbase, int u0, int v0, int) {
-        const int N = a.N, u = u0 + 2 * (int)g;
-        const bool vec = (reinterpret_cast<uintptr_t>(gbase) & 15u) == 0 && a.grid_err == nullptr;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int v = v0 + j;
-            const float4 q = make_float4(acc[j][0] * a.table_inv, acc[j][1] * a.table_inv,
-                                         acc[j][2] * a.table_inv, acc[j][3] * a.table_inv);
-            const bool n0 = q.x != 0.f || q.y != 0.f, n1 = q.z != 0.f || q.w != 0.f;
-            if ((int)t < NPOL && u < N && v < N && (n0 || n1)) {
-                const int64_t off = ((int64_t)t * N + v) * N + u;
-                const float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
-                if (vec) {
-                    atomicAdd(reinterpret_cast<float4*>(gbase + off), q);
-                } else if (a.grid_err) {
-                    if (n0) commit_compensated(gbase + off, a.grid_err + off, q0);
-                    if (n1) commit_compensated(gbase + off + 1, a.grid_err + off + 1, q1);
-                } else {
-                    if (n0) atomicAdd(gbase + off, q0);
-                    if (n1) atomicAdd(gbase + off + 1, q1);
-                }
-            }
+            commit_pair(a, gbase, u0 + 2 * (int)g, v0 + j, (int)t, make_float2(acc[j][0], acc[j][1]),
+                        make_float2(acc[j][2], acc[j][3]));
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[j][i] = 0.f;
         }
@@ -547,45 +686,16 @@ struct MmaWarp {
             for (int p = 0; p < NPOL; ++p) row[p] = __ldg(src + p);
         }
     }
-    struct Entries {
-        uint32_t base, ey;
-        int Q, pc0;
-        __device__ __forceinline__ Entries(const GridArgs& a, const gw_index_rec& rc, int plane, int S,
-                                           int r, int ulo, int vlo) {
-            Q = (S + 1) / 2;                       // pairs per table row
-            // the copy of the slice whose pairs line up with the tile's even
-            // columns, and the pair column of the tile's column 0
-            const int odd = ulo & 1;
-            pc0 = (odd - ulo) / 2;
-            const int64_t slice =
-                __ldg(a.pair_off + plane) +
-                (2 * ((int64_t)(rc.ov + a.beta / 2) * a.beta + (rc.ou + a.beta / 2)) + odd) *
-                    (int64_t)(S * Q);
-            base = (uint32_t)slice + (uint32_t)(pc0 - vlo * Q);
-            ey = (uint32_t)r | (uint32_t)(Q - 1) << 8 | ((rc.flags & GW_FLAG_CONJ) ? kMmaConj : 0u);
-        }
-        __device__ __forceinline__ uint2 operator()(int cu, int cv, int j0, int j1) const {
-            const int pc = pc0 + kBlockU / 2 * cu;
-            const int lo = max(0, -pc), hi = min(kBlockU / 2 - 1, Q - 1 - pc);
-            const uint32_t rows = ((2u << j1) - 1u) & ~((1u << j0) - 1u);
-            const uint32_t cols = (2u << hi) - (1u << lo);
-            return make_uint2(base + (uint32_t)(kBlockV * cv * Q + kBlockU / 2 * cu),
-                              ey | rows << kMmaRows | cols << kMmaCols);
-        }
-        // first and last pair the entry's loads touch
-        __device__ __forceinline__ void span(uint2 e, int cu, int, int j0, int j1, int64_t& lo,
-                                             int64_t& hi) const {
-            const int pc = pc0 + kBlockU / 2 * cu;
-            lo = (int64_t)(uint32_t)(e.x + (uint32_t)(j0 * Q + max(0, -pc)));
-            hi = (int64_t)(uint32_t)(e.x + (uint32_t)(j1 * Q + min(kBlockU / 2 - 1, Q - 1 - pc)));
-        }
-    };
+    using Entries = PairEntries;
 };
 
-template <int NPOL, int SP, int TK, bool NAT>
+// PAIRS: the compute warps that read the pair tables.
+template <int NPOL, int SP, int TK, bool PAIRS>
 struct PickWarp { using W = FmaWarp<NPOL, SP, TK>; };
 template <int NPOL, int SP, int TK>
-struct PickWarp<NPOL, SP, TK, true> { using W = MmaWarp<NPOL, TK>; };
+struct PickWarp<NPOL, SP, TK, true> {
+    using W = std::conditional_t<TK == GW_C64, PairWarp<NPOL>, MmaWarp<NPOL, TK>>;
+};
 
 template <class W, int B>
 struct Smem {
@@ -600,9 +710,9 @@ struct Smem {
     unsigned long long full[B], empty[B];  // mbarriers
 };
 
-template <int NPOL, int SP, int TK, bool NAT, int B>
+template <int NPOL, int SP, int TK, bool PAIRS, int B>
 __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
-    using W = typename PickWarp<NPOL, SP, TK, NAT>::W;
+    using W = typename PickWarp<NPOL, SP, TK, PAIRS>::W;
     using VT = typename W::VT;
     constexpr int R = W::R, kBatch = W::kBatch, kBlockU = W::kBlockU, kBlockV = W::kBlockV;
     constexpr int kBlocksU = kGridTileU / kBlockU;
@@ -706,7 +816,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
 #ifdef GW_DEBUG_BOUNDS
                                 int64_t lo, hi;
                                 entry.span(e, cu, cv, j0, j1, lo, hi);
-                                const int64_t n = NAT ? a.pair_count : a.ptable_elems;
+                                const int64_t n = PAIRS ? a.pair_count : a.ptable_elems;
                                 if (!gw_in_bounds(n == 0 || (lo >= 0 && lo <= hi && hi < n), a.queue + 1))
                                     continue;
 #endif
@@ -800,44 +910,48 @@ __global__ void __launch_bounds__(kThreads, 1) k_grid(GridArgs a) {
 #ifndef GW_GRID_BUFS
 #define GW_GRID_BUFS 4
 #endif
-template <int NPOL, int SP, int TK, bool NAT>
+template <int NPOL, int SP, int TK, bool PAIRS>
 void launch_sp(const GridArgs& a, int num_sms, cudaStream_t s) {
     constexpr int B = GW_GRID_BUFS;
-    const size_t smem = sizeof(Smem<typename PickWarp<NPOL, SP, TK, NAT>::W, B>);
-    cudaFuncSetAttribute(k_grid<NPOL, SP, TK, NAT, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t smem = sizeof(Smem<typename PickWarp<NPOL, SP, TK, PAIRS>::W, B>);
+    cudaFuncSetAttribute(k_grid<NPOL, SP, TK, PAIRS, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grid<NPOL, SP, TK, NAT, B>, kThreads,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grid<NPOL, SP, TK, PAIRS, B>, kThreads,
                                                   smem);
     if (per_sm < 1) per_sm = 1;
-    k_grid<NPOL, SP, TK, NAT, B><<<num_sms * per_sm, kThreads, smem, s>>>(a);
+    k_grid<NPOL, SP, TK, PAIRS, B><<<num_sms * per_sm, kThreads, smem, s>>>(a);
     note_launch();
 }
 
 template <int NPOL, int TK>
 void launch_t(const GridArgs& a, int num_sms, cudaStream_t s) {
-    if constexpr (TK == GW_BF16X2 || TK == GW_F16X2) {
-        if (a.pair_table && a.vis_kind == TK && !a.weight) {
-            launch_sp<NPOL, 0, TK, true>(a, num_sms, s);
-            return;
+    if constexpr (TK == GW_C64 && NPOL <= kPairPolMax) {
+        launch_sp<NPOL, 0, TK, true>(a, num_sms, s);       // such plans have pair tables only
+    } else {
+        if constexpr (TK == GW_BF16X2 || TK == GW_F16X2) {
+            if (a.pair_table && a.vis_kind == TK && !a.weight) {
+                launch_sp<NPOL, 0, TK, true>(a, num_sms, s);
+                return;
+            }
         }
-    }
-    switch (a.pad_stride) {
+        switch (a.pad_stride) {
 #if GW_GRID_LANES_U == 16
-        case 32: launch_sp<NPOL, 32, TK, false>(a, num_sms, s); break;
-        case 48: launch_sp<NPOL, 48, TK, false>(a, num_sms, s); break;
-        case 64: launch_sp<NPOL, 64, TK, false>(a, num_sms, s); break;
-        case 96: launch_sp<NPOL, 96, TK, false>(a, num_sms, s); break;
-        case 160: launch_sp<NPOL, 160, TK, false>(a, num_sms, s); break;
-        default: launch_sp<NPOL, 288, TK, false>(a, num_sms, s); break;
+            case 32: launch_sp<NPOL, 32, TK, false>(a, num_sms, s); break;
+            case 48: launch_sp<NPOL, 48, TK, false>(a, num_sms, s); break;
+            case 64: launch_sp<NPOL, 64, TK, false>(a, num_sms, s); break;
+            case 96: launch_sp<NPOL, 96, TK, false>(a, num_sms, s); break;
+            case 160: launch_sp<NPOL, 160, TK, false>(a, num_sms, s); break;
+            default: launch_sp<NPOL, 288, TK, false>(a, num_sms, s); break;
 #else
-        case 24: launch_sp<NPOL, 24, TK, false>(a, num_sms, s); break;
-        case 32: launch_sp<NPOL, 32, TK, false>(a, num_sms, s); break;
-        case 48: launch_sp<NPOL, 48, TK, false>(a, num_sms, s); break;
-        case 80: launch_sp<NPOL, 80, TK, false>(a, num_sms, s); break;
-        case 144: launch_sp<NPOL, 144, TK, false>(a, num_sms, s); break;
-        default: launch_sp<NPOL, 272, TK, false>(a, num_sms, s); break;
+            case 24: launch_sp<NPOL, 24, TK, false>(a, num_sms, s); break;
+            case 32: launch_sp<NPOL, 32, TK, false>(a, num_sms, s); break;
+            case 48: launch_sp<NPOL, 48, TK, false>(a, num_sms, s); break;
+            case 80: launch_sp<NPOL, 80, TK, false>(a, num_sms, s); break;
+            case 144: launch_sp<NPOL, 144, TK, false>(a, num_sms, s); break;
+            default: launch_sp<NPOL, 272, TK, false>(a, num_sms, s); break;
 #endif
+        }
     }
 }
 

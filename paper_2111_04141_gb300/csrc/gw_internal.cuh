@@ -334,7 +334,7 @@ struct GridArgs {
     const gw_index_rec* rec;
     const void* ptable;          // zero-padded tables of kind table_kind (launch_pad_tables)
     const int64_t* pplane_off;   // device [P]: padded plane offsets
-    // pair tables (launch_pair_tables; null: none): gridding by 16-bit tensor cores
+    // pair tables (launch_pair_tables; null: none)
     const void* pair_table = nullptr;
     const int64_t* pair_off = nullptr;   // device [P]: plane offsets, in pairs
     int64_t pair_count = 0;              // pairs of pair_table (debug bounds checks)
@@ -415,7 +415,8 @@ void launch_pad_tables(const void* tab, int kind, const int64_t* plane_off,
                        const int64_t* pplane_off, const int* support, int P, int beta, int SP,
                        void* ptab, cudaStream_t s);
 
-// Pair tables of the 16-bit gridder: every S x S slice twice, each row extended
+// Pair tables of the 16-bit tensor-core gridder and of the FP32 gridder for at
+// most kPairPolMax polarisations (complex kernels): every S x S slice twice, each row extended
 // to S + 1 entries by a zero, after the row in the first copy and before it
 // in the second.  Whatever the parity of a footprint's first column, one of
 // the copies puts the points (2 x, 2 x + 1) of the grid into one aligned
@@ -424,8 +425,11 @@ void launch_pad_tables(const void* tab, int kind, const int64_t* plane_off,
 inline int64_t pair_table_pairs(int S, int beta) {
     return (int64_t)beta * beta * S * (S + 1);
 }
-void launch_pair_tables(const uint32_t* tab, const int64_t* plane_off, const int64_t* pair_off,
-                        const int* support, int P, int beta, uint32_t* pairs, cudaStream_t s);
+constexpr int kPairPolMax = 2;
+// tab and pairs hold elements of kind `kind` (8 bytes for GW_C64, else 4).
+void launch_pair_tables(const void* tab, int kind, const int64_t* plane_off,
+                        const int64_t* pair_off, const int* support, int P, int beta, void* pairs,
+                        cudaStream_t s);
 
 struct DegridArgs {
     const gw_index_rec* rec;

@@ -1,8 +1,8 @@
-"""The 16-bit tensor-core gridder (tables and visibilities of one 16-bit kind)
-at the edges of its tiles, blocks, groups and supports: against the FP64
-oracle run on exactly the stored values (the products of 16-bit values are
-exact in FP32, so only FP32 sums differ: relative L2 <= 1e-5, the tolerance
-of every FP32 grid)."""
+"""The gridders over pair tables (16-bit tensor cores; FP32 with one or two
+polarisations) at the edges of their tiles, blocks, groups and supports:
+against the FP64 oracle run on exactly the stored values (the products of
+16-bit values are exact in FP32, so only FP32 sums differ: relative L2 <= 1e-5,
+the tolerance of every FP32 grid)."""
 import numpy as np
 import pytest
 import torch
@@ -35,7 +35,9 @@ def case(kind, npol, n, smin, smax, n_w, beta=8, n_times=10):
     prm = Params(**obs.plan_kwargs())
     vis = to_storage(torch.from_numpy(obs.vis), kind)
     held = from_storage(vis).numpy().astype(np.complex128)
-    ref = Oracle(prm, QuantisedTables(KernelTables(prm), kind)).grid(obs.uvw_m, obs.freq_hz, held)
+    kt = KernelTables(prm)
+    ref = Oracle(prm, kt if kind == "c64" else QuantisedTables(kt, kind)).grid(
+        obs.uvw_m, obs.freq_hz, held)
     return obs, vis.to(DEV), ref
 
 
@@ -43,16 +45,25 @@ def case(kind, npol, n, smin, smax, n_w, beta=8, n_times=10):
 # than a tile, every polarisation count, oversampling that is no power of two
 @pytest.mark.parametrize("kind,npol,n,smin,smax,n_w,beta", [
     ("bf16", 1, 66, 1, 1, 1, 8), ("f16", 2, 98, 3, 5, 2, 6), ("bf16", 3, 130, 7, 15, 4, 8),
-    ("f16", 4, 142, 5, 33, 3, 4), ("bf16", 4, 254, 15, 79, 5, 4), ("f16", 1, 190, 7, 65, 3, 2)])
+    ("f16", 4, 142, 5, 33, 3, 4), ("bf16", 4, 254, 15, 79, 5, 4), ("f16", 1, 190, 7, 65, 3, 2),
+    ("c64", 1, 66, 1, 3, 2, 8), ("c64", 2, 98, 3, 5, 2, 6), ("c64", 1, 142, 5, 33, 3, 4),
+    ("c64", 2, 254, 15, 79, 5, 4), ("c64", 1, 600, 41, 255, 3, 2)])
 def test_grid_matches_oracle_on_stored_values(gw, kind, npol, n, smin, smax, n_w, beta):
     obs, vis, ref = case(kind, npol, n, smin, smax, n_w, beta)
     uvw, freq = torch.from_numpy(obs.uvw_m).to(DEV), torch.from_numpy(obs.freq_hz).to(DEV)
     with gw.Plan.from_observation(obs, table_dtype=kind, vis_dtype=kind) as plan:
         plan.set_tuning(grid_kernel=1)
+        err = torch.zeros((npol, n, n), dtype=torch.complex64, device=DEV)
+        comp = plan.grid(uvw, freq, vis, err=err)            # compensated commits
+        plan.fold(comp, err)
+        c = comp.cpu().numpy().astype(np.complex128)
+        assert np.linalg.norm(c - ref) / np.linalg.norm(ref) <= TOL
         # a buffer whose visibilities start one element (4 bytes) off, and a
         # grid on an odd 8-byte boundary: the narrow copies and commits
-        buf = torch.empty(vis.numel() + 2, dtype=vis.dtype, device=DEV)
-        odd = buf[2:].view(vis.shape)
+        # (FP32 pairs of polarisations have to start on 16 bytes)
+        skip = 2 if kind != "c64" else int(npol == 1)
+        buf = torch.empty(vis.numel() + skip, dtype=vis.dtype, device=DEV)
+        odd = buf[skip:].view(vis.shape)
         odd.copy_(vis)
         room = torch.zeros(plan.npol * n * n + 1, dtype=torch.complex64, device=DEV)
         off = room[1:].view(plan.npol, n, n)
