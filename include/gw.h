@@ -131,8 +131,10 @@ typedef struct {
  * FP32 summation order. */
 typedef struct {
     int32_t item_max;       /* records per gridding / staged-degridding work item:
-                               0 = 1024, else 64 .. 2^20 (smaller items spread small
-                               jobs over more SMs, larger ones commit less often) */
+                               0 = automatic (gridding: 255, 510 or 1020 by the size
+                               of the call; staged degridding: 1024), else 64 .. 2^20
+                               (smaller items spread small jobs over more SMs, larger
+                               ones commit less often) */
     int32_t degrid_kernel;  /* 0 = automatic, 1 = shared-memory staged, 2 = global gather */
     int32_t grid_kernel;    /* gw_grid_vis / _compensated: 0 = automatic (direct for chunks of
                                at most 16,384 visibilities and 2^22 tap updates, else

@@ -816,8 +816,18 @@ static int grid_groups(gw_plan p) {
     const int g = p->tuning.plane_groups > 0 ? p->tuning.plane_groups : p->auto_groups;
     return std::max(1, std::min(g, p->max_groups));
 }
-static BinGeom grid_geom(gw_plan p, int groups) {
+// Gridder work items of nvis visibilities: shorter ones for smaller inputs,
+// which spread over more SMs (calls, us, with items of 128 / 256 / 512 / 1024
+// records: 30 k x 1 57.5 / 59.0 / 59.8 / 60.2, 121 k x 4 147 / 145 / 148 / 161,
+// 403 k x 2 292 / 272 / 276 / 290, 472 k x 3 427 / 400 / 391 / 395); multiples of
+// 255, which every gridder stages in whole batches.
+static int grid_items(gw_plan p, int64_t nvis) {
+    if (p->tuning.item_max > 0) return p->tuning.item_max;
+    return nvis <= 262144 ? 255 : (nvis <= 1048576 ? 510 : 1020);
+}
+static BinGeom grid_geom(gw_plan p, int groups, int64_t nvis) {
     BinGeom g = p->geom_grid;
+    g.item_max = grid_items(p, nvis);
     if (groups > 1) {
         g.layer_tiles = g.ntu * g.ntv;
         g.nlayers = groups;
@@ -940,7 +950,7 @@ static gw_status grid_impl(gw_plan p, const double* uvw_m, const double* freq_hz
             continue;
         }
         const int groups = grid_groups(p);
-        const BinGeom geom = grid_geom(p, groups);
+        const BinGeom geom = grid_geom(p, groups, nr * nchan);
         st = index_and_bin(p, uvw_m + 3 * r0, freq_hz, nr, nchan, geom, s);
         if (st != GW_OK) return st;
         GridArgs a;
