@@ -442,6 +442,17 @@ gw_status gw_grid_correct(gw_plan plan, void* image, int32_t direction, void* cu
  * for an FFT library.  Errors: GW_EINVAL, GW_EDEVICE, GW_ECUDA. */
 gw_status gw_grid_shift(gw_plan plan, void* grid, void* cuda_stream);
 
+/* gw_grid_shift and gw_grid_correct(+1) in one pass, with the normalisation:
+ * image (device, [npol][N][N] c64, in place) is the unnormalised inverse FFT
+ * of a grid that was NOT shifted, and
+ *     image[pol][i][j] = image[pol][(i + N/2) % N][(j + N/2) % N]
+ *                        * (-1)^(i+j) * h(m_i) * h(l_j) * scale * scale_dev[pol]
+ * (the shift of the grid is this circular shift of its transform).
+ *   scale_dev  device, [npol] float32, or NULL for ones
+ * Errors: GW_EINVAL, GW_EDEVICE, GW_ECUDA. */
+gw_status gw_image_finish(gw_plan plan, void* image, double scale, const float* scale_dev,
+                          void* cuda_stream);
+
 /* ------------------------------------------------------------------------
  * Stage access (testing, diagnostics, custom pipelines)
  * ------------------------------------------------------------------------ */

@@ -91,6 +91,7 @@ _SIGS = {
                                      ctypes.POINTER(c_i64), c_vp]),
     "gw_grid_correct": (c_i32, [c_vp, c_vp, c_i32, c_vp]),
     "gw_grid_shift": (c_i32, [c_vp, c_vp, c_vp]),
+    "gw_image_finish": (c_i32, [c_vp, c_vp, c_f64, c_vp, c_vp]),
     "gw_index_vis": (c_i32, [c_vp, c_vp, c_vp, c_i64, c_i32, c_vp, ctypes.POINTER(c_i64), c_vp]),
     "gw_plan_copy_tables": (c_i32, [c_vp, c_vp, c_vp, c_vp]),
     "gw_plan_copy_stored_tables": (c_i32, [c_vp, c_vp]),

@@ -1895,6 +1895,21 @@ gw_status gw_grid_correct(gw_plan p, void* image, int32_t direction, void* cuda_
     return e == cudaSuccess ? GW_OK : cuda_fail(e, "correct launch");
 }
 
+gw_status gw_image_finish(gw_plan p, void* image, double scale, const float* scale_dev,
+                          void* cuda_stream) {
+    if (!p) return fail(GW_EINVAL, "null plan");
+    gw_status st = check_device(p);
+    if (st != GW_OK) return st;
+    if (!image) return fail(GW_EINVAL, "null image");
+    if (reinterpret_cast<uintptr_t>(image) % 8 != 0 ||
+        reinterpret_cast<uintptr_t>(scale_dev) % 4 != 0)
+        return fail(GW_EINVAL, "image must be 8-byte and scale_dev 4-byte aligned");
+    launch_finish(reinterpret_cast<float2*>(image), p->d_hf, p->desc.grid_n, p->desc.npol,
+                  (float)scale, scale_dev, (cudaStream_t)cuda_stream);
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? GW_OK : cuda_fail(e, "finish launch");
+}
+
 gw_status gw_grid_shift(gw_plan p, void* grid, void* cuda_stream) {
     if (!p) return fail(GW_EINVAL, "null plan");
     gw_status st = check_device(p);

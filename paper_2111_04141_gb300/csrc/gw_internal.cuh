@@ -544,6 +544,10 @@ int static_scratch_max_tiles();
 // ---- correction (gw_correct.cu) -------------------------------------------
 void launch_correct(float2* image, const float* h, int N, int npol, int mode, cudaStream_t s);
 void launch_shift(float2* grid, int N, int npol, cudaStream_t s);
+// image[p][i][j] = image[p][(i + N/2) % N][(j + N/2) % N] (-1)^(i+j) h(m_i) h(l_j)
+// scale scale_dev[p] (scale_dev null: 1), in place.
+void launch_finish(float2* image, const float* h, int N, int npol, float scale,
+                   const float* scale_dev, cudaStream_t s);
 // image[p][i][j] += sum_l layers[l][p][i][j] exp(+j 2 pi w_l (n_ij - 1)),
 // w_l = wmin + l dw, l_j = (j - N/2) cell, m_i = (i - N/2) cell (w-stacking).
 void launch_wstack_combine(const float2* layers, int nlayers, double wmin, double dw, int N,

@@ -22,13 +22,12 @@ def dirty_image(plan, uvw, freq, vis, weight: Optional[torch.Tensor] = None,
                 normalise: bool = True, stream=None) -> torch.Tensor:
     """[npol, N, N] complex64 dirty image (the real part is the image)."""
     g, dropped = plan.grid(uvw, freq, vis, weight=weight, stream=stream, return_dropped=True)
-    plan.shift(g, stream=stream)
     img = torch.fft.ifft2(g, norm="forward")          # sum_k G_k exp(+j 2 pi k x / N)
-    plan.correct(img, direction=+1, stream=stream)
+    scale, scale_dev = 1.0, None
     if normalise:
         nrow, nchan = uvw.shape[0], freq.shape[0]
         if weight is None:
-            wsum = float(nrow * nchan - dropped)
+            scale = 1.0 / max(float(nrow * nchan - dropped), 1e-30)
         else:
             # drops are visibilities whose footprint leaves the grid: their
             # weights are excluded through the index records' valid flags
@@ -36,10 +35,9 @@ def dirty_image(plan, uvw, freq, vis, weight: Optional[torch.Tensor] = None,
             valid = ((raw[:, 3] >> 16) & 1).to(torch.float32)
             w = weight.reshape(nrow * nchan, -1) * valid[:, None]
             ws = w.sum(0).to(torch.float64).clamp_min(1e-30)     # per polarisation
-            img /= ws.to(img.real.dtype)[:, None, None]
-            return img
-        img /= max(wsum, 1e-30)
-    return img
+            scale_dev = (1.0 / ws).to(torch.float32)
+    # origin shift, correction and normalisation in one pass
+    return plan.finish_image(img, scale=scale, scale_dev=scale_dev, stream=stream)
 
 
 def model_vis(plan, uvw, freq, image: torch.Tensor, stream=None) -> torch.Tensor:

@@ -461,6 +461,19 @@ class Plan:
                   "gw_grid_shift")
         return grid
 
+    def finish_image(self, image, scale: float = 1.0, scale_dev=None, stream=None):
+        """Origin shift, correction (+1) and normalisation of the unnormalised
+        inverse FFT of a grid that was not shifted, in one pass (gw_image_finish)."""
+        _need(image, "image", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
+        if scale_dev is not None:
+            _need(scale_dev, "scale_dev", torch.float32, self.device, (self.npol,))
+            if stream is not None:
+                scale_dev.record_stream(stream)
+        with torch.cuda.device(self.device):
+            check(self._lib.gw_image_finish(self._h, _ptr(image), float(scale), _ptr(scale_dev),
+                                            _stream_ptr(stream, self.device)), "gw_image_finish")
+        return image
+
     def index(self, uvw, freq, stream=None):
         """Raw index records as an int32 tensor [nvis, 4] plus the drop count.
 

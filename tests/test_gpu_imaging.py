@@ -105,3 +105,41 @@ def test_dirty_image_and_model_vis_match_oracle(gw):
         mv = model_vis(plan, u, f, dev(model)).cpu().numpy().reshape(ref_v.shape)
     assert rel_l2(img[:, c, c], ref[:, c, c]) <= 2e-5
     assert rel_l2(mv, ref_v) <= 2e-5
+
+
+# finish_image against shift + correct + divide in FP64: sides with whole and
+# odd halves of 16 bytes (pairs of pixels or single ones), an image off 16
+# bytes, host and device scales.  At most six FP32 roundings a
+# pixel (factors, scale and products): 6 x 2^-24.
+@pytest.mark.parametrize("n,npol,shift", [(8, 1, 0), (10, 3, 0), (130, 2, 0), (256, 4, 0),
+                                          (256, 1, 1), (1030, 1, 1)])
+@pytest.mark.parametrize("device_scale", [False, True])
+def test_finish_is_shift_correct_and_scale(gw, n, npol, shift, device_scale):
+    rng = np.random.default_rng(n + npol)
+    z = (rng.standard_normal((npol, n, n)) + 1j * rng.standard_normal((npol, n, n)))
+    z = z.astype(np.complex64)
+    buf = torch.empty(npol * n * n + shift, dtype=torch.complex64, device=DEV)
+    img = buf[shift:].view(npol, n, n)
+    img.copy_(torch.from_numpy(z))
+    scale_dev = dev(rng.uniform(0.5, 2.0, npol).astype(np.float32)) if device_scale else None
+    with gw.Plan(grid_n=n, cell_rad=1e-3, support_min=1, support_max=3, oversample=4,
+                 n_wplanes=1, w_max_lambda=0.0, npol=npol) as plan:
+        ones = plan.correct(torch.ones_like(img), direction=+1).cpu().numpy().astype(complex)
+        out = plan.finish_image(img, scale=0.37, scale_dev=scale_dev).cpu().numpy()
+    # correct(+1) holds the sign; its FP32 factors are taken as given
+    ref = np.roll(z.astype(complex), (n // 2, n // 2), (1, 2)) * ones * np.float32(0.37)
+    if device_scale:
+        ref *= scale_dev.cpu().numpy()[:, None, None].astype(float)
+    assert np.all(np.abs(out - ref) <= 6 * 2.0 ** -24 * np.abs(ref) + 1e-30)
+
+
+def test_dirty_image_without_weight_is_zero(gw):
+    from paper_2111_04141_gb300.imaging import dirty_image
+    obs = syn.config_2d()
+    n = 128
+    with gw.Plan(grid_n=n, cell_rad=syn.fit_cell(obs.uvw_m, obs.freq_hz, n, 7), support_min=7,
+                 support_max=7, oversample=128, n_wplanes=1, w_max_lambda=0.0, npol=1) as plan:
+        v = torch.ones((obs.nrow, obs.nchan, 1), dtype=torch.complex64, device=DEV)
+        w = torch.zeros((obs.nrow, obs.nchan, 1), dtype=torch.float32, device=DEV)
+        img = dirty_image(plan, dev(obs.uvw_m), dev(obs.freq_hz), v, weight=w)
+    assert torch.count_nonzero(torch.view_as_real(img)) == 0
