@@ -239,6 +239,12 @@ gw_status gw_grid_vis(gw_plan plan, const double* uvw_m, const double* freq_hz, 
                       int32_t nchan, const void* vis, const float* weight, void* grid,
                       int64_t* n_dropped, void* cuda_stream);
 
+/* gw_grid_vis onto a fresh grid: the grid (uninitialised memory of the caller)
+ * is cleared on the stream first.  Arguments and errors as gw_grid_vis. */
+gw_status gw_grid_vis_fresh(gw_plan plan, const double* uvw_m, const double* freq_hz, int64_t nrow,
+                            int32_t nchan, const void* vis, const float* weight, void* grid,
+                            int64_t* n_dropped, void* cuda_stream);
+
 /* gw_grid_vis from HOST inputs (no thesis counterpart): uvw_h, freq_h,
  * vis_h and weight_h (optional) are host arrays with the layouts of
  * gw_grid_vis; grid is on the device.  The rows are processed in steps

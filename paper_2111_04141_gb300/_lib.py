@@ -66,6 +66,8 @@ _SIGS = {
     "gw_plan_get_tuning": (c_i32, [c_vp, ctypes.POINTER(Tuning)]),
     "gw_grid_vis": (c_i32, [c_vp, c_vp, c_vp, c_i64, c_i32, c_vp, c_vp, c_vp,
                             ctypes.POINTER(c_i64), c_vp]),
+    "gw_grid_vis_fresh": (c_i32, [c_vp, c_vp, c_vp, c_i64, c_i32, c_vp, c_vp, c_vp,
+                                  ctypes.POINTER(c_i64), c_vp]),
     "gw_grid_vis_compensated": (c_i32, [c_vp, c_vp, c_vp, c_i64, c_i32, c_vp, c_vp, c_vp, c_vp,
                                         ctypes.POINTER(c_i64), c_vp]),
     "gw_grid_fold": (c_i32, [c_vp, c_vp, c_vp, c_vp]),

@@ -912,8 +912,10 @@ static gw_status grid_impl(gw_plan p, const double* uvw_m, const double* freq_hz
     if (grid_err && reinterpret_cast<uintptr_t>(grid_err) % 8 != 0)
         return fail(GW_EINVAL, "grid_err must be 8-byte aligned");
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    cudaError_t e = reset_dropped ? cudaMemsetAsync(p->sc.dropped, 0, sizeof(unsigned long long), s)
-                                  : cudaSuccess;
+    // the drop counter starts at zero for the calls that read it
+    cudaError_t e = reset_dropped && n_dropped
+                        ? cudaMemsetAsync(p->sc.dropped, 0, sizeof(unsigned long long), s)
+                        : cudaSuccess;
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     const int npol = p->desc.npol;
     const int64_t rpc = rows_per_chunk(p, nchan);
@@ -1008,6 +1010,21 @@ static gw_status grid_impl(gw_plan p, const double* uvw_m, const double* freq_hz
 gw_status gw_grid_vis(gw_plan p, const double* uvw_m, const double* freq_hz, int64_t nrow,
                       int32_t nchan, const void* vis, const float* weight, void* grid,
                       int64_t* n_dropped, void* cuda_stream) {
+    return grid_impl(p, uvw_m, freq_hz, nrow, nchan, vis, weight, grid, nullptr, n_dropped,
+                     cuda_stream);
+}
+
+gw_status gw_grid_vis_fresh(gw_plan p, const double* uvw_m, const double* freq_hz, int64_t nrow,
+                            int32_t nchan, const void* vis, const float* weight, void* grid,
+                            int64_t* n_dropped, void* cuda_stream) {
+    gw_status st = common_checks(p, uvw_m, freq_hz, nrow, nchan);
+    if (st != GW_OK) return st;
+    if (!grid) return fail(GW_EINVAL, "null grid");
+    if (reinterpret_cast<uintptr_t>(grid) % 8 != 0)
+        return fail(GW_EINVAL, "grid must be 8-byte aligned");
+    const size_t n = (size_t)p->desc.npol * p->desc.grid_n * p->desc.grid_n;
+    cudaError_t e = cudaMemsetAsync(grid, 0, sizeof(float2) * n, (cudaStream_t)cuda_stream);
+    if (e != cudaSuccess) return cuda_fail(e, "clearing the grid");
     return grid_impl(p, uvw_m, freq_hz, nrow, nchan, vis, weight, grid, nullptr, n_dropped,
                      cuda_stream);
 }
@@ -1555,7 +1572,8 @@ gw_status gw_degrid_vis(gw_plan p, const double* uvw_m, const double* freq_hz, i
     if (!grid) return fail(GW_EINVAL, "null grid");
     if (nrow > 0 && nchan > 0 && !vis_out) return fail(GW_EINVAL, "null vis_out");
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    cudaError_t e = cudaMemsetAsync(p->sc.dropped, 0, sizeof(unsigned long long), s);
+    cudaError_t e = n_dropped ? cudaMemsetAsync(p->sc.dropped, 0, sizeof(unsigned long long), s)
+                              : cudaSuccess;
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     const int npol = p->desc.npol;
     const size_t vb = dtype_bytes(p->desc.vis_dtype);

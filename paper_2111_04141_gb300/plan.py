@@ -6,6 +6,7 @@ in the library's CUDA kernels.  PyTorch supplies device memory and streams.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 from typing import Optional
 
@@ -41,12 +42,20 @@ def from_storage(vis: torch.Tensor) -> torch.Tensor:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _stream_ptr(stream, device):
-    s = torch.cuda.current_stream(device) if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    # (the raw handle: torch.cuda.current_stream builds a Stream object)
+    return torch._C._cuda_getCurrentRawStream(device.index) if stream is None else stream.cuda_stream
+
+
+_HERE = contextlib.nullcontext()
+
+
+def _on(device):
+    """Context in which ``device`` is current (none needed where it is)."""
+    return _HERE if torch.cuda.current_device() == device.index else torch.cuda.device(device)
 
 
 def _need(t: torch.Tensor, name: str, dtype, device, shape=None):
@@ -192,17 +201,21 @@ class Plan:
         vis = self._vis_arg(vis, "vis", nrow, nchan)
         if weight is not None:
             _need(weight, "weight", torch.float32, self.device, (nrow, nchan, self.npol))
-        if out is None:
-            out = self.new_grid()
         gshape = (self.npol, self.grid_n, self.grid_n)
-        _need(out, "grid", torch.complex64, self.device, gshape)
+        fresh = out is None and err is None      # cleared by the library, on the stream
+        if fresh:
+            out = torch.empty(gshape, dtype=torch.complex64, device=self.device)
+        else:
+            if out is None:
+                out = self.new_grid()
+            _need(out, "grid", torch.complex64, self.device, gshape)
         dropped = ctypes.c_int64(-1)
         dp = ctypes.byref(dropped) if return_dropped else None
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             if err is None:
-                check(self._lib.gw_grid_vis(self._h, _ptr(uvw), _ptr(freq), nrow, nchan,
-                                            _ptr(vis), _ptr(weight), _ptr(out), dp,
-                                            _stream_ptr(stream, self.device)), "gw_grid_vis")
+                call = self._lib.gw_grid_vis_fresh if fresh else self._lib.gw_grid_vis
+                check(call(self._h, _ptr(uvw), _ptr(freq), nrow, nchan, _ptr(vis), _ptr(weight),
+                           _ptr(out), dp, _stream_ptr(stream, self.device)), "gw_grid_vis")
             else:
                 _need(err, "err", torch.complex64, self.device, gshape)
                 check(self._lib.gw_grid_vis_compensated(
@@ -271,7 +284,7 @@ class Plan:
             out = self.new_grid()
         _need(out, "grid", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
         ng, nd = ctypes.c_int64(-1), ctypes.c_int64(-1)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_grid_vis_compressed(self._h, _ptr(uvw), _ptr(freq), nrow, nchan,
                                                    _ptr(vis), _ptr(weight), _ptr(out),
                                                    ctypes.byref(ng), ctypes.byref(nd),
@@ -291,7 +304,7 @@ class Plan:
             out = torch.zeros(shape, dtype=torch.complex64, device=self.device)
         _need(out, "layers", torch.complex64, self.device, shape)
         nd = ctypes.c_int64(-1)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_grid_vis_wstack(self._h, _ptr(uvw), _ptr(freq), nrow, nchan,
                                                _ptr(vis), _ptr(weight), int(n_layers),
                                                float(w_min), float(w_max), _ptr(out),
@@ -306,7 +319,7 @@ class Plan:
         _need(layer_images, "layer_images", torch.complex64, self.device,
               (L, self.npol, self.grid_n, self.grid_n))
         _need(image, "image", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_wstack_combine(self._h, _ptr(layer_images), L, float(w_min),
                                               float(w_max), _ptr(image),
                                               _stream_ptr(stream, self.device)),
@@ -326,7 +339,7 @@ class Plan:
             out = torch.zeros(shape, dtype=torch.complex64, device=self.device)
         _need(out, "fine", torch.complex64, self.device, shape)
         nd = ctypes.c_int64(-1)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_hybrid_grid(self._h, _ptr(uvw), _ptr(freq), nrow, nchan, _ptr(vis),
                                            _ptr(weight), int(sz), _ptr(out),
                                            ctypes.byref(nd) if return_dropped else None,
@@ -343,7 +356,7 @@ class Plan:
         if out is None:
             out = torch.empty(shape, dtype=torch.complex64, device=self.device)
         _need(out, "pruned", torch.complex64, self.device, shape)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_hybrid_prune(self._h, int(sz), _ptr(fine), _ptr(out),
                                             _stream_ptr(stream, self.device)), "gw_hybrid_prune")
         return out
@@ -351,7 +364,7 @@ class Plan:
     def hybrid_shift(self, pruned, stream=None):
         _need(pruned, "pruned", torch.complex64, self.device,
               (self.npol, 2 * self.grid_n, self.grid_n))
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_hybrid_shift(self._h, _ptr(pruned), _stream_ptr(stream, self.device)),
                   "gw_hybrid_shift")
         return pruned
@@ -361,7 +374,7 @@ class Plan:
         if out is None:
             out = self.new_grid()
         _need(out, "image", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_hybrid_image(self._h, int(sz), _ptr(raw), _ptr(out),
                                             _stream_ptr(stream, self.device)), "gw_hybrid_image")
         return out
@@ -392,7 +405,7 @@ class Plan:
             out = self.new_grid()
         _need(out, "grid", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
         nd = ctypes.c_int64(-1)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_grid_vis_host(self._h, _ptr(uvw), _ptr(freq), nrow, nchan,
                                              _ptr(vt), _ptr(weight), _ptr(out),
                                              ctypes.byref(nd) if return_dropped else None,
@@ -405,7 +418,7 @@ class Plan:
         gshape = (self.npol, self.grid_n, self.grid_n)
         _need(grid, "grid", torch.complex64, self.device, gshape)
         _need(err, "err", torch.complex64, self.device, gshape)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_grid_fold(self._h, _ptr(grid), _ptr(err),
                                          _stream_ptr(stream, self.device)), "gw_grid_fold")
         return grid
@@ -418,7 +431,7 @@ class Plan:
             out = self.new_vis(nrow, nchan)
         out = self._vis_arg(out, "vis_out", nrow, nchan)
         dropped = ctypes.c_int64(-1)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_degrid_vis(self._h, _ptr(uvw), _ptr(freq), nrow, nchan, _ptr(grid),
                                           _ptr(out),
                                           ctypes.byref(dropped) if return_dropped else None,
@@ -439,7 +452,7 @@ class Plan:
             out = self.new_vis(nrow, nchan)
         out = self._vis_arg(out, "vis_out", nrow, nchan)
         dropped = ctypes.c_int64(-1)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_degrid_vis_static(self._h, _ptr(uvw), _ptr(freq), nrow, nchan,
                                                  _ptr(grid), _ptr(out),
                                                  ctypes.byref(dropped) if return_dropped else None,
@@ -449,14 +462,14 @@ class Plan:
 
     def correct(self, image, direction: int = 1, stream=None):
         _need(image, "image", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_grid_correct(self._h, _ptr(image), int(direction),
                                             _stream_ptr(stream, self.device)), "gw_grid_correct")
         return image
 
     def shift(self, grid, stream=None):
         _need(grid, "grid", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_grid_shift(self._h, _ptr(grid), _stream_ptr(stream, self.device)),
                   "gw_grid_shift")
         return grid
@@ -469,7 +482,7 @@ class Plan:
             _need(scale_dev, "scale_dev", torch.float32, self.device, (self.npol,))
             if stream is not None:
                 scale_dev.record_stream(stream)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_image_finish(self._h, _ptr(image), float(scale), _ptr(scale_dev),
                                             _stream_ptr(stream, self.device)), "gw_image_finish")
         return image
@@ -482,7 +495,7 @@ class Plan:
         nrow, nchan = self._coords(uvw, freq)
         out = torch.empty((nrow * nchan, 4), dtype=torch.int32, device=self.device)
         dropped = ctypes.c_int64(-1)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_index_vis(self._h, _ptr(uvw), _ptr(freq), nrow, nchan, _ptr(out),
                                          ctypes.byref(dropped), _stream_ptr(stream, self.device)),
                   "gw_index_vis")
@@ -502,7 +515,7 @@ class Plan:
         buf = np.empty(2 * self.info.table_elems, dtype=np.float32)
         offs = np.empty(P + 1, dtype=np.int64)
         sup = np.empty(P, dtype=np.int32)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_plan_copy_tables(self._h, buf.ctypes.data_as(ctypes.c_void_p),
                                                 offs.ctypes.data_as(ctypes.c_void_p),
                                                 sup.ctypes.data_as(ctypes.c_void_p)),
@@ -517,14 +530,14 @@ class Plan:
             buf = np.empty(n, dtype=np.complex64)
         else:
             buf = np.empty((n, 2), dtype=np.uint16)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_plan_copy_stored_tables(self._h, buf.ctypes.data_as(ctypes.c_void_p)),
                   "gw_plan_copy_stored_tables")
         return buf
 
     def corrector(self):
         h = np.empty(self.grid_n, dtype=np.float64)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_plan_copy_corrector(self._h, h.ctypes.data_as(ctypes.c_void_p)),
                   "gw_plan_copy_corrector")
         return h
@@ -532,7 +545,7 @@ class Plan:
     def device_status(self, stream=None):
         """Synchronise the stream and raise GwError (GW_ETIMEDOUT) if a
         bounded device-side wait gave up since the last check."""
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_plan_device_status(self._h, _stream_ptr(stream, self.device)),
                   "gw_plan_device_status")
 
@@ -544,7 +557,7 @@ class Plan:
                   "gw_plan_timing_enable")
             return None
         t = _lib.Timing()
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_plan_timing_get(self._h, ctypes.byref(t)), "gw_plan_timing_get")
         return {name: getattr(t, name) for name, _ in t._fields_}
 
@@ -558,7 +571,7 @@ class Plan:
         offs = np.empty(ntiles + 1, dtype=np.int64)
         cap = capacity if capacity is not None else max(1, nrow * nchan * 16)
         ent = np.empty(cap, dtype=np.uint32)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             check(self._lib.gw_debug_bins(self._h, _ptr(uvw), _ptr(freq), nrow, nchan, int(mode),
                                           offs.ctypes.data_as(ctypes.c_void_p),
                                           ent.ctypes.data_as(ctypes.c_void_p), cap,
