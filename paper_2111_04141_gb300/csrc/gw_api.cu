@@ -145,7 +145,7 @@ struct gw_plan_s {
     // w-stacking bins over layers x tiles (allocated on first use, grown on demand)
     int ws_layers = 0;
     uint32_t *ws_count = nullptr, *ws_offsets = nullptr, *ws_cursor = nullptr,
-             *ws_item_off = nullptr;
+             *ws_item_off = nullptr, *ws_scan_tmp = nullptr;
     Item* ws_items = nullptr;
     int64_t ws_items_cap = 0;
     // hybrid gridding: the 1-D w = 0 kernel (kept from the table build) and
@@ -231,6 +231,7 @@ void plan_free(gw_plan p) {
     dev_free(p->ws_offsets);
     dev_free(p->ws_cursor);
     dev_free(p->ws_item_off);
+    dev_free(p->ws_scan_tmp);
     dev_free(p->ws_items);
     for (int b = 0; b < 2; ++b) {
         dev_free(p->h_uvw[b]);
@@ -1291,8 +1292,9 @@ static gw_status ensure_wstack(gw_plan p, int nlayers) {
     dev_free(p->ws_offsets);
     dev_free(p->ws_cursor);
     dev_free(p->ws_item_off);
+    dev_free(p->ws_scan_tmp);
     dev_free(p->ws_items);
-    p->ws_count = p->ws_offsets = p->ws_cursor = p->ws_item_off = nullptr;
+    p->ws_count = p->ws_offsets = p->ws_cursor = p->ws_item_off = p->ws_scan_tmp = nullptr;
     p->ws_items = nullptr;
     p->ws_layers = 0;
     const int64_t nt = (int64_t)nlayers * p->geom_grid.ntu * p->geom_grid.ntv;
@@ -1302,14 +1304,16 @@ static gw_status ensure_wstack(gw_plan p, int nlayers) {
     if (e == cudaSuccess) e = dmalloc(&p->ws_offsets, (size_t)nt + 1);
     if (e == cudaSuccess) e = dmalloc(&p->ws_cursor, (size_t)nt);
     if (e == cudaSuccess) e = dmalloc(&p->ws_item_off, (size_t)nt + 1);
+    if (e == cudaSuccess) e = dmalloc(&p->ws_scan_tmp, (size_t)scan_tmp_words(nt));
     if (e == cudaSuccess) e = dmalloc(&p->ws_items, (size_t)icap);
     if (e != cudaSuccess) {
         dev_free(p->ws_count);
         dev_free(p->ws_offsets);
         dev_free(p->ws_cursor);
         dev_free(p->ws_item_off);
+        dev_free(p->ws_scan_tmp);
         dev_free(p->ws_items);
-        p->ws_count = p->ws_offsets = p->ws_cursor = p->ws_item_off = nullptr;
+        p->ws_count = p->ws_offsets = p->ws_cursor = p->ws_item_off = p->ws_scan_tmp = nullptr;
         p->ws_items = nullptr;
         return fail(GW_ENOMEM, "allocating w-stacking bins");
     }
@@ -1354,6 +1358,8 @@ gw_status gw_grid_vis_wstack(gw_plan p, const double* uvw_m, const double* freq_
     sc.offsets = p->ws_offsets;
     sc.cursor = p->ws_cursor;
     sc.item_off = p->ws_item_off;
+    sc.scan_tmp = p->ws_scan_tmp;
+    sc.scan_tmp_bins = (int64_t)n_layers * g.layer_tiles;
     sc.items = p->ws_items;
     sc.items_cap = p->ws_items_cap;
     const int npol = p->desc.npol;

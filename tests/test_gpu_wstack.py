@@ -97,3 +97,20 @@ def test_wstacked_image_matches_direct_sum_for_layer_exact_records(gw, w_max, L)
     c = slice(N // 4, 3 * N // 4)
     err = np.max(np.abs(img[:, c, c] - ref[:, c, c])) / np.max(np.abs(ref[:, c, c]))
     assert err <= 2e-5
+
+
+# bins beyond the single-kernel scan (262,144: 2,100 layers of 128 tiles) and
+# just below it, most of them empty
+@pytest.mark.parametrize("n_layers", [2040, 2100])
+def test_many_layers_match_plain_gridding(gw, n_layers):
+    obs = syn.small_case(n_ant=7, n_times=10, n_chan=3, npol=1, grid_n=512, s_min=5, s_max=5,
+                         n_w=1, diameter_m=1500.0)
+    wext = float(np.max(np.abs(obs.uvw_m[:, 2])) * obs.freq_hz.max() / C0)
+    u, f, v = dev(obs.uvw_m), dev(obs.freq_hz), dev(obs.vis)
+    with gw.Plan.from_observation(obs) as plan:
+        got = plan.grid_wstack(u, f, v, n_layers, -wext, wext)
+        ref = plan.grid(u, f, v)             # the layers share the one kernel
+        filled = int((got.abs().amax((1, 2, 3)) > 0).sum())
+    assert filled > 50
+    d = got.sum(0) - ref
+    assert torch.linalg.vector_norm(d) <= 1e-5 * torch.linalg.vector_norm(ref)
