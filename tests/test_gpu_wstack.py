@@ -99,6 +99,30 @@ def test_wstacked_image_matches_direct_sum_for_layer_exact_records(gw, w_max, L)
     assert err <= 2e-5
 
 
+# phases in fixed point (w below 2^18 wavelengths) and in FP64, a field past the
+# horizon, one layer and a recursion over two anchors.  A screen is at most 7
+# FP32 rotations from its anchor, each within 2^-22: 8 x 2^-22 with the sum.
+@pytest.mark.parametrize("w_max,L,field", [(262143.0, 9, 0.3), (262145.0, 9, 0.3), (150.0, 1, 0.5),
+                                           (5000.0, 17, 1.6), (3e5, 3, 1.6)])
+def test_combine_matches_fp64_screens(gw, w_max, L, field):
+    N, npol = 62, 2
+    rng = np.random.default_rng(L)
+    z = rng.normal(size=(L, npol, N, N)) + 1j * rng.normal(size=(L, npol, N, N))
+    z = z.astype(np.complex64)
+    x = (np.arange(N) - N // 2) * (field / N)
+    r2 = np.minimum(x[:, None] ** 2 + x[None, :] ** 2, 1.0)
+    nm1 = np.where(r2 < 1.0, -r2 / (1.0 + np.sqrt(1.0 - r2)), 0.0)
+    w_min = -0.75 * w_max
+    w = np.linspace(w_min, w_max, L) if L > 1 else np.array([w_min])
+    ref = 1.0 + sum(np.roll(z[k].astype(complex), (N // 2, N // 2), (1, 2)) *
+                    np.exp(2j * np.pi * w[k] * nm1) for k in range(L))
+    with gw.Plan(grid_n=N, cell_rad=field / N, support_min=5, support_max=5, oversample=4,
+                 n_wplanes=1, w_max_lambda=0.0, npol=npol) as plan:
+        img = torch.ones((npol, N, N), dtype=torch.complex64, device=DEV)
+        plan.wstack_combine(dev(z), w_min, w_max, img)
+    assert rel_l2(img.cpu().numpy().astype(complex), ref) <= 8 * 2.0 ** -22
+
+
 # bins beyond the single-kernel scan (262,144: 2,100 layers of 128 tiles) and
 # just below it, most of them empty
 @pytest.mark.parametrize("n_layers", [2040, 2100])
