@@ -869,12 +869,17 @@ gw_status gw_plan_info_get(gw_plan p, gw_plan_info* out) {
 //   63 (1.04 M x 4, 2048^2, support 7-127): 16 / 64 4.53 / 4.03 ms
 //   126 (8.3 M x 4, 4096^2, support 7-63): 16 / 32 / 64 9.52 / 9.89 / 10.7 ms
 // Where the region of 16-point tiles does not fit and is served in bands, 32
-// points are taken at any density.
+// points are taken at any density.  A size needs kStagedMinTiles of its tiles,
+// so that every SM gets several (62 k x 4, 1000^2: 16 / 32 points 70 / 85 us;
+// 12 k x 1, 1656^2: 16 / 32 / 64 84 / 45 / 46 us).
 static const BinGeom& staged_geom(gw_plan p, int64_t nvis) {
     const double n = (double)p->desc.grid_n, per = (double)nvis * 256.0;
-    if (per < kStagedSparse64 * n * n) return p->geom_staged64;
-    return per < kStagedSparse32 * n * n || staged_banded(p->hmax, p->desc.npol) ? p->geom_degrid
-                                                                               : p->geom_staged;
+    auto enough = [](const BinGeom& g) { return g.ntu * g.ntv >= kStagedMinTiles; };
+    if (per < kStagedSparse64 * n * n && enough(p->geom_staged64)) return p->geom_staged64;
+    if (staged_banded(p->hmax, p->desc.npol) ||
+        (per < kStagedSparse32 * n * n && enough(p->geom_degrid)))
+        return p->geom_degrid;
+    return p->geom_staged;
 }
 
 // Inputs small enough that launches dominate: gridded and degridded directly.

@@ -397,6 +397,7 @@ constexpr int64_t kDirectMaxTaps = (int64_t)1 << 22;
 // below this many visibilities per 16 x 16 points on average.
 constexpr double kStagedSparse32 = 48.0;
 constexpr double kStagedSparse64 = 6.0;
+constexpr int kStagedMinTiles = 2048;
 // One instantiation set per table kind (gw_grid_c64.cu, gw_grid_bf16.cu, gw_grid_f16.cu,
 // gw_grid_r32.cu).
 void launch_grid_c64(const GridArgs& a, int num_sms, cudaStream_t s);
