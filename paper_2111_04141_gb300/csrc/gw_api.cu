@@ -400,6 +400,31 @@ gw_status index_and_bin(gw_plan p, const double* uvw, const double* freq, int64_
     return GW_OK;
 }
 
+// Table elements before plane q, without the padding between slices.
+int64_t packed_offset(gw_plan p, int q) {
+    int64_t n = 0;
+    for (int i = 0; i < q; ++i)
+        n += (int64_t)p->desc.oversample * p->desc.oversample * p->support[i] * p->support[i];
+    return n;
+}
+
+// Copies a table of `bytes` an element to the host, slices packed.
+cudaError_t copy_packed(gw_plan p, void* out, const void* table, size_t bytes) {
+    char* dst = static_cast<char*>(out);
+    const size_t slices = (size_t)p->desc.oversample * p->desc.oversample;
+    for (size_t q = 0; q < p->support.size(); ++q) {
+        const int S = p->support[q];
+        const size_t row = (size_t)S * S * bytes;
+        cudaError_t e = cudaMemcpy2D(dst, row,
+                                     static_cast<const char*>(table) + p->plane_off[q] * bytes,
+                                     (size_t)slice_elems(S) * bytes, row, slices,
+                                     cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return e;
+        dst += row * slices;
+    }
+    return cudaSuccess;
+}
+
 int64_t rows_per_chunk(gw_plan p, int nchan) {
     int64_t r = p->chunk / (nchan > 0 ? nchan : 1);
     return r < 1 ? 1 : r;
@@ -506,7 +531,7 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     for (int q = 0; q < P; ++q) {
         const double r = P > 1 ? (double)q / (double)(P - 1) : 0.0;
         p->wplane[q] = P > 1 ? desc->w_max_lambda * (r * r) : 0.0;
-        p->plane_off[q + 1] = p->plane_off[q] + (int64_t)beta * beta * p->support[q] * p->support[q];
+        p->plane_off[q + 1] = p->plane_off[q] + (int64_t)beta * beta * slice_elems(p->support[q]);
         p->pplane_off[q + 1] = p->pplane_off[q] + padded_table_elems(p->support[q], beta, p->pad_stride);
     }
     if (p->pplane_off[P] >= (int64_t)1 << 31) {
@@ -847,7 +872,7 @@ gw_status gw_plan_info_get(gw_plan p, gw_plan_info* out) {
     out->grid_tile_v = kGridTileV;
     out->degrid_tile = kTile;
     out->device = p->device;
-    out->table_elems = p->plane_off.back();
+    out->table_elems = packed_offset(p, p->desc.n_wplanes);
     out->chunk_vis = p->chunk;
     out->field = p->field;
     out->taper_c = M_PI * p->desc.support_min / 2.0;
@@ -1968,11 +1993,10 @@ gw_status gw_plan_copy_tables(gw_plan p, float* out, int64_t* plane_offsets, int
     if (!p || !out) return fail(GW_EINVAL, "null argument");
     gw_status st = check_device(p);
     if (st != GW_OK) return st;
-    cudaError_t e = cudaMemcpy(out, p->table, sizeof(float2) * p->plane_off.back(),
-                               cudaMemcpyDeviceToHost);
+    cudaError_t e = copy_packed(p, out, p->table, sizeof(float2));
     if (e != cudaSuccess) return cuda_fail(e, "copying tables");
     if (plane_offsets)
-        for (size_t i = 0; i < p->plane_off.size(); ++i) plane_offsets[i] = p->plane_off[i];
+        for (size_t i = 0; i < p->plane_off.size(); ++i) plane_offsets[i] = packed_offset(p, (int)i);
     if (supports)
         for (size_t i = 0; i < p->support.size(); ++i) supports[i] = p->support[i];
     return GW_OK;
@@ -1983,8 +2007,7 @@ gw_status gw_plan_copy_stored_tables(gw_plan p, void* out) {
     gw_status st = check_device(p);
     if (st != GW_OK) return st;
     const void* src = p->table16 ? (const void*)p->table16 : (const void*)p->table;
-    cudaError_t e = cudaMemcpy(out, src, (size_t)dtype_bytes(p->desc.table_dtype) * p->plane_off.back(),
-                               cudaMemcpyDeviceToHost);
+    cudaError_t e = copy_packed(p, out, src, dtype_bytes(p->desc.table_dtype));
     return e == cudaSuccess ? GW_OK : cuda_fail(e, "copying stored tables");
 }
 

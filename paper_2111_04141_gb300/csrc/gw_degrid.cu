@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kThreads) k_degrid(DegridArgs a) {
         const int S = __ldg(a.support + r.plane), h = S >> 1;
         const typename TE::T* K = reinterpret_cast<const typename TE::T*>(a.table) +
                                   __ldg(a.plane_off + r.plane) +
-                                  ((int64_t)(r.ov + hb) * a.beta + (r.ou + hb)) * S * S;
+                                  ((int64_t)(r.ov + hb) * a.beta + (r.ou + hb)) * slice_elems(S);
         // conj(K_i): K_i = K for w >= 0 (use conj K), K_i = conj K for w < 0 (use K)
         const float s = (r.flags & GW_FLAG_CONJ) ? -1.f : 1.f;
         float acc[NPOL][2];
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(kThreads) k_degrid_direct(DegridArgs a, Direct
         bool valid = (rc.flags & GW_FLAG_VALID) != 0;
         const int S = valid ? __ldg(a.support + rc.plane) : 0, h = S >> 1;
         const int64_t kofs = valid ? __ldg(a.plane_off + rc.plane) +
-                                         ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * S * S : 0;
+                                         ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * slice_elems(S) : 0;
         if (lane == 0) {
             n_valid += valid;
             n_drop += !valid;
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                     const gw_index_rec rc = rcs[k];
                     const int S = __ldg(a.support + rc.plane), h = S >> 1;
                     const int64_t kofs = __ldg(a.plane_off + rc.plane) +
-                                         ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * S * S;
+                                         ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * slice_elems(S);
                     uint32_t rel = (uint32_t)(rc.ku - tx0) | (uint32_t)(rc.kv - ty0) << 8;
                     uint32_t w = (uint32_t)S | ((rc.flags & GW_FLAG_CONJ) ? 1u << 16 : 0u);
 #ifdef GW_DEBUG_BOUNDS

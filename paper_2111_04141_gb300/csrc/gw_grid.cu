@@ -25,7 +25,7 @@ __global__ void k_pad_tables(const T* __restrict__ tab, const int64_t* __restric
         const int row = rem / SP - kGridPadR, col = rem % SP - kGridPadC;
         T v{};
         if (row >= 0 && row < S && col >= 0 && col < S)
-            v = tab[plane_off[p] + o * S * S + (int64_t)row * S + col];
+            v = tab[plane_off[p] + o * slice_elems(S) + (int64_t)row * S + col];
         ptab[pplane_off[p] + e] = v;
     }
 }
@@ -47,7 +47,7 @@ __global__ void k_pad_tables_real(const float2* __restrict__ tab, const int64_t*
         const int row = rem / SP - kGridPadR, col = rem % SP - kGridPadC;
         float v = 0.f;
         if (row >= 0 && row < S && col >= 0 && col < S)
-            v = tab[plane_off[p] + o * S * S + (int64_t)row * S + col].x;
+            v = tab[plane_off[p] + o * slice_elems(S) + (int64_t)row * S + col].x;
         ptab[pplane_off[p] + e] = v;
     }
 }
@@ -69,7 +69,7 @@ __global__ void k_pair_tables(const T* __restrict__ tab, const int64_t* __restri
         const int64_t oc = e / per;                     // 2 x slice + copy
         const int rem = (int)(e - oc * per);
         const int row = rem / W, col = rem - row * W - (int)(oc & 1);
-        dst[e] = col >= 0 && col < S ? src[(oc >> 1) * S * S + (int64_t)row * S + col] : T{};
+        dst[e] = col >= 0 && col < S ? src[(oc >> 1) * slice_elems(S) + (int64_t)row * S + col] : T{};
     }
 }
 
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256) k_grid_direct(GridArgs a, const void* __r
             n_taps += (unsigned long long)(S * S);
         }
         const int64_t kofs = __ldg(a.plane_off + plane) +
-                             ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * S * S;
+                             ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * slice_elems(S);
 #ifdef GW_DEBUG_BOUNDS
         // the slice and the footprint's pixels
         if (!gw_in_bounds((a.table_elems == 0 || (kofs >= 0 && kofs + (int64_t)S * S <= a.table_elems)) &&

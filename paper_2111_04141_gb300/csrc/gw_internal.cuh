@@ -485,6 +485,14 @@ __device__ __forceinline__ bool gw_in_bounds(bool ok, uint32_t* status) {
 __device__ __forceinline__ constexpr bool gw_in_bounds(bool, uint32_t*) { return true; }
 #endif
 
+// Elements from one S x S kernel slice of the unpadded tables to the next:
+// slices start on lines of 128 bytes (32 elements are one line of a 16-bit
+// table, two of an FP32 one), so a warp that reads 32 consecutive kernel
+// values touches the fewest lines (staged degridding, slices S * S elements
+// apart / aligned: 4.2 M visibilities x 1, support 31, 3.06 / 3.00 ms, 8.26 M x 4,
+// supports 7 to 63, 9.34 / 9.21).  Padding elements are zero.
+__host__ __device__ constexpr int slice_elems(int S) { return (S * S + 31) & ~31; }
+
 // Zeroed elements after the last kernel slice of the unpadded tables: the
 // staged degridder loads kernel values up to this many elements past a slice.
 constexpr int64_t kTableSlack = 256;

@@ -294,21 +294,27 @@ __global__ void k_scale(const double2* __restrict__ Kf0, int F, int fmin, int be
     }
 }
 
-// table[((ov' * beta + ou') * S + tv') * S + tu'] = scale * Kf[beta tv - ov - fmin][beta tu - ou - fmin]
+// table[(ov' * beta + ou') * slice_elems(S) + tv' * S + tu'] = scale * Kf[beta tv - ov - fmin][beta tu - ou - fmin]
 // Scaled FP64 entries -> FP32 table and, optionally, a 16-bit table holding
 // round(entry * 2^exp2) (one rounding from FP64, to nearest even).
+// The elements between the slices are zero.
 __global__ void k_slices(const double2* __restrict__ Kf, int F, int fmin, int beta, int S,
                          const double* __restrict__ scale, float2* __restrict__ tab,
                          uint32_t* __restrict__ tab16, int kind16, int exp2) {
-    const int64_t n = (int64_t)beta * beta * S * S;
+    const int L = slice_elems(S), h = S / 2;
+    const int64_t n = (int64_t)beta * beta * L;
     const double sc = *scale;
-    const int h = S / 2;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int tu = (int)(e % S) - h;
-        const int tv = (int)((e / S) % S) - h;
-        const int ou = (int)((e / ((int64_t)S * S)) % beta) - beta / 2;
-        const int ov = (int)(e / ((int64_t)S * S * beta)) - beta / 2;
+        const int64_t o = e / L;
+        const int t = (int)(e - o * L);
+        if (t >= S * S) {
+            tab[e] = make_float2(0.f, 0.f);
+            if (tab16) tab16[e] = 0u;
+            continue;
+        }
+        const int tu = t % S - h, tv = t / S - h;
+        const int ou = (int)(o % beta) - beta / 2, ov = (int)(o / beta) - beta / 2;
         const double2 k = Kf[(int64_t)(beta * tv - ov - fmin) * F + (beta * tu - ou - fmin)];
         const double re = sc * k.x, im = sc * k.y;
         tab[e] = make_float2((float)re, (float)im);
@@ -435,7 +441,7 @@ cudaError_t build_tables(const TableBuild& tb, float2* d_table, uint32_t* d_tabl
                     exp2 = 15 - e2;
                 }
             } else {
-                const int64_t n = (int64_t)beta * beta * S * S;
+                const int64_t n = (int64_t)beta * beta * slice_elems(S);
                 int blocks = (int)std::min<int64_t>((n + 255) / 256, 4096);
                 k_slices<<<blocks, 256, 0, s>>>(Kf, F, fmin, beta, S, scale, d_table + tb.plane_off[p],
                                                 d_table16 ? d_table16 + tb.plane_off[p] : nullptr,
