@@ -269,6 +269,15 @@ constexpr int kLoaderThreads = 128;                       // warps 0-3
 constexpr int kMetaPerLoader = kStagedMeta / kLoaderThreads;
 constexpr int kLoaderBatch = 4;                           // records whose loads a loader issues together
 
+// Last word of a record's metadata: its support (bits 0-8), the conjugation
+// (bit 9) and ceil(2^20 / S) (bits 10-30), with which a lane divides numbers up
+// to 32 by S in one multiplication: their product is at most 32 above the
+// multiple of 2^20 / S that it stands for, S <= 255.
+constexpr uint32_t kMetaSupport = 0x1ffu, kMetaConj = 0x200u;
+__device__ __forceinline__ uint32_t meta_support(int S) {
+    return (uint32_t)S | (uint32_t)((1 << 20) + S - 1) / (uint32_t)S << 10;
+}
+
 __device__ __forceinline__ void loader_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(kLoaderThreads) : "memory");
 }
@@ -300,6 +309,8 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
     const int N = a.N, hb = a.beta / 2;
     const uint32_t nitems = *a.item_count;
     const TT* __restrict__ tab = reinterpret_cast<const TT*>(a.table);
+    constexpr int kElem = NPR ? 16 : 8;       // bytes of an element of the first plane
+    const char* const regc = reinterpret_cast<const char*>(reg);
     // thread 0: the item being served and the next chunk's first record
     Item cur{};
     int next_c0 = 0;
@@ -366,7 +377,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                     const int64_t kofs = __ldg(a.plane_off + rc.plane) +
                                          ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * slice_elems(S);
                     uint32_t rel = (uint32_t)(rc.ku - tx0) | (uint32_t)(rc.kv - ty0) << 8;
-                    uint32_t w = (uint32_t)S | ((rc.flags & GW_FLAG_CONJ) ? 1u << 16 : 0u);
+                    uint32_t w = meta_support(S) | ((rc.flags & GW_FLAG_CONJ) ? kMetaConj : 0u);
 #ifdef GW_DEBUG_BOUNDS
                     // the record's slice, centre tile, region and output row: a
                     // record that fails is replaced by a 1 x 1 one at the
@@ -378,14 +389,14 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                         (a.vis_count == 0 || ids[k] < (uint64_t)a.vis_count);
                     if (!gw_in_bounds(ok, a.queue + 1)) {
                         rel = 8u | 8u << 8;
-                        w = 1u;
+                        w = meta_support(1);
                     }
 #endif
                     const int pos =
                         h > hmax / 2 ? atomicAdd(&c.front, 1) : atomicSub(&c.back, 1) - 1;
 #ifdef GW_DEBUG_BOUNDS
                     if (!gw_in_bounds(pos >= 0 && pos < nc, a.queue + 1)) continue;
-                    if ((w & 0xffffu) == 1u && S != 1) {
+                    if ((w & kMetaSupport) == 1u && S != 1) {
                         meta[pos] = make_uint4(0u, 0u, rel, w);
                         continue;
                     }
@@ -497,8 +508,9 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                 if (r >= nc) break;
                 const uint4 m = meta[r];
                 const uint32_t id = m.x;
-                const int S = (int)(m.w & 0xffffu);
-                const float sg = (m.w >> 16) ? -1.f : 1.f;
+                const int S = (int)(m.w & kMetaSupport);
+                const uint32_t inv = m.w >> 10;
+                const float sg = m.w & kMetaConj ? -1.f : 1.f;
                 // region row and column of tap (0, 0): centre - h + hi; the tap rows
                 // [tv0, tv1) lie in this band
                 const int ry = (int)(m.z >> 8) - (S >> 1) + hi, rx = (int)(m.z & 0xffu) - (S >> 1) + hi;
@@ -507,33 +519,47 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                 if (GEN && tv1 <= tv0) continue;
                 const TT* K = tab + m.y + tv0 * S;
                 const int n = (tv1 - tv0) * S;
-                // flattened taps t = lane + 32 i; the region index advances by
-                // `step` per 32 taps, plus `wrap` when the tap column wraps
-                const int dq = 32 / S, dr = 32 - dq * S;
-                const int step = dq * RSP + dr, wrap = RSP - S;
-                int tu = lane % S;
+                // flattened taps t = lane + 32 i; the region offset (in bytes of a
+                // plane) advances by `step` per 32 taps, plus `wrap` when the tap
+                // column wraps
+                const int dq = (int)(32u * inv >> 20), dr = 32 - dq * S;
+                const int lq = (int)((uint32_t)lane * inv >> 20);
+                const int step = (dq * RSP + dr) * kElem, wrap = (RSP - S) * kElem;
+                int tu = lane - lq * S;
                 const int base = (ry + tv0 - yb) * RSP + rx;
-                int off = base + (lane / S) * RSP + tu;
+                int off = (base + lq * RSP + tu) * kElem;
                 // a1 = sum K.re G, a2 = sum K.im G (packed FP32x2 FMAs); the
                 // conjugation sign is applied once at the end
                 float2 a1[NPOL], a2[NPOL];
 #pragma unroll
                 for (int p = 0; p < NPOL; ++p) a1[p] = a2[p] = make_float2(0.f, 0.f);
                 auto tap = [&](const float2 k, const int o) {
-                    const float2 kxx = make_float2(k.x, k.x), kyy = make_float2(k.y, k.y);
+                    if constexpr (NPOL == 1) {
+                        // one use of each: packing K.re and K.im twice would cost
+                        // more than the packed FMAs save
+                        const float2 g = *reinterpret_cast<const float2*>(regc + o);
+                        a1[0].x = fmaf(k.x, g.x, a1[0].x);
+                        a1[0].y = fmaf(k.x, g.y, a1[0].y);
+                        a2[0].x = fmaf(k.y, g.x, a2[0].x);
+                        a2[0].y = fmaf(k.y, g.y, a2[0].y);
+                    } else {
+                        const float2 kxx = make_float2(k.x, k.x), kyy = make_float2(k.y, k.y);
 #pragma unroll
-                    for (int q = 0; q < NPR; ++q) {
-                        const float4 g = reg[(size_t)q * plane + o];
-                        const float2 g0 = make_float2(g.x, g.y), g1 = make_float2(g.z, g.w);
-                        a1[2 * q] = __ffma2_rn(kxx, g0, a1[2 * q]);
-                        a2[2 * q] = __ffma2_rn(kyy, g0, a2[2 * q]);
-                        a1[2 * q + 1] = __ffma2_rn(kxx, g1, a1[2 * q + 1]);
-                        a2[2 * q + 1] = __ffma2_rn(kyy, g1, a2[2 * q + 1]);
-                    }
-                    if (NPOL % 2) {
-                        const float2 g = single[o];
-                        a1[NPOL - 1] = __ffma2_rn(kxx, g, a1[NPOL - 1]);
-                        a2[NPOL - 1] = __ffma2_rn(kyy, g, a2[NPOL - 1]);
+                        for (int q = 0; q < NPR; ++q) {
+                            const float4 g =
+                                *reinterpret_cast<const float4*>(regc + q * plane * kElem + o);
+                            const float2 g0 = make_float2(g.x, g.y), g1 = make_float2(g.z, g.w);
+                            a1[2 * q] = __ffma2_rn(kxx, g0, a1[2 * q]);
+                            a2[2 * q] = __ffma2_rn(kyy, g0, a2[2 * q]);
+                            a1[2 * q + 1] = __ffma2_rn(kxx, g1, a1[2 * q + 1]);
+                            a2[2 * q + 1] = __ffma2_rn(kyy, g1, a2[2 * q + 1]);
+                        }
+                        if (NPOL % 2) {
+                            const float2 g = *reinterpret_cast<const float2*>(
+                                regc + NPR * plane * kElem + o / 2);
+                            a1[NPOL - 1] = __ffma2_rn(kxx, g, a1[NPOL - 1]);
+                            a2[NPOL - 1] = __ffma2_rn(kyy, g, a2[NPOL - 1]);
+                        }
                     }
                 };
                 auto advance = [&]() {
@@ -565,14 +591,13 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                     }
                     kp += 32 * D;
                 }
-                // the last (< D) full steps and the partial one, from the front
-                // of the ring
-                for (; i <= nfull; ++i) {
-                    const bool live = i < nfull || lane + 32 * nfull < n;
-                    tap(live ? TE::cvt(kq[0]) : make_float2(0.f, 0.f), live ? off : zoff);
-                    advance();
+                // the last (< D) full steps and the partial one
 #pragma unroll
-                    for (int d = 0; d + 1 < D; ++d) kq[d] = kq[d + 1];
+                for (int d = 0; d < D; ++d) {
+                    if (i + d > nfull) break;
+                    const bool live = i + d < nfull || lane + 32 * nfull < n;
+                    tap(live ? TE::cvt(kq[d]) : make_float2(0.f, 0.f), live ? off : zoff * kElem);
+                    advance();
                 }
                 // conj(K_i) G with K_i = K (w >= 0) or conj K (w < 0):
                 // re = sum K.re G.re + s K.im G.im, im = sum K.re G.im - s K.im G.re
@@ -582,45 +607,31 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                     acc[p][0] = fmaf(sg, a2[p].y, a1[p].x);
                     acc[p][1] = fmaf(-sg, a2[p].x, a1[p].y);
                 }
-                if constexpr (NPOL == 4) {
-                    // reduce-scatter butterfly: lanes with bit 4 set keep pols 2, 3,
-                    // then bit 3 picks one of the two; 12 shuffles instead of 40
-                    const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0;
-                    const float k0r = (b4 ? acc[2][0] : acc[0][0]) +
-                                      __shfl_xor_sync(0xffffffffu, b4 ? acc[0][0] : acc[2][0], 16);
-                    const float k0i = (b4 ? acc[2][1] : acc[0][1]) +
-                                      __shfl_xor_sync(0xffffffffu, b4 ? acc[0][1] : acc[2][1], 16);
-                    const float k1r = (b4 ? acc[3][0] : acc[1][0]) +
-                                      __shfl_xor_sync(0xffffffffu, b4 ? acc[1][0] : acc[3][0], 16);
-                    const float k1i = (b4 ? acc[3][1] : acc[1][1]) +
-                                      __shfl_xor_sync(0xffffffffu, b4 ? acc[1][1] : acc[3][1], 16);
-                    float re = (b3 ? k1r : k0r) + __shfl_xor_sync(0xffffffffu, b3 ? k0r : k1r, 8);
-                    float im = (b3 ? k1i : k0i) + __shfl_xor_sync(0xffffffffu, b3 ? k0i : k1i, 8);
+                // reduce-scatter over the lanes: of the 2 NPOL sums (8 for 3
+                // polarisations, two of them zero) a lane keeps the half that
+                // its top bit picks, and so on down to one, which the lanes
+                // left sum; 6, 7 and 10 shuffles (1, 2 and 3-4 polarisations)
+                // where whole sums took 10, 20 and 40
+                constexpr int NV = NPOL == 3 ? 8 : 2 * NPOL;
+                float v[NV];
 #pragma unroll
-                    for (int d = 4; d > 0; d >>= 1) {
-                        re += __shfl_xor_sync(0xffffffffu, re, d);
-                        im += __shfl_xor_sync(0xffffffffu, im, d);
-                    }
-                    if ((lane & 7) == 0) {
-                        const int p = (b4 ? 2 : 0) + (b3 ? 1 : 0);
-                        finish(r, p, id, tv0, tv1 < S, re, im);
-                    }
-                } else {
+                for (int k = 0; k < NV; ++k) v[k] = k < 2 * NPOL ? acc[k / 2][k % 2] : 0.f;
+                int d = 16;
 #pragma unroll
-                    for (int p = 0; p < NPOL; ++p)
+                for (int w = NV / 2; w > 0; w >>= 1, d >>= 1) {
+                    const bool up = (lane & d) != 0;
 #pragma unroll
-                        for (int d = 16; d > 0; d >>= 1) {
-                            acc[p][0] += __shfl_xor_sync(0xffffffffu, acc[p][0], d);
-                            acc[p][1] += __shfl_xor_sync(0xffffffffu, acc[p][1], d);
-                        }
-                    if (lane < NPOL) {
-                        float re = acc[0][0], im = acc[0][1];
-#pragma unroll
-                        for (int p = 1; p < NPOL; ++p)
-                            if (lane == p) { re = acc[p][0]; im = acc[p][1]; }
-                        finish(r, lane, id, tv0, tv1 < S, re, im);
-                    }
+                    for (int k = 0; k < w; ++k)
+                        v[k] = (up ? v[k + w] : v[k]) +
+                               __shfl_xor_sync(0xffffffffu, up ? v[k] : v[k + w], d);
                 }
+                constexpr int kLow = 32 / NV;     // lanes that hold parts of the same sum
+#pragma unroll
+                for (; d > 0; d >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
+                // the lanes of the real part fetch the imaginary one
+                const float im = __shfl_down_sync(0xffffffffu, v[0], kLow);
+                if ((lane & (2 * kLow - 1)) == 0 && lane / (2 * kLow) < NPOL)
+                    finish(r, lane / (2 * kLow), id, tv0, tv1 < S, v[0], im);
             }
             __syncthreads();   // band consumed; after the last, the next chunk's metadata is in place
         }
