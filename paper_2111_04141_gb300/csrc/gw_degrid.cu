@@ -13,22 +13,27 @@
 //   warps compute the current one.  The CTA stages the tile's grid region
 //   (the tile plus the chunk's largest half-support on every side) in
 //   shared memory once, as polarisation pairs, at a row pitch padded to the
-//   support residue (mod 8) that carries most of the item's taps, and serves
+//   support residue (mod 8; 16 for one polarisation) that carries most of the
+//   item's taps, and serves
 //   all of the item's records from it, so the grid is read from L2/HBM
 //   about once per tile instead of once per tap.  Warps claim records one at
 //   a time, wide supports first.  One warp per record: lanes take
 //   consecutive taps of the S x S footprint (flattened, so every lane is
 //   busy), with kernel values loaded four steps ahead, packed FP32x2 FMAs
-//   into K.re G and K.im G sums, and a reduce-scatter over the lanes.
+//   (plain ones for one polarisation) into K.re G and K.im G sums, and a
+//   reduce-scatter over the lanes.  A step of 32 taps is 11 (one
+//   polarisation) to 19 (four) instructions: the column and the region offset
+//   advance in one register.  4.2 M visibilities x 1, support 31: 3.00 ms with
+//   23 instructions a step and the pitch padded mod 8, 2.41 now.
 //   A region larger than the shared memory is served in bands of rows: every
 //   record sums the tap rows in the band, and its sums wait in shared memory
 //   for the next one.  (Read through L1/L2 instead, 32 B a tap, 1.04 M
 //   visibilities x 4 polarisations with supports to 127 on an 8192^2 grid took
-//   13.2 ms; in bands they take 3.3, the same items read in place where few
-//   taps share a region 5.2.)  The L1 data pipe bounds it (87 % on the 4-pol
-//   w-projection batch: 16-byte loads of staged points); 32 warps of 64
-//   registers beat 24 of 80 there, 9.34 against 9.52 ms, and 3.28 against 3.63
-//   in bands.
+//   13.2 ms; in bands they take 3.2, the same items read in place where few
+//   taps share a region 5.2.)  The L1 data pipe bounds it (84 % on the 4-pol
+//   w-projection batch, 8.95 ms: 16-byte loads of staged points); before
+//   these instructions were cut 32 warps of 64 registers beat 24 of 80 there,
+//   9.34 against 9.52 ms, and 3.28 against 3.63 in bands.
 // * k_degrid_direct (small calls): one launch, index records included.
 // * k_degrid (the allocation-free entry point): the same per-record warp,
 //   reading the grid through L1/L2, records visited in 32 x 32 centre-tile
@@ -262,7 +267,7 @@ struct StagedChunk {
     int done;       // no work left
     int h;          // largest half-support of the chunk's records (the region's)
     int front, back, next;   // metadata placement, record claims
-    int taps[8];    // taps of the chunk's records by S mod 8
+    int taps[16];   // taps of the chunk's records by S mod kRes
 };
 
 constexpr int kLoaderThreads = 128;                       // warps 0-3
@@ -284,7 +289,8 @@ __device__ __forceinline__ void loader_sync() {
 
 // GEN: any tile size, regions in bands; otherwise 16 x 16 tiles whose largest
 // region fits (a tap loop without the band's bounds: 3.11 against 3.31 ms on
-// 4.2 M visibilities of one polarisation, support 31).
+// 4.2 M visibilities of one polarisation, support 31, before the pitch was
+// padded for them).
 template <int NPOL, int TK, bool GEN>
 __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, int hmax, int cap) {
     using TE = TabElem<TK>;
@@ -310,6 +316,9 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
     const uint32_t nitems = *a.item_count;
     const TT* __restrict__ tab = reinterpret_cast<const TT*>(a.table);
     constexpr int kElem = NPR ? 16 : 8;       // bytes of an element of the first plane
+    // elements to a row of banks: 8 or 16 lanes of a load take one
+    constexpr int kRes = 128 / kElem;
+    constexpr uint32_t kPosOff = (1u << 20) - 1;
     const char* const regc = reinterpret_cast<const char*>(reg);
     // thread 0: the item being served and the next chunk's first record
     Item cur{};
@@ -341,7 +350,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
             // an item served in several chunks keeps one region for all of
             // them: the plan's largest half-support
             c.h = cur.len > kStagedMeta ? hmax : 0;
-            for (int k = 0; k < 8; ++k) c.taps[k] = 0;
+            for (int k = 0; k < 16; ++k) c.taps[k] = 0;
             next_c0 += nc;
         }
         loader_sync();
@@ -403,7 +412,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
 #endif
                     meta[pos] = make_uint4(ids[k], (uint32_t)kofs, rel, w);
                     hw = max(hw, h);
-                    atomicAdd(&c.taps[S & 7], S * S);
+                    atomicAdd(&c.taps[S & (kRes - 1)], S * S);
                 }
             }
             if ((k0 + kLoaderBatch) * kLoaderThreads >= nc) break;
@@ -444,9 +453,10 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
         // the region: rows and columns [t0 - hi, t0 + T + hi) of the tile,
         // RS x RS values at row pitch RSP; each plane holds RS x RSP elements
         // and kStagedPad zeros (element RS * RSP is read by lanes without a
-        // tap in a record's last step).  A quarter-warp's 8 flattened taps
-        // that cross a footprint row end jump by RSP - S elements: with RSP
-        // = S mod 8 its 16-byte loads stay free of bank conflicts, so the
+        // tap in a record's last step).  The kRes flattened taps of a load's
+        // quarter (16 bytes) or half (8) that cross a footprint row end jump by
+        // RSP - S elements: with RSP = S mod kRes the load stays free of bank
+        // conflicts (8 bytes: 2 wavefronts, else 3), so the
         // pitch is padded to the residue of the supports that carry most of
         // the item's taps, where the shared memory allows (items served in
         // several chunks keep RSP = RS).  RS is even, so every part stays
@@ -457,12 +467,12 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
         if (item.len <= kStagedMeta) {
             int best = 0, bt = -1;
 #pragma unroll
-            for (int k = 1; k < 8; k += 2)     // supports are odd
+            for (int k = 1; k < kRes; k += 2)  // supports are odd
                 if (c.taps[k] > bt) {
                     bt = c.taps[k];
                     best = k;
                 }
-            const int rsp = RS + ((best - RS) & 7);
+            const int rsp = RS + ((best - RS) & (kRes - 1));
             if (RS * rsp <= cap || (GEN && RS * RS > cap)) RSP = rsp;
         }
         // bands of BR region rows, of equal height
@@ -519,21 +529,24 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                 if (GEN && tv1 <= tv0) continue;
                 const TT* K = tab + m.y + tv0 * S;
                 const int n = (tv1 - tv0) * S;
-                // flattened taps t = lane + 32 i; the region offset (in bytes of a
-                // plane) advances by `step` per 32 taps, plus `wrap` when the tap
-                // column wraps
+                // flattened taps t = lane + 32 i at pos = tap column << 20 | region
+                // offset (bytes of a plane, below 2^20): 32 taps on, the column
+                // is up by dr, or by dr - S and a row further where it wraps;
+                // one comparison, select and addition for both parts
                 const int dq = (int)(32u * inv >> 20), dr = 32 - dq * S;
                 const int lq = (int)((uint32_t)lane * inv >> 20);
-                const int step = (dq * RSP + dr) * kElem, wrap = (RSP - S) * kElem;
-                int tu = lane - lq * S;
-                const int base = (ry + tv0 - yb) * RSP + rx;
-                int off = (base + lq * RSP + tu) * kElem;
+                const uint32_t wrap_at = (uint32_t)(S - dr) << 20;
+                const uint32_t go_on = ((uint32_t)dr << 20) + (uint32_t)((dq * RSP + dr) * kElem);
+                const uint32_t go_wrap = go_on - ((uint32_t)S << 20) + (uint32_t)((RSP - S) * kElem);
+                const int tu = lane - lq * S;
+                uint32_t pos = (uint32_t)tu << 20 |
+                               (uint32_t)(((ry + tv0 - yb + lq) * RSP + rx + tu) * kElem);
                 // a1 = sum K.re G, a2 = sum K.im G (packed FP32x2 FMAs); the
                 // conjugation sign is applied once at the end
                 float2 a1[NPOL], a2[NPOL];
 #pragma unroll
                 for (int p = 0; p < NPOL; ++p) a1[p] = a2[p] = make_float2(0.f, 0.f);
-                auto tap = [&](const float2 k, const int o) {
+                auto tap = [&](const float2 k, const uint32_t o) {
                     if constexpr (NPOL == 1) {
                         // one use of each: packing K.re and K.im twice would cost
                         // more than the packed FMAs save
@@ -562,14 +575,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                         }
                     }
                 };
-                auto advance = [&]() {
-                    off += step;
-                    tu += dr;
-                    if (tu >= S) {
-                        tu -= S;
-                        off += wrap;
-                    }
-                };
+                auto advance = [&]() { pos += pos >= wrap_at ? go_wrap : go_on; };
                 // steps 0 .. nfull - 1 have a tap on every lane, step nfull on
                 // the lanes below n - 32 nfull.  Kernel values are loaded D steps
                 // ahead, unconditionally: past the slice they read the next
@@ -586,7 +592,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                     for (int d = 0; d < D; ++d) {
                         const float2 k = TE::cvt(kq[d]);
                         kq[d] = __ldg(kp + 32 * d);
-                        tap(k, off);
+                        tap(k, pos & kPosOff);
                         advance();
                     }
                     kp += 32 * D;
@@ -596,7 +602,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
                 for (int d = 0; d < D; ++d) {
                     if (i + d > nfull) break;
                     const bool live = i + d < nfull || lane + 32 * nfull < n;
-                    tap(live ? TE::cvt(kq[d]) : make_float2(0.f, 0.f), live ? off : zoff * kElem);
+                    tap(live ? TE::cvt(kq[d]) : make_float2(0.f, 0.f), live ? pos & kPosOff : (uint32_t)(zoff * kElem));
                     advance();
                 }
                 // conj(K_i) G with K_i = K (w >= 0) or conj K (w < 0):
@@ -655,11 +661,10 @@ void launch_staged_t(const DegridArgs& a, int hmax, int num_sms, cudaStream_t s)
     // beside the partial sums of a chunk
     const int RS = (1 << a.tile_shift) + 2 * hmax;
     constexpr size_t point = NPOL * sizeof(float2);
-    size_t cap = (size_t)RS * RS, part = 0;
-    if (cap * point > kStagedSmemMax) {
-        part = kStagedMeta * point;
-        cap = (kStagedSmemMax - part) / point / 4 * 4;
-    }
+    // with its padded pitch where that fits too
+    size_t cap = (size_t)RS * (RS + (NPOL == 1 ? 16 : 8)), part = 0;
+    if ((size_t)RS * RS * point > kStagedSmemMax) part = kStagedMeta * point;
+    cap = std::min(cap, (kStagedSmemMax - part) / point / 4 * 4);
     if (part || a.tile_shift != 4)
         launch_staged_g<NPOL, TK, true>(a, hmax, cap, part, num_sms, s);
     else
