@@ -138,31 +138,39 @@ __device__ __forceinline__ void screen_fixed(double w30, double nm1, float& s, f
 // the sum is FP32.  The layer images are the inverse transforms of the
 // unshifted layer grids: the centring factor (-1)^(u + v) of the grid is the
 // circular shift by N/2 of its transform, applied here in the read (N is
-// even).  One thread per pixel; the layers are read once, coalesced.
+// even).  The layers are read once, coalesced.
 //
 // FIXED: FP64 operations bound the kernel, not the layers it reads, so n - 1 =
 // sqrt(1 - r^2) - 1 is an FP32 square root and one Newton step (error below
 // 2e-14), and every phase one FP64 operation (screen_fixed).  Otherwise (w of
 // 2^18 wavelengths and more) the phases are reduced in FP64.  16 layers of
 // 2048^2 x 1: 521 us reduced in FP64, 270 us fixed.
-template <bool FIXED>
-__global__ void k_wstack_combine(const float2* __restrict__ layers, int nlayers, double wmin,
-                                 double dw, int N, int npol, double cell,
-                                 float2* __restrict__ image) {
+//
+// The four pixels (+-i, +-j) from the image's centre have the same screens: a
+// thread serves all four (their transform rows are i and N - i), so the
+// phases and the recursion are formed once for them.  The same 16 layers: 270
+// us with a thread a pixel, 104 us here (0.54 GB read, 5.2 TB/s: HBM bound).
+template <bool FIXED, int NPOL>
+__global__ void __launch_bounds__(256) k_wstack_combine(const float2* __restrict__ layers,
+                                                        int nlayers, double wmin, double dw, int N,
+                                                        double cell, float2* __restrict__ image) {
     const int64_t n = (int64_t)N * N;
-    const int half = N / 2;
+    const int half = N / 2, side = half + 1;
     const double c2 = cell * cell;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)((uint32_t)e / (uint32_t)N), j = (int)(e - (int64_t)i * N);
-        const int is = i + half < N ? i + half : i - half;
-        const int js = j + half < N ? j + half : j - half;
-        const int64_t es = (int64_t)is * N + js;      // pixel of the unshifted transform
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < side * side;
+         e += gridDim.x * blockDim.x) {
+        const int i = e / side, j = e - i * side;     // offsets from the centre, 0 .. N/2
+        // the pixels in the unshifted transform; 0 and N/2 have no mirror
+        const bool mi = i > 0 && i < half, mj = j > 0 && j < half;
+        const bool on[4] = {true, mj, mi, mi && mj};
+        const int rows[2] = {i, mi ? N - i : i}, cols[2] = {j, mj ? N - j : j};
+        int es[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) es[q] = rows[q >> 1] * N + cols[q & 1];
         double nm1;
         if constexpr (FIXED) {
             // r^2 = cell^2 (l^2 + m^2), the sum of squares an exact integer
-            const int q = (j - half) * (j - half) + (i - half) * (i - half);
-            const double a = __fma_rn(-c2, (double)q, 1.0);
+            const double a = __fma_rn(-c2, (double)(i * i + j * j), 1.0);
             nm1 = 0.0;
             if (a > 0.0) {
                 const float s0 = sqrtf((float)a);
@@ -171,7 +179,7 @@ __global__ void k_wstack_combine(const float2* __restrict__ layers, int nlayers,
                 nm1 = (sd - 1.0) + (double)corr;
             }
         } else {
-            const double l = (j - half) * cell, m = (i - half) * cell;
+            const double l = j * cell, m = i * cell;
             const double r2 = l * l + m * m;
             nm1 = r2 < 1.0 ? -r2 / (1.0 + sqrt(1.0 - r2)) : 0.0;
         }
@@ -180,29 +188,45 @@ __global__ void k_wstack_combine(const float2* __restrict__ layers, int nlayers,
             screen_fixed(dw * kPhaseScale, nm1, s1, c1);
         else
             screen_pi(2.0 * dw * nm1, s1, c1);
-        float acc[4][2] = {};
+        float acc[4][NPOL][2] = {};
         float cr = 1.f, ci = 0.f;
-        for (int L = 0; L < nlayers; ++L) {
+        const float2* layer = layers;
+        for (int L = 0; L < nlayers; ++L, layer += NPOL * n) {
+            float2 v[4][NPOL];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int p = 0; p < NPOL; ++p) v[q][p] = __ldcs(layer + p * n + es[q]);
             if ((L & 7) == 0) {
                 if constexpr (FIXED)
                     screen_fixed((wmin + L * dw) * kPhaseScale, nm1, ci, cr);
                 else
                     screen_pi(2.0 * (wmin + L * dw) * nm1, ci, cr);
             }
-            for (int p = 0; p < npol && p < 4; ++p) {
-                const float2 v = __ldcs(layers + ((int64_t)L * npol + p) * n + es);
-                acc[p][0] = fmaf(v.x, cr, fmaf(-v.y, ci, acc[p][0]));
-                acc[p][1] = fmaf(v.x, ci, fmaf(v.y, cr, acc[p][1]));
-            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int p = 0; p < NPOL; ++p) {
+                    acc[q][p][0] = fmaf(v[q][p].x, cr, fmaf(-v[q][p].y, ci, acc[q][p][0]));
+                    acc[q][p][1] = fmaf(v[q][p].x, ci, fmaf(v[q][p].y, cr, acc[q][p][1]));
+                }
             const float nr = cr * c1 - ci * s1, ni = cr * s1 + ci * c1;
             cr = nr;
             ci = ni;
         }
-        for (int p = 0; p < npol && p < 4; ++p) {
-            float2 o = image[(int64_t)p * n + e];
-            o.x += acc[p][0];
-            o.y += acc[p][1];
-            image[(int64_t)p * n + e] = o;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (!on[q]) continue;
+            const int r = rows[q >> 1], c = cols[q & 1];
+            const int64_t px = (int64_t)(r < half ? r + half : r - half) * N +
+                               (c < half ? c + half : c - half);
+#pragma unroll
+            for (int p = 0; p < NPOL; ++p) {
+                float2 o = image[p * n + px];
+                o.x += acc[q][p][0];
+                o.y += acc[q][p][1];
+                image[p * n + px] = o;
+            }
         }
     }
 }
@@ -250,12 +274,17 @@ void launch_wstack_combine(const float2* layers, int nlayers, double wmin, doubl
                            int npol, double cell, float2* image, cudaStream_t s) {
     // |n - 1| <= 1; the sum of squares of pixel offsets fits 31 bits for any N
     const double w = std::max(std::abs(wmin), std::abs(wmin + (nlayers - 1) * dw));
-    const unsigned blocks = blocks_for((int64_t)N * N);
-    if (std::max(w, std::abs(dw)) < kPhaseTurns)
-        k_wstack_combine<true><<<blocks, 256, 0, s>>>(layers, nlayers, wmin, dw, N, npol, cell, image);
-    else
-        k_wstack_combine<false><<<blocks, 256, 0, s>>>(layers, nlayers, wmin, dw, N, npol, cell,
-                                                       image);
+    const unsigned blocks = blocks_for((int64_t)(N / 2 + 1) * (N / 2 + 1));
+    const bool fixed = std::max(w, std::abs(dw)) < kPhaseTurns;
+    auto go = [&](auto f, auto g) {
+        (fixed ? f : g)<<<blocks, 256, 0, s>>>(layers, nlayers, wmin, dw, N, cell, image);
+    };
+    switch (npol) {
+        case 1: go(k_wstack_combine<true, 1>, k_wstack_combine<false, 1>); break;
+        case 2: go(k_wstack_combine<true, 2>, k_wstack_combine<false, 2>); break;
+        case 3: go(k_wstack_combine<true, 3>, k_wstack_combine<false, 3>); break;
+        default: go(k_wstack_combine<true, 4>, k_wstack_combine<false, 4>); break;
+    }
     note_launch();
 }
 
