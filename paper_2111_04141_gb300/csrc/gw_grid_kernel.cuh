@@ -455,12 +455,28 @@ struct PairEntries {
     }
 };;
 
+// A pair of the FP32 table, zero where `on` is false: one predicated load.  (A
+// conditional one became a branch: 1 polarisation 2.94 ms, so 2.82.  With two
+// polarisations, and in FmaWarp, the conditional loads schedule better: 1.57
+// against 1.59 ms and 8.23 against 8.79.)
+__device__ __forceinline__ float4 load_pair(const float4* __restrict__ p, bool on) {
+    float4 v;
+    asm("{.reg .pred q; setp.ne.u32 q, %5, 0;\n"
+        " mov.f32 %0, 0f00000000; mov.f32 %1, 0f00000000;\n"
+        " mov.f32 %2, 0f00000000; mov.f32 %3, 0f00000000;\n"
+        " @q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];}"
+        : "=&f"(v.x), "=&f"(v.y), "=&f"(v.z), "=&f"(v.w)
+        : "l"(p), "r"((uint32_t)on));
+    return v;
+}
+
 // FP32 tables with one or two polarisations.  With so few FMAs an entry the
 // gathers bound the kernel (each a quarter-warp's cache lines), and a 16-byte
 // load of a pair takes 8 lanes through one 128-byte row: about 7.5 lines for
 // 64 points against 11.5 for two 8-byte loads of 8 x 4 points.  4.2 M
 // visibilities, 1 polarisation, support 31, 2048^2: 3.65 ms with FmaWarp; here
-// 3.30 / 3.23 / 2.98 / 2.90 with 3 / 4 / 5 / 6 entries in flight.  With more
+// 3.30 / 3.23 / 2.98 / 2.90 with 3 / 4 / 5 / 6 entries in flight (2.82 with
+// predicated loads).  With more
 // polarisations the FMAs share the bound and the 8 x 16 blocks of FmaWarp
 // stay ahead (4: 8.2 against 9.2 ms on the 4096^2 batch).
 // Lane (g, r) = (lane % 8, lane / 8): points 2 g, 2 g + 1 of rows r and r + 4.
@@ -492,10 +508,15 @@ struct PairWarp {
         const uint32_t q = ((en.y >> 8) & 0x7fu) + 1u, off = en.x + g + r * q;
         const uint32_t c = 1u << (kPairCols + g);
         const uint32_t m0 = c | 1u << (kPairRows + r), m1 = c | 1u << (kPairRows + 4 + r);
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
         ey[d] = en.y;
-        K[d][0] = (en.y & m0) == m0 ? __ldg(tab + off) : z;
-        K[d][1] = (en.y & m1) == m1 ? __ldg(tab + (off + 4 * q)) : z;
+        if constexpr (NPOL == 1) {
+            K[d][0] = load_pair(tab + off, (~en.y & m0) == 0);
+            K[d][1] = load_pair(tab + (off + 4 * q), (~en.y & m1) == 0);
+        } else {
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            K[d][0] = (en.y & m0) == m0 ? __ldg(tab + off) : z;
+            K[d][1] = (en.y & m1) == m1 ? __ldg(tab + (off + 4 * q)) : z;
+        }
     }
     __device__ __forceinline__ void fill(const uint2* lst, const VT (*)[NPOL]) {
 #pragma unroll
