@@ -128,7 +128,7 @@ struct gw_plan_s {
     gw_plan_desc desc{};
     int device = -1;
     int num_sms = 0;
-    BinGeom geom_grid{}, geom_degrid{}, geom_staged{}, geom_staged64{};
+    BinGeom geom_grid{}, geom_degrid{}, geom_staged{}, geom_staged64{}, geom_staged128{};
     int hmax = 0;        // largest half-support over the planes
     int ntiles = 0;      // bins allocated (max over the geometries and plane groups)
     int max_groups = 1;  // plane groups the bins are allocated for (gw_tuning.plane_groups)
@@ -350,6 +350,7 @@ void apply_tuning(gw_plan p) {
     p->geom_degrid.item_max = im;
     p->geom_staged.item_max = im;
     p->geom_staged64.item_max = im;
+    p->geom_staged128.item_max = im;
 }
 
 enum Stage { kStIndex = 0, kStBin = 1, kStGrid = 2, kStDegrid = 3 };
@@ -512,6 +513,7 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     p->geom_degrid = BinGeom{1, 5, 5, (N + kTile - 1) / kTile, (N + kTile - 1) / kTile};
     p->geom_staged = BinGeom{1, 4, 4, (N + 15) / 16, (N + 15) / 16};
     p->geom_staged64 = BinGeom{1, 6, 6, (N + 63) / 64, (N + 63) / 64};
+    p->geom_staged128 = BinGeom{1, 7, 7, (N + 127) / 128, (N + 127) / 128};
     p->ntiles = std::max({p->geom_grid.ntu * p->geom_grid.ntv,
                           p->geom_degrid.ntu * p->geom_degrid.ntv,
                           p->geom_staged.ntu * p->geom_staged.ntv});
@@ -730,6 +732,7 @@ gw_status gw_plan_clone(gw_plan src, int64_t max_vis_per_call, void* cuda_stream
     p->geom_degrid = src->geom_degrid;
     p->geom_staged = src->geom_staged;
     p->geom_staged64 = src->geom_staged64;
+    p->geom_staged128 = src->geom_staged128;
     p->hmax = src->hmax;
     p->ntiles = src->ntiles;
     p->max_groups = src->max_groups;
@@ -890,16 +893,25 @@ gw_status gw_plan_info_get(gw_plan p, gw_plan_info* out) {
 // staged once for the records centred in it, so sparse inputs take larger
 // tiles.  By visibilities per 16 x 16 points (kernel times):
 //   16 (255 k x 4, 2048^2, support 7-41): 16 / 32 / 64-point tiles 380 / 260 / 331 us
-//   4  (1.04 M x 4, 8192^2, support 7-127): 32 / 64 / 128 4.88 / 3.63 / 3.52 ms
+//   4  (1.04 M x 4, 8192^2, support 7-127): 32 / 64 / 128 4.88 / 3.17 / 2.99 ms
 //   63 (1.04 M x 4, 2048^2, support 7-127): 16 / 64 4.53 / 4.03 ms
 //   126 (8.3 M x 4, 4096^2, support 7-63): 16 / 32 / 64 9.52 / 9.89 / 10.7 ms
 // Where the region of 16-point tiles does not fit and is served in bands, 32
-// points are taken at any density.  A size needs kStagedMinTiles of its tiles,
+// points are taken at any density.  128 points are taken where their margins
+// are most of a 64-point tile's region, or where there is next to nothing in a
+// tile: 64 / 128 points, kernels in ms, 8192^2,
+//   0.23 (60 k), support 7-41: x 1 0.40 / 0.27, x 4 0.76 / 0.61
+//   1 and 2 (261 k, 522 k) x 4, support 7-41: 0.50 / 0.53, 0.68 / 0.77
+//   4 (1.04 M) x 4, support to 65 / 79 / 95: 1.53 / 1.63, 1.85 / 1.91, 2.28 / 2.27
+//   2 and 6 (0.5 M, 1.6 M) x 4, support to 127: 1.84 / 1.80, 4.22 / 4.05
+// (binning takes 85 us with 64, 42 with 128).  A size needs kStagedMinTiles of its tiles,
 // so that every SM gets several (62 k x 4, 1000^2: 16 / 32 points 70 / 85 us;
 // 12 k x 1, 1656^2: 16 / 32 / 64 84 / 45 / 46 us).
 static const BinGeom& staged_geom(gw_plan p, int64_t nvis) {
     const double n = (double)p->desc.grid_n, per = (double)nvis * 256.0;
     auto enough = [](const BinGeom& g) { return g.ntu * g.ntv >= kStagedMinTiles; };
+    const double sparse128 = p->hmax >= kStagedWide128 ? kStagedSparse64 : kStagedSparse128;
+    if (per < sparse128 * n * n && enough(p->geom_staged128)) return p->geom_staged128;
     if (per < kStagedSparse64 * n * n && enough(p->geom_staged64)) return p->geom_staged64;
     if (staged_banded(p->hmax, p->desc.npol) ||
         (per < kStagedSparse32 * n * n && enough(p->geom_degrid)))

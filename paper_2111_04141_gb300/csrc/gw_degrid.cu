@@ -8,8 +8,8 @@
 // Three kernels:
 // * k_degrid_staged (used by gw_degrid_vis): one CTA of 32 warps per SM
 //   serves chunks of work items (at most 1,024 records centred in one tile of
-//   16 x 16 points, or 32 x 32 or 64 x 64 for sparse inputs).  Warps 0-3 load the records' metadata (id, kernel slice, centre,
-//   support) into one of two shared buffers, the next chunk's while all
+//   16 x 16 points, or 32 x 32 to 128 x 128 for sparse inputs).  Warps 0-3
+//   load the records' metadata (id, kernel slice, centre, support) into one of two shared buffers, the next chunk's while all
 //   warps compute the current one.  The CTA stages the tile's grid region
 //   (the tile plus the chunk's largest half-support on every side) in
 //   shared memory once, as polarisation pairs, at a row pitch padded to the
@@ -29,7 +29,7 @@
 //   record sums the tap rows in the band, and its sums wait in shared memory
 //   for the next one.  (Read through L1/L2 instead, 32 B a tap, 1.04 M
 //   visibilities x 4 polarisations with supports to 127 on an 8192^2 grid took
-//   13.2 ms; in bands they take 3.2, the same items read in place where few
+//   13.2 ms; in bands they take 3.0, the same items read in place where few
 //   taps share a region 5.2.)  The L1 data pipe bounds it (84 % on the 4-pol
 //   w-projection batch, 8.95 ms: 16-byte loads of staged points); before
 //   these instructions were cut 32 warps of 64 registers beat 24 of 80 there,

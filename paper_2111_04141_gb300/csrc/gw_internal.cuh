@@ -393,10 +393,13 @@ constexpr int64_t kGroupTargetBytes = 64ll << 20;
 // Bands of tile rows a banded read-back may use (gw_grid_vis_devcount_readback).
 constexpr int kReadbackBandsMax = 64;
 constexpr int64_t kDirectMaxTaps = (int64_t)1 << 22;
-// Staged degridding takes 32 x 32 and 64 x 64 centre tiles instead of 16 x 16
-// below this many visibilities per 16 x 16 points on average.
+// Staged degridding takes 32 x 32, 64 x 64 and 128 x 128 centre tiles instead
+// of 16 x 16 below this many visibilities per 16 x 16 points on average, 128
+// with supports above 2 kStagedWide128 already below kStagedSparse64.
 constexpr double kStagedSparse32 = 48.0;
 constexpr double kStagedSparse64 = 6.0;
+constexpr double kStagedSparse128 = 0.5;
+constexpr int kStagedWide128 = 48;
 constexpr int kStagedMinTiles = 2048;
 // One instantiation set per table kind (gw_grid_c64.cu, gw_grid_bf16.cu, gw_grid_f16.cu,
 // gw_grid_r32.cu).

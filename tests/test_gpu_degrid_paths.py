@@ -95,3 +95,13 @@ def test_dense_tiles_and_long_items(gw, smax, item_max):
                          n_w=3, beta=4, diameter_m=1000.0, seed=31)
     obs.uvw_m[:, :2] *= 0.06
     check(gw, obs, bands=smax == 71, degrid_kernel=1, item_max=item_max)
+
+
+# large grids with few records: centre tiles of 64 x 64 (17 k on 2900^2) and of
+# 128 x 128 points, the last tile of a row cut off, in one piece and in bands
+@pytest.mark.parametrize("npol,n,n_ant,n_times,smin,smax", [
+    (1, 2900, 20, 30, 3, 17), (2, 2900, 20, 30, 5, 41), (1, 5830, 6, 9, 1, 9), (1, 5830, 6, 9, 9, 127)])
+def test_sparse_inputs_take_large_tiles(gw, npol, n, n_ant, n_times, smin, smax):
+    obs = syn.small_case(n_ant=n_ant, n_times=n_times, n_chan=3, npol=npol, grid_n=n, s_min=smin,
+                         s_max=smax, n_w=3, beta=4, diameter_m=20.0 * n, seed=37)
+    check(gw, obs, bands=smax > 17, degrid_kernel=1)
