@@ -236,7 +236,7 @@ __global__ void k_scatter(const gw_index_rec* __restrict__ rec, int64_t nvis, De
 // memory, one atomic each.  The scatter recounts its chunk, reserves one run
 // per (CTA, tile) in the tile's bin with a single global atomic, and places
 // the entries with shared-memory cursors that start at the run bases.
-constexpr int kBinSmThreads = 512;
+constexpr int kBinSmThreads = 1024;
 constexpr int kBinSmTilesMax = 49152;     // 192 KB of u32 counters
 // Fewest CTAs worth it, at one CTA per ntiles records.  255 k records over
 // 16,384 tiles (15 CTAs) bin in 115 us with shared histograms and 55 us with
@@ -244,29 +244,64 @@ constexpr int kBinSmTilesMax = 49152;     // 192 KB of u32 counters
 // 32,768 (95 CTAs) in 300 and 500, 30 k over 512 (59 CTAs) in 24 and 39.
 constexpr int kBinSmBlocksMin = 48;
 
+// Work on the records [c0, c1) of a CTA, kBinIlp loads of a thread in flight:
+// one at a time with 512 threads, the loads' latency bounded these kernels (bin
+// stage, us, before / now: 3.1 M records over 32,768 bins 275 / 199, 4.2 M over
+// 2,048 and 16,384 258 / 229, 255 k over 4,096 39 / 32, 8.3 M over 8,192 261 /
+// 259).  Lanes of one bin sharing an atomic (match_any) were slower: 437 / 337 on
+// the first two.
+constexpr int kBinIlp = 4;
+
+template <class F>
+__device__ __forceinline__ void each_record(const gw_index_rec* __restrict__ rec, int64_t c0,
+                                            int64_t c1, F f) {
+    for (int64_t i0 = c0 + threadIdx.x; i0 < c1; i0 += kBinIlp * kBinSmThreads) {
+        gw_index_rec r[kBinIlp];
+#pragma unroll
+        for (int k = 0; k < kBinIlp; ++k) {
+            const int64_t i = i0 + k * kBinSmThreads;
+            if (i < c1) r[k] = load_rec(rec, i);
+            else r[k].flags = 0;
+        }
+#pragma unroll
+        for (int k = 0; k < kBinIlp; ++k)
+            if (r[k].flags & GW_FLAG_VALID) f(r[k], (uint32_t)(i0 + k * kBinSmThreads));
+    }
+}
+
+// Calls f with the bin of each tile that a record meets.
+template <class F>
+__device__ __forceinline__ void each_bin(const gw_index_rec& r, const BinGeom& g, int P, int smin,
+                                         int smax, F f) {
+    const TileRange t = tile_range(r, g, P, smin, smax);
+    const int lbase = g.layer_tiles ? (r.plane / g.group_planes) * g.layer_tiles : 0;
+    for (int tv = t.tv0; tv <= t.tv1; ++tv)
+        for (int tu = t.tu0; tu <= t.tu1; ++tu) f(lbase + tv * g.ntu + tu);
+}
+
+__device__ __forceinline__ void clear_hist(uint32_t* hist, int ntiles) {
+    for (int t = threadIdx.x * 4; t < ntiles; t += 4 * kBinSmThreads)
+        *reinterpret_cast<uint4*>(hist + t) = make_uint4(0u, 0u, 0u, 0u);
+}
+
 __global__ void __launch_bounds__(kBinSmThreads) k_count_sm(
     const gw_index_rec* __restrict__ rec, int64_t nvis, DevCount dc, BinGeom g, int P, int smin,
     int smax, int ntiles, uint32_t* __restrict__ count, unsigned long long* __restrict__ work) {
-    extern __shared__ uint32_t hist[];
+    extern __shared__ __align__(16) uint32_t hist[];
     nvis = dc.clamp(nvis);
-    for (int t = threadIdx.x; t < ntiles; t += blockDim.x) hist[t] = 0;
+    clear_hist(hist, ntiles);
     __syncthreads();
     const int64_t chunk = (nvis + gridDim.x - 1) / gridDim.x;
     const int64_t c0 = blockIdx.x * chunk, c1 = min(nvis, c0 + chunk);
     unsigned long long n_valid = 0, n_taps = 0;
-    for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
-        const gw_index_rec r = load_rec(rec, i);
-        if (!(r.flags & GW_FLAG_VALID)) continue;
+    each_record(rec, c0, c1, [&](const gw_index_rec& r, uint32_t) {
         const int S = plane_support(r.plane, P, smin, smax);
         ++n_valid;
         n_taps += (unsigned long long)(S * S);
-        const TileRange t = tile_range(r, g, P, smin, smax);
-        const int lbase = g.layer_tiles ? (r.plane / g.group_planes) * g.layer_tiles : 0;
-        for (int tv = t.tv0; tv <= t.tv1; ++tv)
-            for (int tu = t.tu0; tu <= t.tu1; ++tu) atomicAdd(hist + lbase + tv * g.ntu + tu, 1u);
-    }
+        each_bin(r, g, P, smin, smax, [&](int t) { atomicAdd(hist + t, 1u); });
+    });
     __syncthreads();
-    for (int t = threadIdx.x; t < ntiles; t += blockDim.x)
+    for (int t = threadIdx.x; t < ntiles; t += kBinSmThreads)
         if (hist[t]) atomicAdd(count + t, hist[t]);
     for (int d = 16; d > 0; d >>= 1) {
         n_valid += __shfl_down_sync(0xffffffffu, n_valid, d);
@@ -282,38 +317,36 @@ __global__ void __launch_bounds__(kBinSmThreads) k_scatter_sm(
     const gw_index_rec* __restrict__ rec, int64_t nvis, DevCount dc, BinGeom g, int P, int smin,
     int smax, int ntiles, const uint32_t* __restrict__ offsets, uint32_t* __restrict__ cursor,
     uint32_t* __restrict__ entries) {
-    extern __shared__ uint32_t hist[];
+    extern __shared__ __align__(16) uint32_t hist[];
     nvis = dc.clamp(nvis);
-    for (int t = threadIdx.x; t < ntiles; t += blockDim.x) hist[t] = 0;
+    clear_hist(hist, ntiles);
     __syncthreads();
     const int64_t chunk = (nvis + gridDim.x - 1) / gridDim.x;
     const int64_t c0 = blockIdx.x * chunk, c1 = min(nvis, c0 + chunk);
-    for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
-        const gw_index_rec r = load_rec(rec, i);
-        if (!(r.flags & GW_FLAG_VALID)) continue;
-        const TileRange t = tile_range(r, g, P, smin, smax);
-        const int lbase = g.layer_tiles ? (r.plane / g.group_planes) * g.layer_tiles : 0;
-        for (int tv = t.tv0; tv <= t.tv1; ++tv)
-            for (int tu = t.tu0; tu <= t.tu1; ++tu) atomicAdd(hist + lbase + tv * g.ntu + tu, 1u);
-    }
+    each_record(rec, c0, c1, [&](const gw_index_rec& r, uint32_t) {
+        each_bin(r, g, P, smin, smax, [&](int t) { atomicAdd(hist + t, 1u); });
+    });
     __syncthreads();
     // this CTA's run in each bin: absolute position of its first entry
-    for (int t = threadIdx.x; t < ntiles; t += blockDim.x) {
-        const uint32_t c = hist[t];
-        if (c) hist[t] = offsets[t] + atomicAdd(cursor + t, c);
+    for (int t0 = threadIdx.x; t0 < ntiles; t0 += kBinIlp * kBinSmThreads) {
+        uint32_t c[kBinIlp], o[kBinIlp];
+#pragma unroll
+        for (int k = 0; k < kBinIlp; ++k) {
+            const int t = t0 + k * kBinSmThreads;
+            c[k] = t < ntiles ? hist[t] : 0u;
+            o[k] = c[k] ? __ldg(offsets + t) : 0u;
+            c[k] = c[k] ? atomicAdd(cursor + t, c[k]) : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < kBinIlp; ++k) {
+            const int t = t0 + k * kBinSmThreads;
+            if (t < ntiles) hist[t] = o[k] + c[k];
+        }
     }
     __syncthreads();
-    for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
-        const gw_index_rec r = load_rec(rec, i);
-        if (!(r.flags & GW_FLAG_VALID)) continue;
-        const TileRange t = tile_range(r, g, P, smin, smax);
-        const int lbase = g.layer_tiles ? (r.plane / g.group_planes) * g.layer_tiles : 0;
-        for (int tv = t.tv0; tv <= t.tv1; ++tv)
-            for (int tu = t.tu0; tu <= t.tu1; ++tu) {
-                const uint32_t pos = atomicAdd(hist + lbase + tv * g.ntu + tu, 1u);
-                entries[pos] = (uint32_t)i;
-            }
-    }
+    each_record(rec, c0, c1, [&](const gw_index_rec& r, uint32_t id) {
+        each_bin(r, g, P, smin, smax, [&](int t) { entries[atomicAdd(hist + t, 1u)] = id; });
+    });
 }
 
 }  // namespace
@@ -327,7 +360,7 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
     // part of its work) with enough of them for kBinSmBlocksMin CTAs; smaller
     // inputs keep the global-atomic kernels, which spread over all SMs
     int sm_blocks = 0;
-    const size_t hsm = sizeof(uint32_t) * (size_t)ntiles;
+    const size_t hsm = sizeof(uint32_t) * (size_t)((ntiles + 3) / 4 * 4);
     if (ntiles <= kBinSmTilesMax && nvis >= (int64_t)kBinSmBlocksMin * ntiles) {
         int dev = 0, nsm = 0, c_sm = 0, s_sm = 0;
         cudaGetDevice(&dev);
