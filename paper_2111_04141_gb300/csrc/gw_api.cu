@@ -384,17 +384,23 @@ struct StageTimer {
     }
 };
 
+IndexBins index_bins(gw_plan p, const BinGeom& geom) {
+    return IndexBins{geom, p->desc.n_wplanes, p->desc.support_min, p->desc.support_max, &p->sc};
+}
+
 // Index + bin one chunk of rows; leaves records and bins in the plan scratch.
 gw_status index_and_bin(gw_plan p, const double* uvw, const double* freq, int64_t nrow, int nchan,
                         const BinGeom& geom, cudaStream_t s) {
+    const IndexBins ib = index_bins(p, geom);
+    bool counted;
     {
         StageTimer t(p, kStIndex, s);
-        launch_index(uvw, freq, nrow, nchan, p->ip, p->sc.rec, p->sc.dropped, s);
+        counted = launch_index(uvw, freq, nrow, nchan, p->ip, p->sc.rec, p->sc.dropped, s, nullptr, &ib);
     }
     {
         StageTimer t(p, kStBin, s);
         launch_bin(p->sc.rec, nrow * (int64_t)nchan, geom, p->desc.n_wplanes,
-                   p->desc.support_min, p->desc.support_max, p->sc, s);
+                   p->desc.support_min, p->desc.support_max, p->sc, s, DevCount{}, counted);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "index/bin launch");
@@ -1409,14 +1415,17 @@ gw_status gw_grid_vis_wstack(gw_plan p, const double* uvw_m, const double* freq_
     for (int64_t r0 = 0; r0 < nrow && nchan > 0; r0 += rpc) {
         const int64_t nr = std::min(rpc, nrow - r0);
         const int64_t v0 = r0 * nchan;
+        const IndexBins ib{g, 1, p->desc.support_min, p->desc.support_min, &sc};
+        bool counted;
         {
             StageTimer t(p, kStIndex, s);
-            launch_index(uvw_m + 3 * r0, freq_hz, nr, nchan, ip, sc.rec, sc.dropped, s);
+            counted = launch_index(uvw_m + 3 * r0, freq_hz, nr, nchan, ip, sc.rec, sc.dropped, s,
+                                   nullptr, &ib);
         }
         {
             StageTimer t(p, kStBin, s);
             launch_bin(sc.rec, nr * (int64_t)nchan, g, 1, p->desc.support_min,
-                       p->desc.support_min, sc, s);
+                       p->desc.support_min, sc, s, DevCount{}, counted);
         }
         GridArgs a;
         a.rec = sc.rec;
@@ -1706,9 +1715,11 @@ gw_status gw_grid_vis_devcount(gw_plan p, const double* uvw_m, const double* fre
     cudaError_t e = cudaMemsetAsync(p->sc.dropped, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     const DevCount dc{d_nrow, nchan};
-    launch_index(uvw_m, freq_hz, max_nrow, nchan, p->ip, p->sc.rec, p->sc.dropped, s, d_nrow);
+    const IndexBins ib = index_bins(p, p->geom_grid);
+    const bool counted = launch_index(uvw_m, freq_hz, max_nrow, nchan, p->ip, p->sc.rec,
+                                      p->sc.dropped, s, d_nrow, &ib);
     launch_bin(p->sc.rec, max_nrow * (int64_t)nchan, p->geom_grid, p->desc.n_wplanes,
-               p->desc.support_min, p->desc.support_max, p->sc, s, dc);
+               p->desc.support_min, p->desc.support_max, p->sc, s, dc, counted);
     GridArgs a;
     a.rec = p->sc.rec;
     a.ptable = p->ptable;
@@ -1787,9 +1798,11 @@ gw_status gw_grid_vis_devcount_readback(gw_plan p, const double* uvw_m, const do
         e = cudaMemsetAsync(p->sc.dropped, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
         const DevCount dc{d_nrow, nchan};
-        launch_index(uvw_m, freq_hz, max_nrow, nchan, p->ip, p->sc.rec, p->sc.dropped, s, d_nrow);
+        const IndexBins ib = index_bins(p, p->geom_grid);
+        const bool counted = launch_index(uvw_m, freq_hz, max_nrow, nchan, p->ip, p->sc.rec,
+                                          p->sc.dropped, s, d_nrow, &ib);
         launch_bin(p->sc.rec, max_nrow * (int64_t)nchan, p->geom_grid, p->desc.n_wplanes,
-                   p->desc.support_min, p->desc.support_max, p->sc, s, dc);
+                   p->desc.support_min, p->desc.support_max, p->sc, s, dc, counted);
     }
     GridArgs a;
     a.rec = p->sc.rec;
@@ -1854,9 +1867,11 @@ gw_status gw_degrid_vis_devcount(gw_plan p, const double* uvw_m, const double* f
     launch_zero_vis(vis_out, vk, nmax, npol, dc, s);
     const bool staged = p->tuning.degrid_kernel != 2;
     const BinGeom& geom = staged ? p->geom_staged : p->geom_degrid;
-    launch_index(uvw_m, freq_hz, max_nrow, nchan, p->ip, p->sc.rec, p->sc.dropped, s, d_nrow);
+    const IndexBins ib = index_bins(p, geom);
+    const bool counted = launch_index(uvw_m, freq_hz, max_nrow, nchan, p->ip, p->sc.rec,
+                                      p->sc.dropped, s, d_nrow, &ib);
     launch_bin(p->sc.rec, nmax, geom, p->desc.n_wplanes, p->desc.support_min,
-               p->desc.support_max, p->sc, s, dc);
+               p->desc.support_max, p->sc, s, dc, counted);
     DegridArgs a;
     a.rec = p->sc.rec;
     a.grid = reinterpret_cast<const float2*>(grid);
@@ -1916,9 +1931,11 @@ gw_status gw_degrid_vis_static(gw_plan p, const double* uvw_m, const double* fre
         e = cudaMemsetAsync(vis_out, 0, (size_t)dtype_bytes(p->desc.vis_dtype) * nvis * p->desc.npol, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     if (nvis > 0) {
-        launch_index(uvw_m, freq_hz, nrow, nchan, p->ip, sc.rec, sc.dropped, s);
+        const IndexBins ib{g, p->desc.n_wplanes, p->desc.support_min, p->desc.support_max, &sc};
+        const bool counted = launch_index(uvw_m, freq_hz, nrow, nchan, p->ip, sc.rec, sc.dropped, s,
+                                          nullptr, &ib);
         launch_bin(sc.rec, nvis, g, p->desc.n_wplanes, p->desc.support_min, p->desc.support_max,
-                   sc, s);
+                   sc, s, DevCount{}, counted);
         DegridArgs a;
         a.rec = sc.rec;
         a.grid = reinterpret_cast<const float2*>(grid);

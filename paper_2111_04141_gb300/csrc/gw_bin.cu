@@ -17,26 +17,6 @@ namespace gw {
 
 namespace {
 
-struct TileRange {
-    int tu0, tu1, tv0, tv1;
-};
-
-__device__ __forceinline__ TileRange tile_range(const gw_index_rec& r, const BinGeom& g, int P,
-                                                int smin, int smax) {
-    TileRange t;
-    if (g.mode == 1) {
-        t.tu0 = t.tu1 = r.ku >> g.su;
-        t.tv0 = t.tv1 = r.kv >> g.sv;
-    } else {
-        const int h = plane_support(r.plane, P, smin, smax) / 2;
-        t.tu0 = (r.ku - h) >> g.su;
-        t.tu1 = (r.ku + h) >> g.su;
-        t.tv0 = (r.kv - h) >> g.sv;
-        t.tv1 = (r.kv + h) >> g.sv;
-    }
-    return t;
-}
-
 __device__ __forceinline__ gw_index_rec load_rec(const gw_index_rec* rec, int64_t i) {
     int4 v = __ldg(reinterpret_cast<const int4*>(rec) + i);
     return *reinterpret_cast<gw_index_rec*>(&v);
@@ -236,13 +216,6 @@ __global__ void k_scatter(const gw_index_rec* __restrict__ rec, int64_t nvis, De
 // memory, one atomic each.  The scatter recounts its chunk, reserves one run
 // per (CTA, tile) in the tile's bin with a single global atomic, and places
 // the entries with shared-memory cursors that start at the run bases.
-constexpr int kBinSmThreads = 1024;
-constexpr int kBinSmTilesMax = 49152;     // 192 KB of u32 counters
-// Fewest CTAs worth it, at one CTA per ntiles records.  255 k records over
-// 16,384 tiles (15 CTAs) bin in 115 us with shared histograms and 55 us with
-// global atomics, 1.03 M over 32,768 (31 CTAs) in 290 and 120; 3.1 M over
-// 32,768 (95 CTAs) in 300 and 500, 30 k over 512 (59 CTAs) in 24 and 39.
-constexpr int kBinSmBlocksMin = 48;
 
 // Work on the records [c0, c1) of a CTA, kBinIlp loads of a thread in flight:
 // one at a time with 512 threads, the loads' latency bounded these kernels (bin
@@ -267,21 +240,6 @@ __device__ __forceinline__ void each_record(const gw_index_rec* __restrict__ rec
         for (int k = 0; k < kBinIlp; ++k)
             if (r[k].flags & GW_FLAG_VALID) f(r[k], (uint32_t)(i0 + k * kBinSmThreads));
     }
-}
-
-// Calls f with the bin of each tile that a record meets.
-template <class F>
-__device__ __forceinline__ void each_bin(const gw_index_rec& r, const BinGeom& g, int P, int smin,
-                                         int smax, F f) {
-    const TileRange t = tile_range(r, g, P, smin, smax);
-    const int lbase = g.layer_tiles ? (r.plane / g.group_planes) * g.layer_tiles : 0;
-    for (int tv = t.tv0; tv <= t.tv1; ++tv)
-        for (int tu = t.tu0; tu <= t.tu1; ++tu) f(lbase + tv * g.ntu + tu);
-}
-
-__device__ __forceinline__ void clear_hist(uint32_t* hist, int ntiles) {
-    for (int t = threadIdx.x * 4; t < ntiles; t += 4 * kBinSmThreads)
-        *reinterpret_cast<uint4*>(hist + t) = make_uint4(0u, 0u, 0u, 0u);
 }
 
 __global__ void __launch_bounds__(kBinSmThreads) k_count_sm(
@@ -352,16 +310,16 @@ __global__ void __launch_bounds__(kBinSmThreads) k_scatter_sm(
 }  // namespace
 
 void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, int smin, int smax,
-                Scratch& sc, cudaStream_t s, DevCount dc) {
-    const int ntiles = g.ntu * g.ntv * (g.layer_tiles ? g.nlayers : 1);
-    cudaMemsetAsync(sc.count, 0, sizeof(uint32_t) * ntiles, s);
+                Scratch& sc, cudaStream_t s, DevCount dc, bool counted) {
+    const int ntiles = bin_count(g);
+    if (!counted) cudaMemsetAsync(sc.count, 0, sizeof(uint32_t) * ntiles, s);
     // per-CTA shared histograms when the bins fit and every CTA has at
     // least ntiles records (zeroing and flushing its histogram stays a small
     // part of its work) with enough of them for kBinSmBlocksMin CTAs; smaller
     // inputs keep the global-atomic kernels, which spread over all SMs
     int sm_blocks = 0;
     const size_t hsm = sizeof(uint32_t) * (size_t)((ntiles + 3) / 4 * 4);
-    if (ntiles <= kBinSmTilesMax && nvis >= (int64_t)kBinSmBlocksMin * ntiles) {
+    if (bin_in_shared(nvis, ntiles)) {
         int dev = 0, nsm = 0, c_sm = 0, s_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -376,7 +334,7 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
     int64_t blocks = (nvis + threads - 1) / threads;
     if (blocks > current_sm_count() * 8) blocks = current_sm_count() * 8;
     if (blocks < 1) blocks = 1;
-    if (nvis > 0) {
+    if (nvis > 0 && !counted) {
         if (sm_blocks > 0)
             k_count_sm<<<sm_blocks, kBinSmThreads, hsm, s>>>(rec, nvis, dc, g, P, smin, smax, ntiles,
                                                              sc.count, sc.work);

@@ -278,11 +278,6 @@ struct DevCount {
     }
 };
 
-// ---- index stage (gw_index.cu) --------------------------------------------
-void launch_index(const double* uvw, const double* freq, int64_t nrow, int nchan,
-                  const IndexParams& prm, gw_index_rec* out, unsigned long long* dropped,
-                  cudaStream_t s, const int64_t* d_nrow = nullptr);
-
 // ---- binner (gw_bin.cu) ----------------------------------------------------
 // mode 0: footprint tiles (every tile a record's footprint touches)
 // mode 1: centre tile (the tile holding pixel (ku, kv))
@@ -295,12 +290,77 @@ struct BinGeom {
     int nlayers = 1;       // layers binned when layer_tiles > 0 (ntu * ntv * nlayers tiles)
     int group_planes = 1;  // planes per layer: 1 for w-stacking layers, more for plane groups
 };
+inline int bin_count(const BinGeom& g) {
+    return g.ntu * g.ntv * (g.layer_tiles ? g.nlayers : 1);
+}
+
+// Tiles [tu0, tu1] x [tv0, tv1] that a record is binned into.
+struct TileRange {
+    int tu0, tu1, tv0, tv1;
+};
+
+__device__ __forceinline__ TileRange tile_range(const gw_index_rec& r, const BinGeom& g, int P,
+                                                int smin, int smax) {
+    TileRange t;
+    if (g.mode == 1) {
+        t.tu0 = t.tu1 = r.ku >> g.su;
+        t.tv0 = t.tv1 = r.kv >> g.sv;
+    } else {
+        const int h = plane_support(r.plane, P, smin, smax) / 2;
+        t.tu0 = (r.ku - h) >> g.su;
+        t.tu1 = (r.ku + h) >> g.su;
+        t.tv0 = (r.kv - h) >> g.sv;
+        t.tv1 = (r.kv + h) >> g.sv;
+    }
+    return t;
+}
+
+// Calls f with the bin of each tile that a record meets.
+template <class F>
+__device__ __forceinline__ void each_bin(const gw_index_rec& r, const BinGeom& g, int P, int smin,
+                                         int smax, F f) {
+    const TileRange t = tile_range(r, g, P, smin, smax);
+    const int lbase = g.layer_tiles ? (r.plane / g.group_planes) * g.layer_tiles : 0;
+    for (int tv = t.tv0; tv <= t.tv1; ++tv)
+        for (int tu = t.tu0; tu <= t.tu1; ++tu) f(lbase + tv * g.ntu + tu);
+}
+
+// Histograms in shared memory: CTAs of kBinSmThreads threads.
+constexpr int kBinSmThreads = 1024;
+constexpr int kBinSmTilesMax = 49152;     // 192 KB of u32 counters
+// Fewest CTAs worth it, at one CTA per ntiles records.  255 k records over
+// 16,384 tiles (15 CTAs) bin in 115 us with shared histograms and 55 us with
+// global atomics, 1.03 M over 32,768 (31 CTAs) in 290 and 120; 3.1 M over
+// 32,768 (95 CTAs) in 300 and 500, 30 k over 512 (59 CTAs) in 24 and 39.
+constexpr int kBinSmBlocksMin = 48;
+inline bool bin_in_shared(int64_t nvis, int ntiles) {
+    return ntiles <= kBinSmTilesMax && nvis >= (int64_t)kBinSmBlocksMin * ntiles;
+}
+
+__device__ __forceinline__ void clear_hist(uint32_t* hist, int ntiles) {
+    for (int t = threadIdx.x * 4; t < ntiles; t += 4 * kBinSmThreads)
+        *reinterpret_cast<uint4*>(hist + t) = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// ---- index stage (gw_index.cu) --------------------------------------------
+// With `bins` the records are also counted into their bins where that saves a
+// kernel; it then returns true, which launch_bin is told.
+struct IndexBins {
+    BinGeom g;
+    int P, smin, smax;
+    Scratch* sc;
+};
+bool launch_index(const double* uvw, const double* freq, int64_t nrow, int nchan,
+                  const IndexParams& prm, gw_index_rec* out, unsigned long long* dropped,
+                  cudaStream_t s, const int64_t* d_nrow = nullptr, const IndexBins* bins = nullptr);
+
+// ---- binner launches (gw_bin.cu) -------------------------------------------
 // Words of Scratch::scan_tmp for a multi-CTA scan over ntiles bins.
 int64_t scan_tmp_words(int64_t ntiles);
 // Also accumulates sc.work[0] += valid records, sc.work[1] += sum of S_p^2.
 // Work items are written only when sc.items is non-null.
 void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, int smin, int smax,
-                Scratch& sc, cudaStream_t s, DevCount dc = DevCount{});
+                Scratch& sc, cudaStream_t s, DevCount dc = DevCount{}, bool counted = false);
 
 // ---- kernel tables (gw_tables.cu) -----------------------------------------
 struct TableBuild {
