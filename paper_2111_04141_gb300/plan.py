@@ -202,7 +202,9 @@ class Plan:
         if weight is not None:
             _need(weight, "weight", torch.float32, self.device, (nrow, nchan, self.npol))
         gshape = (self.npol, self.grid_n, self.grid_n)
-        fresh = out is None and err is None      # cleared by the library, on the stream
+        # cleared by the library, on the current stream (a grid for another stream
+        # is cleared on the one that allocates it)
+        fresh = out is None and err is None and stream is None
         if fresh:
             out = torch.empty(gshape, dtype=torch.complex64, device=self.device)
         else:
