@@ -40,8 +40,8 @@ FFMA_PER_SM_PER_CLK = 128
 
 # DRAM traffic of the gridding kernel from one ncu capture, valid only for the
 # kernel source it was taken on (sha256 of gw_grid_kernel.cuh); null otherwise.
-GRID_TRAFFIC = {"sha256": "1ee91684f8fa3ecd5a1cc714157b1691bdf3c0bbce0a8d1c95030106c9a3d36f",
-                "bytes_per_launch": 0.964303e9 + 0.264140e9,
+GRID_TRAFFIC = {"sha256": "7f1d6b08e8ace1744f53a0b6c51b489ff5bf98e59b2c4261b42e85713275b78b",
+                "bytes_per_launch": 0.963154e9 + 0.264228e9,
                 "capture": "profiles/k_grid_wproj4096.md"}
 
 

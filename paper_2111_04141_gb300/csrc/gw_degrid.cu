@@ -21,18 +21,18 @@
 //   consecutive taps of the S x S footprint (flattened, so every lane is
 //   busy), with kernel values loaded four steps ahead, packed FP32x2 FMAs
 //   (plain ones for one polarisation) into K.re G and K.im G sums, and a
-//   reduce-scatter over the lanes.  A step of 32 taps is 11 (one
-//   polarisation) to 19 (four) instructions: the column and the region offset
-//   advance in one register.  4.2 M visibilities x 1, support 31: 3.00 ms with
-//   23 instructions a step and the pitch padded mod 8, 2.41 now.
+//   reduce-scatter over the lanes.  The tap column and the region offset
+//   advance in one register.  4.2 M visibilities x 1, support 31 (31 steps of 32
+//   taps): 3.00 ms with 714 instructions a record and the pitch padded mod 8,
+//   2.40 with 550.
 //   A region larger than the shared memory is served in bands of rows: every
 //   record sums the tap rows in the band, and its sums wait in shared memory
 //   for the next one.  (Read through L1/L2 instead, 32 B a tap, 1.04 M
 //   visibilities x 4 polarisations with supports to 127 on an 8192^2 grid took
 //   13.2 ms; in bands they take 3.0, the same items read in place where few
-//   taps share a region 5.2.)  The L1 data pipe bounds it (84 % on the 4-pol
-//   w-projection batch, 8.95 ms: 16-byte loads of staged points); before
-//   these instructions were cut 32 warps of 64 registers beat 24 of 80 there,
+//   taps share a region 5.2.)  The L1 data pipe bounds it (90 % on the 4-pol
+//   w-projection batch, 8.94 ms: 16-byte loads of staged points); before
+//   its instructions were cut 32 warps of 64 registers beat 24 of 80 there,
 //   9.34 against 9.52 ms, and 3.28 against 3.63 in bands.
 // * k_degrid_direct (small calls): one launch, index records included.
 // * k_degrid (the allocation-free entry point): the same per-record warp,
