@@ -30,6 +30,7 @@ struct CountBins {
     BinGeom g;
     int P, smin, smax, ntiles;
     uint32_t* count;
+    uint32_t* cursor;            // cleared with COUNT 2
     unsigned long long* work;    // valid records, sum of S^2
 };
 
@@ -55,7 +56,10 @@ __global__ void __launch_bounds__(COUNT == 2 ? kBinSmThreads : 256)
     for (int j = threadIdx.x; j < nthr; j += blockDim.x) thr[j] = wplane_threshold(j, p);
     // (the tables are padded to 16 bytes)
     uint32_t* hist = reinterpret_cast<uint32_t*>(sh + ((nc + nthr + 1) & ~1));
-    if constexpr (COUNT == 2) clear_hist(hist, cb.ntiles);
+    if constexpr (COUNT == 2) {
+        clear_hist(hist, cb.ntiles);
+        clear_cursors(cb.cursor, cb.ntiles);
+    }
     unsigned long long n_valid = 0, n_taps = 0;
     __syncthreads();
     if (d_nrow) nrow = min(nrow, *d_nrow);     // row count read on the device
@@ -127,7 +131,8 @@ bool launch_index(const double* uvw, const double* freq, int64_t nrow, int nchan
     size_t smem = tables;
     if (bins) {
         const int ntiles = bin_count(bins->g);
-        cb = CountBins{bins->g, bins->P, bins->smin, bins->smax, ntiles, bins->sc->count, bins->sc->work};
+        cb = CountBins{bins->g, bins->P, bins->smin, bins->smax, ntiles, bins->sc->count,
+                       bins->sc->cursor, bins->sc->work};
         mode = 1;
         if (bin_in_shared(nvis, ntiles)) {
             // a CTA per ntiles records at least, as in the binner; where that

@@ -337,6 +337,12 @@ inline bool bin_in_shared(int64_t nvis, int ntiles) {
     return ntiles <= kBinSmTilesMax && nvis >= (int64_t)kBinSmBlocksMin * ntiles;
 }
 
+// Cursors of the bins, by all CTAs of a kernel ahead of the scatter.
+__device__ __forceinline__ void clear_cursors(uint32_t* cursor, int ntiles) {
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x)
+        cursor[t] = 0;
+}
+
 __device__ __forceinline__ void clear_hist(uint32_t* hist, int ntiles) {
     for (int t = threadIdx.x * 4; t < ntiles; t += 4 * kBinSmThreads)
         *reinterpret_cast<uint4*>(hist + t) = make_uint4(0u, 0u, 0u, 0u);
