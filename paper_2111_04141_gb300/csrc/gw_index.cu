@@ -23,6 +23,7 @@ namespace {
 
 constexpr int kChanCache = 1024;   // channel factors kept in shared memory
 constexpr size_t kIndexSmemMax = 227 * 1024;
+constexpr int64_t kIndexGlobalMax = 1 << 19;
 
 // What the records are counted into (COUNT: 0 nothing, 1 the bins' counters, 2 a
 // histogram of the CTA in shared memory, added to them at the end).
@@ -30,7 +31,7 @@ struct CountBins {
     BinGeom g;
     int P, smin, smax, ntiles;
     uint32_t* count;
-    uint32_t* cursor;            // cleared with COUNT 2
+    uint32_t* cursor;            // cleared for the scatter
     unsigned long long* work;    // valid records, sum of S^2
 };
 
@@ -56,10 +57,8 @@ __global__ void __launch_bounds__(COUNT == 2 ? kBinSmThreads : 256)
     for (int j = threadIdx.x; j < nthr; j += blockDim.x) thr[j] = wplane_threshold(j, p);
     // (the tables are padded to 16 bytes)
     uint32_t* hist = reinterpret_cast<uint32_t*>(sh + ((nc + nthr + 1) & ~1));
-    if constexpr (COUNT == 2) {
-        clear_hist(hist, cb.ntiles);
-        clear_cursors(cb.cursor, cb.ntiles);
-    }
+    if constexpr (COUNT == 2) clear_hist(hist, cb.ntiles);
+    if constexpr (COUNT != 0) clear_cursors(cb.cursor, cb.ntiles);
     unsigned long long n_valid = 0, n_taps = 0;
     __syncthreads();
     if (d_nrow) nrow = min(nrow, *d_nrow);     // row count read on the device
@@ -137,7 +136,10 @@ bool launch_index(const double* uvw, const double* freq, int64_t nrow, int nchan
         if (bin_in_shared(nvis, ntiles)) {
             // a CTA per ntiles records at least, as in the binner; where that
             // leaves SMs idle and a thread more than one record, the FP64 work
-            // would wait for it (255 k records, 62 CTAs): counted apart
+            // would wait for it: the counters themselves for moderate numbers
+            // of centre bins (255 k records over 4,096: 43 us for both stages
+            // against 50 counted apart), else counted apart (footprint bins
+            // contend more: 30 k over 512, 36 us with the counters, 29 in CTAs)
             const size_t hsm = sizeof(uint32_t) * (size_t)((ntiles + 3) / 4 * 4);
             int per_sm = 0;
             if (tables + hsm <= kIndexSmemMax &&
@@ -146,7 +148,9 @@ bool launch_index(const double* uvw, const double* freq, int64_t nrow, int nchan
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_index<2>, kBinSmThreads,
                                                               tables + hsm);
             const int64_t b = std::min<int64_t>((int64_t)per_sm * current_sm_count(), nvis / ntiles);
-            mode = b >= current_sm_count() || (b > 0 && nvis <= b * kBinSmThreads) ? 2 : 0;
+            mode = b >= current_sm_count() || (b > 0 && nvis <= b * kBinSmThreads) ? 2
+                   : bins->g.mode == 1 && nvis <= kIndexGlobalMax                 ? 1
+                                                                                  : 0;
             if (mode == 2) {
                 blocks = b;
                 threads = kBinSmThreads;
