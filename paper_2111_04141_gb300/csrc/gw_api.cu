@@ -534,6 +534,12 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
         p->support[q] = plane_support(q, P, desc->support_min, desc->support_max);
         smax_real = std::max(smax_real, p->support[q]);
     }
+    double per_vis = 0.0;
+    for (int q = 0; q < P; ++q) {
+        const double e = p->support[q] - 1;
+        per_vis += (e / kGridTileU + 1) * (e / kGridTileV + 1) / P;
+    }
+    p->geom_grid.per_vis = (float)per_vis;
     p->pad_stride = padded_stride(smax_real);
     p->hmax = smax_real / 2;
     for (int q = 0; q < P; ++q) {

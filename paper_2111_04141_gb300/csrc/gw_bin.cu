@@ -373,12 +373,12 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
     const int ntiles = bin_count(g);
     if (!counted) cudaMemsetAsync(sc.count, 0, sizeof(uint32_t) * ntiles, s);
     // per-CTA shared histograms when the bins fit and every CTA has at
-    // least ntiles records (zeroing and flushing its histogram stays a small
+    // least ntiles pairs of a record and a bin (zeroing and flushing its histogram stays a small
     // part of its work) with enough of them for kBinSmBlocksMin CTAs; smaller
     // inputs keep the global-atomic kernels, which spread over all SMs
     int sm_blocks = 0;
     const size_t hsm = sizeof(uint32_t) * (size_t)((ntiles + 3) / 4 * 4);
-    if (bin_in_shared(nvis, ntiles)) {
+    if (bin_in_shared(nvis, g)) {
         int dev = 0, nsm = 0, c_sm = 0, s_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -389,7 +389,7 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
             &s_sm, ntiles <= kScanFusedMax ? k_scatter_sm<true> : k_scatter_sm<false>, kBinSmThreads, hsm);
         sm_blocks = (int)std::min<int64_t>((int64_t)std::min(c_sm, s_sm) * nsm,
-                                           nvis / ntiles);
+                                           bin_sm_blocks(nvis, g));
     }
     const int threads = 256;
     int64_t blocks = (nvis + threads - 1) / threads;

@@ -133,8 +133,8 @@ bool launch_index(const double* uvw, const double* freq, int64_t nrow, int nchan
         cb = CountBins{bins->g, bins->P, bins->smin, bins->smax, ntiles, bins->sc->count,
                        bins->sc->cursor, bins->sc->work};
         mode = 1;
-        if (bin_in_shared(nvis, ntiles)) {
-            // a CTA per ntiles records at least, as in the binner; where that
+        if (bin_in_shared(nvis, bins->g)) {
+            // a CTA per ntiles pairs at least, as in the binner; where that
             // leaves SMs idle and a thread more than one record, the FP64 work
             // would wait for it: the counters themselves for moderate numbers
             // of centre bins (255 k records over 4,096: 43 us for both stages
@@ -147,7 +147,7 @@ bool launch_index(const double* uvw, const double* freq, int64_t nrow, int nchan
                                      (int)kIndexSmemMax) == cudaSuccess)
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_index<2>, kBinSmThreads,
                                                               tables + hsm);
-            const int64_t b = std::min<int64_t>((int64_t)per_sm * current_sm_count(), nvis / ntiles);
+            const int64_t b = std::min((int64_t)per_sm * current_sm_count(), bin_sm_blocks(nvis, bins->g));
             mode = b >= current_sm_count() || (b > 0 && nvis <= b * kBinSmThreads) ? 2
                    : bins->g.mode == 1 && nvis <= kIndexGlobalMax                 ? 1
                                                                                   : 0;

@@ -289,6 +289,7 @@ struct BinGeom {
     int layer_tiles = 0;   // > 0: tile id += (record.plane / group_planes) * layer_tiles
     int nlayers = 1;       // layers binned when layer_tiles > 0 (ntu * ntv * nlayers tiles)
     int group_planes = 1;  // planes per layer: 1 for w-stacking layers, more for plane groups
+    float per_vis = 1.f;   // bins that a record of the mean plane meets
 };
 inline int bin_count(const BinGeom& g) {
     return g.ntu * g.ntv * (g.layer_tiles ? g.nlayers : 1);
@@ -328,13 +329,18 @@ __device__ __forceinline__ void each_bin(const gw_index_rec& r, const BinGeom& g
 // Histograms in shared memory: CTAs of kBinSmThreads threads.
 constexpr int kBinSmThreads = 1024;
 constexpr int kBinSmTilesMax = 49152;     // 192 KB of u32 counters
-// Fewest CTAs worth it, at one CTA per ntiles records.  255 k records over
-// 16,384 tiles (15 CTAs) bin in 115 us with shared histograms and 55 us with
-// global atomics, 1.03 M over 32,768 (31 CTAs) in 290 and 120; 3.1 M over
-// 32,768 (95 CTAs) in 300 and 500, 30 k over 512 (59 CTAs) in 24 and 39.
+// CTAs that get at least as many (record, bin) pairs as there are bins, and the
+// fewest of them worth it.  255 k pairs over 16,384 bins (15 CTAs) bin in 115 us
+// with shared histograms and 55 us with global atomics, 1.2 M over 32,768 (38
+// CTAs) in 290 and 120; 63 k over 512 (124 CTAs) in 24 and 39, 218 k over 1,568
+// (139 CTAs; 41 k records of supports to 109) in 30 and 109
+// together with the index stage.
 constexpr int kBinSmBlocksMin = 48;
-inline bool bin_in_shared(int64_t nvis, int ntiles) {
-    return ntiles <= kBinSmTilesMax && nvis >= (int64_t)kBinSmBlocksMin * ntiles;
+inline int64_t bin_sm_blocks(int64_t nvis, const BinGeom& g) {
+    return (int64_t)((double)nvis * g.per_vis / bin_count(g));
+}
+inline bool bin_in_shared(int64_t nvis, const BinGeom& g) {
+    return bin_count(g) <= kBinSmTilesMax && bin_sm_blocks(nvis, g) >= kBinSmBlocksMin;
 }
 
 // Cursors of the bins, by all CTAs of a kernel ahead of the scatter.
