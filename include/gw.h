@@ -135,7 +135,8 @@ typedef struct {
                                of the call; staged degridding: 1024), else 64 .. 2^20
                                (smaller items spread small jobs over more SMs, larger
                                ones commit less often) */
-    int32_t degrid_kernel;  /* 0 = automatic, 1 = shared-memory staged, 2 = global gather */
+    int32_t degrid_kernel;  /* 0 = automatic (small chunks directly, in one launch, else
+                               staged), 1 = shared-memory staged, 2 = global gather */
     int32_t grid_kernel;    /* gw_grid_vis / _compensated: 0 = automatic (direct for chunks of
                                at most 16,384 visibilities and 2^22 tap updates, else
                                binned), 1 = binned register-tile gridder, 2 = direct

@@ -134,6 +134,7 @@ struct gw_plan_s {
     int max_groups = 1;  // plane groups the bins are allocated for (gw_tuning.plane_groups)
     int auto_groups = 1; // plane groups chosen when plane_groups = 0
     int pad_stride = 0;
+    double mean_s2 = 0.0;        // mean S^2 over the planes
     double field = 0, table_scale = 0;
     std::vector<int> support;
     std::vector<double> wplane;
@@ -537,6 +538,7 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
     double per_vis = 0.0;
     for (int q = 0; q < P; ++q) {
         const double e = p->support[q] - 1;
+        p->mean_s2 += (e + 1) * (e + 1) / P;
         per_vis += (e / kGridTileU + 1) * (e / kGridTileV + 1) / P;
     }
     p->geom_grid.per_vis = (float)per_vis;
@@ -750,6 +752,7 @@ gw_status gw_plan_clone(gw_plan src, int64_t max_vis_per_call, void* cuda_stream
     p->max_groups = src->max_groups;
     p->auto_groups = src->auto_groups;
     p->pad_stride = src->pad_stride;
+    p->mean_s2 = src->mean_s2;
     p->field = src->field;
     p->table_scale = src->table_scale;
     p->support = src->support;
@@ -931,16 +934,26 @@ static const BinGeom& staged_geom(gw_plan p, int64_t nvis) {
     return p->geom_staged;
 }
 
-// Inputs small enough that launches dominate: gridded and degridded directly.
+// Taps of nvis visibilities on planes of the mean S^2, in those of one
+// polarisation: each further one costs half of the first.
+static double direct_taps(gw_plan p, int64_t nvis) {
+    return (double)nvis * p->mean_s2 * 0.5 * (1 + p->desc.npol);
+}
+// Direct (unbinned) degridding of small inputs.  Calls, us, staged / direct
+// (support 7-33, mean S^2 456, unless named): 1024^2, 16 k visibilities x 1 72 / 29,
+// x 2 73 / 34, x 4 81 / 59, uv within a tenth of the grid 80 / 29, 30 k x 1 81 / 48, 60 k x
+// 1 92 / 84; 4096^2 x 1, 60 k 132 / 87; support 31, 8 k x 4 118 / 80; support 7-63, 16 k x 1
+// 84 / 43; beyond the line 30 k x 4 92 / 88, support 7-63, 16 k x 4 112 / 150.
 static bool direct_size(gw_plan p, int64_t nvis) {
-    const int64_t smax = p->support.empty() ? 1 : p->support.back();
-    return nvis <= kDirectMaxVis && nvis * smax * smax * p->desc.npol <= kDirectMaxTaps;
+    return nvis <= kDirectDegridVis && direct_taps(p, nvis) <= kDirectDegridTaps;
 }
 // Direct (unbinned) gridding of a chunk of nvis visibilities: forced by the
 // tuning, or automatic for small inputs.
 static bool use_direct(gw_plan p, int64_t nvis) {
     if (p->tuning.grid_kernel == 1) return false;
-    return p->tuning.grid_kernel == 2 || direct_size(p, nvis);
+    const int64_t smax = p->support.empty() ? 1 : p->support.back();
+    return p->tuning.grid_kernel == 2 ||
+           (nvis <= kDirectMaxVis && nvis * smax * smax * p->desc.npol <= kDirectMaxTaps);
 }
 
 static void set_pairs(GridArgs& a, gw_plan p) {

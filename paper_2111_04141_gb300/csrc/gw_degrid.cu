@@ -159,9 +159,11 @@ __global__ void __launch_bounds__(kThreads) k_degrid_direct(DegridArgs a, Direct
         rv.z = __shfl_sync(0xffffffffu, rv.z, 0);
         rv.w = __shfl_sync(0xffffffffu, rv.w, 0);
         const gw_index_rec rc = *reinterpret_cast<const gw_index_rec*>(&rv);
-        float acc[NPOL][2];
+        // K.re G and K.im G apart, as in the staged kernel: half the length of
+        // the chains, and the sums of conj(K_i) at the end
+        float2 a1[NPOL], a2[NPOL];
 #pragma unroll
-        for (int p = 0; p < NPOL; ++p) acc[p][0] = acc[p][1] = 0.f;
+        for (int p = 0; p < NPOL; ++p) a1[p] = a2[p] = make_float2(0.f, 0.f);
         bool valid = (rc.flags & GW_FLAG_VALID) != 0;
         const int S = valid ? __ldg(a.support + rc.plane) : 0, h = S >> 1;
         const int64_t kofs = valid ? __ldg(a.plane_off + rc.plane) +
@@ -181,20 +183,34 @@ __global__ void __launch_bounds__(kThreads) k_degrid_direct(DegridArgs a, Direct
 #endif
         const typename TE::T* K = reinterpret_cast<const typename TE::T*>(a.table) + kofs;
         const float s = (rc.flags & GW_FLAG_CONJ) ? -1.f : 1.f;
+        // tap (tv, tu) = (t / S, t % S), advanced without division
+        const int dq = valid ? 32 / S : 0, dr = 32 - dq * S;
+        int tv = valid ? lane / S : 0, tu = lane - tv * S;
+#pragma unroll 4
         for (int t = lane; t < S * S; t += 32) {
-            const int tv = t / S, tu = t - tv * S;
             const float2 k = TE::load(K + t);
-            const float ki = s * k.y;
             const int64_t pix = (int64_t)(rc.kv - h + tv) * N + (rc.ku - h + tu);
 #pragma unroll
             for (int p = 0; p < NPOL; ++p) {
                 const float2 g = __ldg(a.grid + (int64_t)p * N * N + pix);
-                // (k.x - j ki) * (g.x + j g.y)
-                acc[p][0] = fmaf(k.x, g.x, acc[p][0]);
-                acc[p][0] = fmaf(ki, g.y, acc[p][0]);
-                acc[p][1] = fmaf(k.x, g.y, acc[p][1]);
-                acc[p][1] = fmaf(-ki, g.x, acc[p][1]);
+                a1[p].x = fmaf(k.x, g.x, a1[p].x);
+                a1[p].y = fmaf(k.x, g.y, a1[p].y);
+                a2[p].x = fmaf(k.y, g.x, a2[p].x);
+                a2[p].y = fmaf(k.y, g.y, a2[p].y);
             }
+            tu += dr;
+            tv += dq;
+            if (tu >= S) {
+                tu -= S;
+                ++tv;
+            }
+        }
+        // (K.re - j s K.im) (G.re + j G.im)
+        float acc[NPOL][2];
+#pragma unroll
+        for (int p = 0; p < NPOL; ++p) {
+            acc[p][0] = fmaf(s, a2[p].y, a1[p].x);
+            acc[p][1] = fmaf(-s, a2[p].x, a1[p].y);
         }
 #pragma unroll
         for (int p = 0; p < NPOL; ++p)

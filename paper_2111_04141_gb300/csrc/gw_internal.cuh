@@ -456,6 +456,9 @@ void launch_grid_direct(const GridArgs& a, const void* table, const DirectIndex&
 // Direct gridding is chosen for at most this many visibilities per chunk and
 // this many tap updates (visibilities x S_max^2 x npol).
 constexpr int64_t kDirectMaxVis = 16384;
+// Direct degridding: visibilities, and taps (visibilities x mean S^2 x (1 + npol) / 2).
+constexpr int64_t kDirectDegridVis = 65536;
+constexpr double kDirectDegridTaps = 33554432.0;
 // Plane groups of the binned gridder: at most this many, chosen
 // automatically when FP32 padded tables exceed kGroupTableBytes (about the
 // L2), with about kGroupTargetBytes of tables per group.

@@ -105,3 +105,19 @@ def test_sparse_inputs_take_large_tiles(gw, npol, n, n_ant, n_times, smin, smax)
     obs = syn.small_case(n_ant=n_ant, n_times=n_times, n_chan=3, npol=npol, grid_n=n, s_min=smin,
                          s_max=smax, n_w=3, beta=4, diameter_m=20.0 * n, seed=37)
     check(gw, obs, bands=smax > 17, degrid_kernel=1)
+
+
+# one launch for small calls against the staged kernel: the same sums in the
+# same order, at supports around a warp's 32 taps and every polarisation count
+@pytest.mark.parametrize("npol,n,smin,smax,n_w", [
+    (1, 130, 1, 1, 1), (2, 98, 5, 7, 2), (3, 142, 31, 33, 3), (4, 300, 5, 65, 4), (1, 600, 41, 255, 3)])
+def test_direct_equals_staged(gw, npol, n, smin, smax, n_w):
+    obs = drop_some(syn.small_case(n_ant=6, n_times=9, n_chan=3, npol=npol, grid_n=n, s_min=smin,
+                                   s_max=smax, n_w=n_w, beta=4, diameter_m=1100.0, seed=43))
+    rng = np.random.default_rng(5)
+    shape = (npol, n, n)
+    grid = (rng.normal(size=shape) + 1j * rng.normal(size=shape)).astype(np.complex64)
+    direct, dropped, _ = degrid(gw, obs, grid, True, degrid_kernel=0)
+    staged, again, _ = degrid(gw, obs, grid, True, degrid_kernel=1)
+    assert dropped == again
+    assert np.linalg.norm(direct - staged) <= 2 * TOL * np.linalg.norm(staged)
