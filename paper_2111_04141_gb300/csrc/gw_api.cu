@@ -860,14 +860,16 @@ static int grid_groups(gw_plan p) {
     const int g = p->tuning.plane_groups > 0 ? p->tuning.plane_groups : p->auto_groups;
     return std::max(1, std::min(g, p->max_groups));
 }
-// Gridder work items of nvis visibilities: shorter ones for smaller inputs,
-// which spread over more SMs (calls, us, with items of 128 / 256 / 512 / 1024
-// records: 30 k x 1 57.5 / 59.0 / 59.8 / 60.2, 121 k x 4 147 / 145 / 148 / 161,
-// 403 k x 2 292 / 272 / 276 / 290, 472 k x 3 427 / 400 / 391 / 395); multiples of
-// 255, which every gridder stages in whole batches.
+// Gridder work items: shorter ones where longer ones would be too few to spread
+// over the SMs (calls, us, with items of 255 / 510 / 1,020 records: 30 k x 1,
+// 1024^2 53.5 / 53.8 / -, 121 k x 4 137 / 140 / 161, 403 k x 2, 512^2 248 / 263 / 290,
+// 472 k x 3 372 / 367 / 395), no shorter, because every item adds its sums to the
+// grid once (relative errors of 893 k x 3 on 376^2: 5.2 / 4.2 / 3.8 e-7).  Multiples
+// of 255, which every gridder stages in whole batches.
 static int grid_items(gw_plan p, int64_t nvis) {
     if (p->tuning.item_max > 0) return p->tuning.item_max;
-    return nvis <= 262144 ? 255 : (nvis <= 1048576 ? 510 : 1020);
+    const double pairs = (double)nvis * p->geom_grid.per_vis;
+    return pairs >= 1020.0 * 8 * p->num_sms ? 1020 : (pairs >= 510.0 * 2.5 * p->num_sms ? 510 : 255);
 }
 static BinGeom grid_geom(gw_plan p, int groups, int64_t nvis) {
     BinGeom g = p->geom_grid;
@@ -941,19 +943,30 @@ static double direct_taps(gw_plan p, int64_t nvis) {
 }
 // Direct (unbinned) degridding of small inputs.  Calls, us, staged / direct
 // (support 7-33, mean S^2 456, unless named): 1024^2, 16 k visibilities x 1 72 / 29,
-// x 2 73 / 34, x 4 81 / 59, uv within a tenth of the grid 80 / 29, 30 k x 1 81 / 48, 60 k x
-// 1 92 / 84; 4096^2 x 1, 60 k 132 / 87; support 31, 8 k x 4 118 / 80; support 7-63, 16 k x 1
-// 84 / 43; beyond the line 30 k x 4 92 / 88, support 7-63, 16 k x 4 112 / 150.
+// x 4 82 / 40, uv within a tenth of the grid x 4 118 / 39, 60 k x 1 93 / 79; 4096^2 x 1, 60 k
+// 132 / 79; 8192^2 x 4, 20 k 519 / 90; support 5, 60 k x 1 81 / 56; beyond the line
+// support 7-63, 16 k x 4 112 / 150 (before the kernel kept four taps in flight).
 static bool direct_size(gw_plan p, int64_t nvis) {
     return nvis <= kDirectDegridVis && direct_taps(p, nvis) <= kDirectDegridTaps;
 }
 // Direct (unbinned) gridding of a chunk of nvis visibilities: forced by the
-// tuning, or automatic for small inputs.
+// tuning, or automatic for small inputs.  The direct gridder's time grows with
+// the taps, the binned one has a fixed part.  Calls of 16,128 visibilities,
+// us, binned / direct: support 7-33 (mean S^2 456) 1024^2 x 1 57 / 39, x 2 63 / 44,
+// x 4 68 / 55, bfloat16 58 / 39, uv within a tenth of the grid 66 / 39, on one pixel
+// 108 / 72; support 31 x 3 73 / 87; support 7-63 (1,486) 72 / 74.  Every tap is added to
+// the grid by itself, so beyond 2^22 taps only where few meet in a pixel
+// (relative errors binned / direct: 5 taps a pixel 1.0 / 0.8 e-7, 237 2.6 / 3.9 e-7).
+// More visibilities gain only on sparse grids, and there not with concentrated
+// uv (60 k x 1 on 4096^2 144 / 116, within 0.3 of it 97 / 116).
 static bool use_direct(gw_plan p, int64_t nvis) {
     if (p->tuning.grid_kernel == 1) return false;
+    if (p->tuning.grid_kernel == 2) return true;
+    if (nvis > kDirectMaxVis) return false;
     const int64_t smax = p->support.empty() ? 1 : p->support.back();
-    return p->tuning.grid_kernel == 2 ||
-           (nvis <= kDirectMaxVis && nvis * smax * smax * p->desc.npol <= kDirectMaxTaps);
+    const double n = (double)p->desc.grid_n;
+    return nvis * smax * smax * p->desc.npol <= kDirectMaxTaps ||
+           (direct_taps(p, nvis) <= kDirectGridTaps && nvis * p->mean_s2 <= kDirectPerPixel * n * n);
 }
 
 static void set_pairs(GridArgs& a, gw_plan p) {

@@ -453,10 +453,14 @@ struct DirectIndex {
 };
 void launch_grid_direct(const GridArgs& a, const void* table, const DirectIndex& di,
                         unsigned long long* work, cudaStream_t s);
-// Direct gridding is chosen for at most this many visibilities per chunk and
-// this many tap updates (visibilities x S_max^2 x npol).
+// Direct gridding is chosen for at most kDirectMaxVis visibilities per chunk and
+// kDirectMaxTaps tap updates (visibilities x S_max^2 x npol), or kDirectGridTaps
+// taps (visibilities x mean S^2 x (1 + npol) / 2) of which kDirectPerPixel meet
+// in a grid point on average; degridding by the second measure alone.
 constexpr int64_t kDirectMaxVis = 16384;
-// Direct degridding: visibilities, and taps (visibilities x mean S^2 x (1 + npol) / 2).
+constexpr int64_t kDirectMaxTaps = (int64_t)1 << 22;
+constexpr double kDirectGridTaps = 16777216.0;
+constexpr double kDirectPerPixel = 8.0;
 constexpr int64_t kDirectDegridVis = 65536;
 constexpr double kDirectDegridTaps = 33554432.0;
 // Plane groups of the binned gridder: at most this many, chosen
@@ -467,7 +471,6 @@ constexpr int64_t kGroupTableBytes = 128ll << 20;
 constexpr int64_t kGroupTargetBytes = 64ll << 20;
 // Bands of tile rows a banded read-back may use (gw_grid_vis_devcount_readback).
 constexpr int kReadbackBandsMax = 64;
-constexpr int64_t kDirectMaxTaps = (int64_t)1 << 22;
 // Staged degridding takes 32 x 32, 64 x 64 and 128 x 128 centre tiles instead
 // of 16 x 16 below this many visibilities per 16 x 16 points on average, 128
 // with supports above 2 kStagedWide128 already below kStagedSparse64.
