@@ -185,6 +185,18 @@ class Plan:
         return torch.empty(vis_shape(self.vis_dtype, nrow, nchan, self.npol),
                            dtype=_TORCH[self.vis_dtype], device=self.device)
 
+    def _for_stream(self, t: torch.Tensor, stream) -> torch.Tensor:
+        """A tensor allocated here (and cleared, where it is) on the current
+        stream, for work on ``stream``: that stream waits for the current one,
+        whose pending work may still use the memory the tensor was given, and
+        the allocator keeps the memory until ``stream`` is done with it."""
+        if stream is not None:
+            here = torch.cuda.current_stream(self.device)
+            if stream.cuda_stream != here.cuda_stream:
+                stream.wait_stream(here)
+                t.record_stream(stream)
+        return t
+
     def new_grid(self) -> torch.Tensor:
         return torch.zeros((self.npol, self.grid_n, self.grid_n), dtype=torch.complex64,
                            device=self.device)
@@ -203,13 +215,13 @@ class Plan:
             _need(weight, "weight", torch.float32, self.device, (nrow, nchan, self.npol))
         gshape = (self.npol, self.grid_n, self.grid_n)
         # cleared by the library, on the current stream (a grid for another stream
-        # is cleared on the one that allocates it)
+        # is cleared on the one that allocates it, which that one waits for)
         fresh = out is None and err is None and stream is None
         if fresh:
             out = torch.empty(gshape, dtype=torch.complex64, device=self.device)
         else:
             if out is None:
-                out = self.new_grid()
+                out = self._for_stream(self.new_grid(), stream)
             _need(out, "grid", torch.complex64, self.device, gshape)
         dropped = ctypes.c_int64(-1)
         dp = ctypes.byref(dropped) if return_dropped else None
@@ -283,7 +295,7 @@ class Plan:
         if weight is not None:
             _need(weight, "weight", torch.float32, self.device, (nrow, nchan, self.npol))
         if out is None:
-            out = self.new_grid()
+            out = self._for_stream(self.new_grid(), stream)
         _need(out, "grid", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
         ng, nd = ctypes.c_int64(-1), ctypes.c_int64(-1)
         with _on(self.device):
@@ -303,7 +315,8 @@ class Plan:
             _need(weight, "weight", torch.float32, self.device, (nrow, nchan, self.npol))
         shape = (int(n_layers), self.npol, self.grid_n, self.grid_n)
         if out is None:
-            out = torch.zeros(shape, dtype=torch.complex64, device=self.device)
+            out = self._for_stream(torch.zeros(shape, dtype=torch.complex64, device=self.device),
+                                   stream)
         _need(out, "layers", torch.complex64, self.device, shape)
         nd = ctypes.c_int64(-1)
         with _on(self.device):
@@ -338,7 +351,8 @@ class Plan:
             _need(weight, "weight", torch.float32, self.device, (nrow, nchan, self.npol))
         shape = self.fine_shape()
         if out is None:
-            out = torch.zeros(shape, dtype=torch.complex64, device=self.device)
+            out = self._for_stream(torch.zeros(shape, dtype=torch.complex64, device=self.device),
+                                   stream)
         _need(out, "fine", torch.complex64, self.device, shape)
         nd = ctypes.c_int64(-1)
         with _on(self.device):
@@ -356,7 +370,8 @@ class Plan:
         shape = (self.npol, 2 * self.grid_n, self.grid_n)
         _need(fine, "fine", torch.complex64, self.device, self.fine_shape())
         if out is None:
-            out = torch.empty(shape, dtype=torch.complex64, device=self.device)
+            out = self._for_stream(torch.empty(shape, dtype=torch.complex64, device=self.device),
+                                   stream)
         _need(out, "pruned", torch.complex64, self.device, shape)
         with _on(self.device):
             check(self._lib.gw_hybrid_prune(self._h, int(sz), _ptr(fine), _ptr(out),
@@ -374,7 +389,7 @@ class Plan:
     def hybrid_image(self, sz, raw, out=None, stream=None):
         _need(raw, "raw", torch.complex64, self.device, (self.npol, 2 * self.grid_n, self.grid_n))
         if out is None:
-            out = self.new_grid()
+            out = self._for_stream(self.new_grid(), stream)
         _need(out, "image", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
         with _on(self.device):
             check(self._lib.gw_hybrid_image(self._h, int(sz), _ptr(raw), _ptr(out),
@@ -404,7 +419,7 @@ class Plan:
         if weight is not None:
             host(weight, "weight", torch.float32)
         if out is None:
-            out = self.new_grid()
+            out = self._for_stream(self.new_grid(), stream)
         _need(out, "grid", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
         nd = ctypes.c_int64(-1)
         with _on(self.device):
@@ -430,7 +445,7 @@ class Plan:
         nrow, nchan = self._coords(uvw, freq)
         _need(grid, "grid", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
         if out is None:
-            out = self.new_vis(nrow, nchan)
+            out = self._for_stream(self.new_vis(nrow, nchan), stream)
         out = self._vis_arg(out, "vis_out", nrow, nchan)
         dropped = ctypes.c_int64(-1)
         with _on(self.device):
@@ -451,7 +466,7 @@ class Plan:
         nrow, nchan = self._coords(uvw, freq)
         _need(grid, "grid", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
         if out is None:
-            out = self.new_vis(nrow, nchan)
+            out = self._for_stream(self.new_vis(nrow, nchan), stream)
         out = self._vis_arg(out, "vis_out", nrow, nchan)
         dropped = ctypes.c_int64(-1)
         with _on(self.device):
@@ -482,8 +497,6 @@ class Plan:
         _need(image, "image", torch.complex64, self.device, (self.npol, self.grid_n, self.grid_n))
         if scale_dev is not None:
             _need(scale_dev, "scale_dev", torch.float32, self.device, (self.npol,))
-            if stream is not None:
-                scale_dev.record_stream(stream)
         with _on(self.device):
             check(self._lib.gw_image_finish(self._h, _ptr(image), float(scale), _ptr(scale_dev),
                                             _stream_ptr(stream, self.device)), "gw_image_finish")
@@ -495,7 +508,8 @@ class Plan:
         Column 0 = ku, 1 = kv, 2 = (ou & 0xffff) | (ov << 16), 3 = plane | flags << 16.
         """
         nrow, nchan = self._coords(uvw, freq)
-        out = torch.empty((nrow * nchan, 4), dtype=torch.int32, device=self.device)
+        out = self._for_stream(torch.empty((nrow * nchan, 4), dtype=torch.int32,
+                                           device=self.device), stream)
         dropped = ctypes.c_int64(-1)
         with _on(self.device):
             check(self._lib.gw_index_vis(self._h, _ptr(uvw), _ptr(freq), nrow, nchan, _ptr(out),
