@@ -138,9 +138,8 @@ typedef struct {
     int32_t degrid_kernel;  /* 0 = automatic (small chunks directly, in one launch, else
                                staged), 1 = shared-memory staged, 2 = global gather */
     int32_t grid_kernel;    /* gw_grid_vis / _compensated: 0 = automatic (direct for chunks of
-                               at most 16,384 visibilities and 2^22 tap updates, or up
-                               to 2^24 where few meet in a pixel, else binned),
-                               1 = binned register-tile gridder, 2 = direct
+                               at most 16,384 visibilities and 2^22 tap updates, else
+                               binned), 1 = binned register-tile gridder, 2 = direct
                                (one global atomic per tap and polarisation, no bins) */
     int32_t compress_min_gain; /* gw_grid_vis_compressed: 0 = always compress; g in
                                1..1000 = first compress a sample (the first rows, up to

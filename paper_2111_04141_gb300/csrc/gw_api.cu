@@ -951,22 +951,18 @@ static bool direct_size(gw_plan p, int64_t nvis) {
 }
 // Direct (unbinned) gridding of a chunk of nvis visibilities: forced by the
 // tuning, or automatic for small inputs.  The direct gridder's time grows with
-// the taps, the binned one has a fixed part.  Calls of 16,128 visibilities,
-// us, binned / direct: support 7-33 (mean S^2 456) 1024^2 x 1 57 / 39, x 2 63 / 44,
-// x 4 68 / 55, bfloat16 58 / 39, uv within a tenth of the grid 66 / 39, on one pixel
-// 108 / 72; support 31 x 3 73 / 87; support 7-63 (1,486) 72 / 74.  Every tap is added to
-// the grid by itself, so beyond 2^22 taps only where few meet in a pixel
-// (relative errors binned / direct: 5 taps a pixel 1.0 / 0.8 e-7, 237 2.6 / 3.9 e-7).
-// More visibilities gain only on sparse grids, and there not with concentrated
-// uv (60 k x 1 on 4096^2 144 / 116, within 0.3 of it 97 / 116).
+// the taps, the binned one has a fixed part (3,840 x 1, support 7, 256^2: 12 / 30 us),
+// but every tap is added to the grid by itself where the binned one sums up to
+// an item's records first, so where many meet in a pixel its error is the larger
+// one (relative errors binned / direct of 16,128 x 1, support 7-33: 2.6 / 3.9 e-7
+// with 237 taps a pixel).  How many meet is not known on the host, so the line
+// is no higher than 2^22 taps of the widest support, although calls of 2^24
+// gain (the same on 1024^2: 57 / 39 us, 5 taps a pixel, 1.0 / 0.8 e-7).
 static bool use_direct(gw_plan p, int64_t nvis) {
     if (p->tuning.grid_kernel == 1) return false;
-    if (p->tuning.grid_kernel == 2) return true;
-    if (nvis > kDirectMaxVis) return false;
     const int64_t smax = p->support.empty() ? 1 : p->support.back();
-    const double n = (double)p->desc.grid_n;
-    return nvis * smax * smax * p->desc.npol <= kDirectMaxTaps ||
-           (direct_taps(p, nvis) <= kDirectGridTaps && nvis * p->mean_s2 <= kDirectPerPixel * n * n);
+    return p->tuning.grid_kernel == 2 ||
+           (nvis <= kDirectMaxVis && nvis * smax * smax * p->desc.npol <= kDirectMaxTaps);
 }
 
 static void set_pairs(GridArgs& a, gw_plan p) {

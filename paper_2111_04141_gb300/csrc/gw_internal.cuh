@@ -453,14 +453,11 @@ struct DirectIndex {
 };
 void launch_grid_direct(const GridArgs& a, const void* table, const DirectIndex& di,
                         unsigned long long* work, cudaStream_t s);
-// Direct gridding is chosen for at most kDirectMaxVis visibilities per chunk and
-// kDirectMaxTaps tap updates (visibilities x S_max^2 x npol), or kDirectGridTaps
-// taps (visibilities x mean S^2 x (1 + npol) / 2) of which kDirectPerPixel meet
-// in a grid point on average; degridding by the second measure alone.
+// Direct gridding is chosen for at most this many visibilities per chunk and
+// this many tap updates (visibilities x S_max^2 x npol).
 constexpr int64_t kDirectMaxVis = 16384;
 constexpr int64_t kDirectMaxTaps = (int64_t)1 << 22;
-constexpr double kDirectGridTaps = 16777216.0;
-constexpr double kDirectPerPixel = 8.0;
+// Direct degridding: visibilities, and taps (visibilities x mean S^2 x (1 + npol) / 2).
 constexpr int64_t kDirectDegridVis = 65536;
 constexpr double kDirectDegridTaps = 33554432.0;
 // Plane groups of the binned gridder: at most this many, chosen
