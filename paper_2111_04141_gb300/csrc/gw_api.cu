@@ -347,7 +347,7 @@ gw_status alloc_scratch(gw_plan p) {
 // Work-item size and degridding kernel choice of a plan (gw_plan_set_tuning).
 void apply_tuning(gw_plan p) {
     const int im = p->tuning.item_max > 0 ? p->tuning.item_max : kItemMax;
-    p->geom_grid.item_max = im;
+    p->geom_grid.item_max = p->tuning.item_max > 0 ? p->tuning.item_max : kItemLong;
     p->geom_degrid.item_max = im;
     p->geom_staged.item_max = im;
     p->geom_staged64.item_max = im;

@@ -34,7 +34,9 @@ constexpr int kGridLanesU = GW_GRID_LANES_U;
 constexpr int kGridLanesV = 32 / kGridLanesU;
 constexpr int kGridPadR = kGridLanesV - 1;
 constexpr int kGridPadC = kGridLanesU - 1;
-constexpr int kItemMax = 1024;        // default max bin entries per work item
+constexpr int kItemMax = 1024;        // default max bin entries per staged-degridding work item
+constexpr int kItemLong = 1020;       // the same of a gridding one: whole batches of 255 entries,
+                                      // which every gridder stages
 constexpr int kItemMin = 64;          // smallest work-item size a plan may be tuned to
 
 // Support of plane p: the odd integer nearest
