@@ -860,20 +860,24 @@ static int grid_groups(gw_plan p) {
     const int g = p->tuning.plane_groups > 0 ? p->tuning.plane_groups : p->auto_groups;
     return std::max(1, std::min(g, p->max_groups));
 }
-// Gridder work items: shorter ones where longer ones would be too few to spread
-// over the SMs (calls, us, with items of 255 / 510 / 1,020 records: 30 k x 1,
-// 1024^2 53.5 / 53.8 / -, 121 k x 4 137 / 140 / 161, 403 k x 2, 512^2 248 / 263 / 290,
-// 472 k x 3 372 / 367 / 395), no shorter, because every item adds its sums to the
-// grid once (relative errors of 893 k x 3 on 376^2: 5.2 / 4.2 / 3.8 e-7).  Multiples
-// of 255, which every gridder stages in whole batches.
-static int grid_items(gw_plan p, int64_t nvis) {
-    if (p->tuning.item_max > 0) return p->tuning.item_max;
-    const double pairs = (double)nvis * p->geom_grid.per_vis;
-    return pairs >= 1020.0 * 8 * p->num_sms ? 1020 : (pairs >= 510.0 * 2.5 * p->num_sms ? 510 : 255);
+// Gridder work items of a call whose size the host knows: 1,020 records, but
+// shorter ones where those would be too few to spread over the SMs (calls, us,
+// with items of 255 / 510 / 1,020 records: 31 k x 4, 300^2 69 / 81 / 119, 121 k x 4,
+// 1024^2 135 / 136 / 149, 403 k x 2, 512^2 243 / 256 / 281).
+// Every item adds its sums to the grid once, so bins of many short ones round
+// there more often: relative errors of 564 k x 3 on 376^2 (12,700 entries a bin)
+// 2.7 / 2.3 / 2.3 e-7, of 48 k coherent visibilities in a few tiles 1.8 e-7 with 255
+// and 1.0 e-7 with 1,020.  So no bin is cut into more items than eight or than
+// 1,020 records make (item_limit), whatever the distribution.
+static void set_grid_items(gw_plan p, BinGeom& g, int64_t nvis) {
+    if (p->tuning.item_max > 0) return;
+    const double pairs = (double)nvis * g.per_vis;
+    g.item_max = pairs >= 1020.0 * 8 * p->num_sms ? 1020 : (pairs >= 510.0 * 2.5 * p->num_sms ? 510 : 255);
+    g.item_limit = 8u * (uint32_t)g.item_max;
 }
 static BinGeom grid_geom(gw_plan p, int groups, int64_t nvis) {
     BinGeom g = p->geom_grid;
-    g.item_max = grid_items(p, nvis);
+    set_grid_items(p, g, nvis);
     if (groups > 1) {
         g.layer_tiles = g.ntu * g.ntv;
         g.nlayers = groups;

@@ -50,7 +50,7 @@ __global__ void k_count(const gw_index_rec* __restrict__ rec, int64_t nvis, DevC
     }
 }
 
-// Exclusive scans of count[] -> offsets[] and of ceil(count / item_max) ->
+// Exclusive scans of count[] -> offsets[] and of the bins' work items ->
 // item_off[], with zeroed cursors and the work items, in segments of kScanSeg
 // bins, one CTA each.
 // Up to kScanSingleMax bins one kernel does it: every CTA first sums the bins
@@ -91,16 +91,17 @@ __device__ __forceinline__ void block_excl_scan2(uint32_t& a, uint32_t& b, uint3
 }
 
 // Work items of a warp's 32 bins (the lanes' sizes c, item counts ni, first
-// entries ra and items rb): runs of at most item_max entries.  The warp writes
+// entries ra and items rb).  The warp writes
 // its bins one after another, so that a bin of thousands of items is not one
 // thread's.
 __device__ __forceinline__ void write_items(Item* __restrict__ items, int bin0, int lane, uint32_t c,
                                             uint32_t ni, uint32_t ra, uint32_t rb,
-                                            uint32_t item_max) {
+                                            const ItemRule& rule) {
     for (uint32_t left = __ballot_sync(0xffffffffu, ni != 0); left; left &= left - 1) {
         const int src = __ffs(left) - 1;
         const uint32_t nc = __shfl_sync(0xffffffffu, c, src), nn = __shfl_sync(0xffffffffu, ni, src);
         const uint32_t st = __shfl_sync(0xffffffffu, ra, src), o = __shfl_sync(0xffffffffu, rb, src);
+        const uint32_t item_max = rule.size(nc);
         for (uint32_t k = lane; k < nn; k += 32) {
             Item it;
             it.tile = bin0 + src;
@@ -115,20 +116,19 @@ __device__ __forceinline__ void write_items(Item* __restrict__ items, int bin0, 
 // pass 0: segment totals; pass 1: the rest, from scanned totals; pass 2: all in
 // one kernel.
 __global__ void __launch_bounds__(kScanThreads) k_scan_seg(
-    const uint32_t* __restrict__ count, int n, uint32_t item_max, int pass,
+    const uint32_t* __restrict__ count, int n, ItemRule rule, int pass,
     uint32_t* __restrict__ seg_tot, uint32_t* __restrict__ offsets,
     uint32_t* __restrict__ item_off, uint32_t* __restrict__ cursor, Item* __restrict__ items) {
     __shared__ uint32_t sa[32], sb[32];
     const int s0 = blockIdx.x * kScanSeg, i = s0 + (int)threadIdx.x, lane = threadIdx.x & 31;
-    const uint32_t c = i < n ? count[i] : 0u, ni = (c + item_max - 1) / item_max;
+    const uint32_t c = i < n ? count[i] : 0u, ni = rule.items(c);
     uint32_t ra = 0, rb = 0;
     if (pass == 2 && s0 > 0) {
         uint32_t pa = 0, pb = 0;                     // bins before this segment
         for (int k = threadIdx.x; k < s0 / 4; k += kScanThreads) {
             const uint4 q = __ldg(reinterpret_cast<const uint4*>(count) + k);
             pa += q.x + q.y + q.z + q.w;
-            pb += (q.x + item_max - 1) / item_max + (q.y + item_max - 1) / item_max +
-                  (q.z + item_max - 1) / item_max + (q.w + item_max - 1) / item_max;
+            pb += rule.items(q.x) + rule.items(q.y) + rule.items(q.z) + rule.items(q.w);
         }
         pa = __reduce_add_sync(0xffffffffu, pa);
         pb = __reduce_add_sync(0xffffffffu, pb);
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_seg(
         item_off[n] = rb + ni;
     }
     if (!items) return;                              // (the allocation-free degrid path)
-    write_items(items, i - lane, lane, c, ni, ra, rb, item_max);
+    write_items(items, i - lane, lane, c, ni, ra, rb, rule);
 }
 
 // Exclusive scan of the segment totals in place (one CTA, nseg <= 32 * 1024);
@@ -315,14 +315,14 @@ __global__ void __launch_bounds__(kBinSmThreads) k_scatter_sm(
     // this CTA's run in each bin: absolute position of its first entry
     if constexpr (SCAN) {
         __shared__ uint32_t sa[32], sb[32];
-        const uint32_t item_max = (uint32_t)g.item_max;
+        const ItemRule rule(g);
         const int lane = threadIdx.x & 31;
         uint32_t ra = 0, rb = 0;                         // before the segment
 #pragma unroll
         for (int k = 0; k < kSegs; ++k) {
             if (k * kScanSeg >= ntiles) break;
             const int t = k * kScanSeg + (int)threadIdx.x;
-            const uint32_t c = cnt[k], ni = (c + item_max - 1) / item_max;
+            const uint32_t c = cnt[k], ni = rule.items(c);
             uint32_t ea = c, eb = ni;
             block_excl_scan2(ea, eb, sa, sb);
             ea += ra;
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kBinSmThreads) k_scatter_sm(
                     offsets[ntiles] = ra;
                     item_off[ntiles] = rb;
                 }
-                if (items) write_items(items, t - lane, lane, c, ni, ea, eb, item_max);
+                if (items) write_items(items, t - lane, lane, c, ni, ea, eb, rule);
             }
             __syncthreads();
         }
@@ -414,14 +414,14 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
         return;
     }
     if (ntiles <= kScanSingleMax || !sc.scan_tmp || ntiles > sc.scan_tmp_bins) {
-        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, (uint32_t)g.item_max, 2, nullptr, sc.offsets,
+        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, ItemRule(g), 2, nullptr, sc.offsets,
                                                  sc.item_off, sc.cursor, sc.items);
         note_launch();
     } else {
-        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, (uint32_t)g.item_max, 0, sc.scan_tmp,
+        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, ItemRule(g), 0, sc.scan_tmp,
                                                  sc.offsets, sc.item_off, sc.cursor, sc.items);
         k_scan_top<<<1, kScanThreads, 0, s>>>(sc.scan_tmp, nseg, ntiles, sc.offsets, sc.item_off);
-        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, (uint32_t)g.item_max, 1, sc.scan_tmp,
+        k_scan_seg<<<nseg, kScanThreads, 0, s>>>(sc.count, ntiles, ItemRule(g), 1, sc.scan_tmp,
                                                  sc.offsets, sc.item_off, sc.cursor, sc.items);
         note_launch(3);
     }
