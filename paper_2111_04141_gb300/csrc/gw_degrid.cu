@@ -34,10 +34,10 @@
 //   w-projection batch, 8.94 ms: 16-byte loads of staged points); before
 //   its instructions were cut 32 warps of 64 registers beat 24 of 80 there,
 //   9.34 against 9.52 ms, and 3.28 against 3.63 in bands.
-// * k_degrid_direct (small calls): one launch, index records included.
-// * k_degrid (the allocation-free entry point): the same per-record warp,
-//   reading the grid through L1/L2, records visited in 32 x 32 centre-tile
-//   order.
+// * k_degrid_direct (small calls): one launch, index records included; the same
+//   per-record warp, reading the grid through L1/L2.
+// * k_degrid (the allocation-free entry point, and degrid_kernel = 2): the same
+//   over binned records, visited in 32 x 32 centre-tile order.
 #include "gw_internal.cuh"
 
 namespace gw {
@@ -46,60 +46,93 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// A warp's sum of conj(K_i) G over one visibility's S x S footprint, read through
+// L1/L2, in every lane: kernel slice K, centre (ku, kv), sg = -1 for the conjugate
+// kernel.  Lanes take consecutive taps (t / S, t % S), the loads of four of a
+// lane's steps in flight: latency bounds it.  A loop over the rows with lanes
+// along them leaves lanes idle and the unrolling to the compiler, which took it
+// one way or the other with the length of a slice: 258 k, support 7-127, 8192^2,
+// x 4 4.6 or 9.7 ms, here 4.2; x 1 2.6, here 1.2.
+template <int NPOL, int TK>
+__device__ __forceinline__ void gather_sum(const DegridArgs& a, const typename TabElem<TK>::T* K,
+                                           int S, int ku, int kv, float sg, int lane,
+                                           float (&acc)[NPOL][2]) {
+    using TE = TabElem<TK>;
+    const int h = S >> 1, N = a.N;
+    // K.re G and K.im G apart, as in the staged kernel: half the length of the
+    // chains, and the sums of conj(K_i) at the end
+    float2 a1[NPOL], a2[NPOL];
+#pragma unroll
+    for (int p = 0; p < NPOL; ++p) a1[p] = a2[p] = make_float2(0.f, 0.f);
+    // tap (tv, tu), advanced without division
+    const int dq = 32 / S, dr = 32 - dq * S;
+    int tv = lane / S, tu = lane - tv * S;
+#pragma unroll 4
+    for (int t = lane; t < S * S; t += 32) {
+        const float2 k = TE::load(K + t);
+        const int64_t pix = (int64_t)(kv - h + tv) * N + (ku - h + tu);
+#pragma unroll
+        for (int p = 0; p < NPOL; ++p) {
+            const float2 g = __ldg(a.grid + (int64_t)p * N * N + pix);
+            a1[p].x = fmaf(k.x, g.x, a1[p].x);
+            a1[p].y = fmaf(k.x, g.y, a1[p].y);
+            a2[p].x = fmaf(k.y, g.x, a2[p].x);
+            a2[p].y = fmaf(k.y, g.y, a2[p].y);
+        }
+        tu += dr;
+        tv += dq;
+        if (tu >= S) {
+            tu -= S;
+            ++tv;
+        }
+    }
+    // (K.re - j s K.im) (G.re + j G.im)
+#pragma unroll
+    for (int p = 0; p < NPOL; ++p) {
+        acc[p][0] = fmaf(sg, a2[p].y, a1[p].x);
+        acc[p][1] = fmaf(-sg, a2[p].x, a1[p].y);
+    }
+#pragma unroll
+    for (int p = 0; p < NPOL; ++p)
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            acc[p][0] += __shfl_xor_sync(0xffffffffu, acc[p][0], d);
+            acc[p][1] += __shfl_xor_sync(0xffffffffu, acc[p][1], d);
+        }
+}
+
+// Stores visibility i from every lane's copy of the sums.
+template <int NPOL>
+__device__ __forceinline__ void store_sums(const DegridArgs& a, int64_t i, int lane,
+                                           const float (&acc)[NPOL][2]) {
+    if (lane < NPOL) {
+        float re = acc[0][0], im = acc[0][1];
+#pragma unroll
+        for (int p = 1; p < NPOL; ++p)
+            if (lane == p) { re = acc[p][0]; im = acc[p][1]; }
+        store_vis(a.vis_out, a.vis_kind, i * NPOL + lane, re * a.table_inv, im * a.table_inv);
+    }
+}
+
 template <int NPOL, int TK>
 __global__ void __launch_bounds__(kThreads) k_degrid(DegridArgs a) {
-    using TE = TabElem<TK>;
+    using TT = typename TabElem<TK>::T;
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const uint32_t n = *a.n_entries;
-    const int N = a.N;
     const int hb = a.beta / 2;
     for (int64_t e = warp0; e < n; e += nwarps) {
         const uint32_t id = __ldg(a.entries + e);
         int4 rv = __ldg(reinterpret_cast<const int4*>(a.rec) + id);
         const gw_index_rec r = *reinterpret_cast<gw_index_rec*>(&rv);
-        const int S = __ldg(a.support + r.plane), h = S >> 1;
-        const typename TE::T* K = reinterpret_cast<const typename TE::T*>(a.table) +
-                                  __ldg(a.plane_off + r.plane) +
-                                  ((int64_t)(r.ov + hb) * a.beta + (r.ou + hb)) * slice_elems(S);
+        const int S = __ldg(a.support + r.plane);
+        const TT* K = reinterpret_cast<const TT*>(a.table) + __ldg(a.plane_off + r.plane) +
+                      ((int64_t)(r.ov + hb) * a.beta + (r.ou + hb)) * slice_elems(S);
         // conj(K_i): K_i = K for w >= 0 (use conj K), K_i = conj K for w < 0 (use K)
-        const float s = (r.flags & GW_FLAG_CONJ) ? -1.f : 1.f;
         float acc[NPOL][2];
-#pragma unroll
-        for (int p = 0; p < NPOL; ++p) acc[p][0] = acc[p][1] = 0.f;
-        for (int tv = 0; tv < S; ++tv) {
-            const int64_t row = r.kv - h + tv;
-            for (int tu = lane; tu < S; tu += 32) {
-                const float2 k = TE::load(K + tv * S + tu);
-                const float ki = s * k.y;
-                const int64_t col = r.ku - h + tu;
-#pragma unroll
-                for (int p = 0; p < NPOL; ++p) {
-                    const float2 g = __ldg(a.grid + ((int64_t)p * N + row) * N + col);
-                    // (k.x - j ki) * (g.x + j g.y)
-                    acc[p][0] = fmaf(k.x, g.x, acc[p][0]);
-                    acc[p][0] = fmaf(ki, g.y, acc[p][0]);
-                    acc[p][1] = fmaf(k.x, g.y, acc[p][1]);
-                    acc[p][1] = fmaf(-ki, g.x, acc[p][1]);
-                }
-            }
-        }
-#pragma unroll
-        for (int p = 0; p < NPOL; ++p)
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                acc[p][0] += __shfl_xor_sync(0xffffffffu, acc[p][0], d);
-                acc[p][1] += __shfl_xor_sync(0xffffffffu, acc[p][1], d);
-            }
-        if (lane < NPOL) {
-            float re = acc[0][0], im = acc[0][1];
-#pragma unroll
-            for (int p = 1; p < NPOL; ++p)
-                if (lane == p) { re = acc[p][0]; im = acc[p][1]; }
-            store_vis(a.vis_out, a.vis_kind, (int64_t)id * NPOL + lane, re * a.table_inv,
-                      im * a.table_inv);
-        }
+        gather_sum<NPOL, TK>(a, K, S, r.ku, r.kv, (r.flags & GW_FLAG_CONJ) ? -1.f : 1.f, lane, acc);
+        store_sums<NPOL>(a, id, lane, acc);
     }
 }
 
@@ -126,7 +159,7 @@ constexpr int kDirectChanCache = 256;   // channel factors kept in shared memory
 template <int NPOL, int TK>
 __global__ void __launch_bounds__(kThreads) k_degrid_direct(DegridArgs a, DirectIndex di,
                                                             unsigned long long* __restrict__ work) {
-    using TE = TabElem<TK>;
+    using TT = typename TabElem<TK>::T;
     extern __shared__ long long sh_idx[];
     __shared__ unsigned long long s_cnt[3];   // the block's valid, taps, dropped
     const int nthr = di.p.P > 1 ? di.p.P - 1 : 0;
@@ -140,7 +173,7 @@ __global__ void __launch_bounds__(kThreads) k_degrid_direct(DegridArgs a, Direct
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int hb = a.beta / 2, N = a.N;
+    const int hb = a.beta / 2;
     const int64_t nvis = di.nrow * (int64_t)di.nchan;
     unsigned long long n_valid = 0, n_taps = 0, n_drop = 0;
     for (int64_t i = warp0; i < nvis; i += nwarps) {
@@ -159,13 +192,8 @@ __global__ void __launch_bounds__(kThreads) k_degrid_direct(DegridArgs a, Direct
         rv.z = __shfl_sync(0xffffffffu, rv.z, 0);
         rv.w = __shfl_sync(0xffffffffu, rv.w, 0);
         const gw_index_rec rc = *reinterpret_cast<const gw_index_rec*>(&rv);
-        // K.re G and K.im G apart, as in the staged kernel: half the length of
-        // the chains, and the sums of conj(K_i) at the end
-        float2 a1[NPOL], a2[NPOL];
-#pragma unroll
-        for (int p = 0; p < NPOL; ++p) a1[p] = a2[p] = make_float2(0.f, 0.f);
-        bool valid = (rc.flags & GW_FLAG_VALID) != 0;
-        const int S = valid ? __ldg(a.support + rc.plane) : 0, h = S >> 1;
+        const bool valid = (rc.flags & GW_FLAG_VALID) != 0;
+        const int S = valid ? __ldg(a.support + rc.plane) : 0;
         const int64_t kofs = valid ? __ldg(a.plane_off + rc.plane) +
                                          ((int64_t)(rc.ov + hb) * a.beta + (rc.ou + hb)) * slice_elems(S) : 0;
         if (lane == 0) {
@@ -175,57 +203,22 @@ __global__ void __launch_bounds__(kThreads) k_degrid_direct(DegridArgs a, Direct
         }
 #ifdef GW_DEBUG_BOUNDS
         // the slice, the footprint's pixels and the output row
+        const int h = S >> 1, N = a.N;
         if (valid && !gw_in_bounds((a.table_elems == 0 || (kofs >= 0 && kofs + (int64_t)S * S <= a.table_elems)) &&
                                        rc.ku - h >= 0 && rc.ku + h < N && rc.kv - h >= 0 && rc.kv + h < N &&
                                        (a.vis_count == 0 || i < a.vis_count),
                                    a.queue ? a.queue + 1 : nullptr))
             continue;
 #endif
-        const typename TE::T* K = reinterpret_cast<const typename TE::T*>(a.table) + kofs;
-        const float s = (rc.flags & GW_FLAG_CONJ) ? -1.f : 1.f;
-        // tap (tv, tu) = (t / S, t % S), advanced without division
-        const int dq = valid ? 32 / S : 0, dr = 32 - dq * S;
-        int tv = valid ? lane / S : 0, tu = lane - tv * S;
-#pragma unroll 4
-        for (int t = lane; t < S * S; t += 32) {
-            const float2 k = TE::load(K + t);
-            const int64_t pix = (int64_t)(rc.kv - h + tv) * N + (rc.ku - h + tu);
-#pragma unroll
-            for (int p = 0; p < NPOL; ++p) {
-                const float2 g = __ldg(a.grid + (int64_t)p * N * N + pix);
-                a1[p].x = fmaf(k.x, g.x, a1[p].x);
-                a1[p].y = fmaf(k.x, g.y, a1[p].y);
-                a2[p].x = fmaf(k.y, g.x, a2[p].x);
-                a2[p].y = fmaf(k.y, g.y, a2[p].y);
-            }
-            tu += dr;
-            tv += dq;
-            if (tu >= S) {
-                tu -= S;
-                ++tv;
-            }
-        }
-        // (K.re - j s K.im) (G.re + j G.im)
         float acc[NPOL][2];
+        if (valid) {
+            gather_sum<NPOL, TK>(a, reinterpret_cast<const TT*>(a.table) + kofs, S, rc.ku, rc.kv,
+                                 (rc.flags & GW_FLAG_CONJ) ? -1.f : 1.f, lane, acc);
+        } else {
 #pragma unroll
-        for (int p = 0; p < NPOL; ++p) {
-            acc[p][0] = fmaf(s, a2[p].y, a1[p].x);
-            acc[p][1] = fmaf(-s, a2[p].x, a1[p].y);
+            for (int p = 0; p < NPOL; ++p) acc[p][0] = acc[p][1] = 0.f;
         }
-#pragma unroll
-        for (int p = 0; p < NPOL; ++p)
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                acc[p][0] += __shfl_xor_sync(0xffffffffu, acc[p][0], d);
-                acc[p][1] += __shfl_xor_sync(0xffffffffu, acc[p][1], d);
-            }
-        if (lane < NPOL) {
-            float re = acc[0][0], im = acc[0][1];
-#pragma unroll
-            for (int p = 1; p < NPOL; ++p)
-                if (lane == p) { re = acc[p][0]; im = acc[p][1]; }
-            store_vis(a.vis_out, a.vis_kind, i * NPOL + lane, re * a.table_inv, im * a.table_inv);
-        }
+        store_sums<NPOL>(a, i, lane, acc);
     }
     // counts are held by lane 0 of each warp: one global atomic per block
     if (lane == 0) {

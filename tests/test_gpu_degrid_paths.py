@@ -86,6 +86,14 @@ def test_regions_in_bands(gw, npol, n, smin, smax, n_w):
     check(gw, obs, bands=True, degrid_kernel=1)
 
 
+# the global gather at supports of several warps' widths
+@pytest.mark.parametrize("npol,n,smin,smax,n_w", [(4, 400, 31, 127, 3), (2, 600, 41, 255, 3)])
+def test_gather_of_wide_supports(gw, npol, n, smin, smax, n_w):
+    obs = syn.small_case(n_ant=6, n_times=8, n_chan=2, npol=npol, grid_n=n, s_min=smin, s_max=smax,
+                         n_w=n_w, beta=2, diameter_m=1000.0, seed=29)
+    check(gw, drop_some(obs), degrid_kernel=2)
+
+
 # thousands of records centred in a few tiles (dense: 16 x 16 tiles), with
 # items of one chunk and of several
 @pytest.mark.parametrize("smax", [9, 71])
