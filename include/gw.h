@@ -133,8 +133,8 @@ typedef struct {
     int32_t item_max;       /* records per gridding / staged-degridding work item:
                                0 = automatic (gridding: 1020, and in gw_grid_vis,
                                _fresh, _host and _compensated 255 or 510 for small calls,
-                               in tiles of few records; staged degridding: 1024), else
-                               64 .. 2^20 (smaller items spread small jobs over more
+                               in tiles of few records; staged degridding: 128 to 1024
+                               by the size of the call), else 64 .. 2^20 (smaller items spread small jobs over more
                                SMs, larger ones commit less often) */
     int32_t degrid_kernel;  /* 0 = automatic (small chunks directly, in one launch, else
                                staged), 1 = shared-memory staged, 2 = global gather */

@@ -940,6 +940,29 @@ static const BinGeom& staged_geom(gw_plan p, int64_t nvis) {
     return p->geom_staged;
 }
 
+// Records per staged work item where the host knows their number: shorter ones
+// where kItemMax would leave SMs without one, as concentrated visibilities do
+// (kernels, us, 128 / 256 / 1,024 records: 48 k x 4 in a sixteenth of 1200^2,
+// support 7-127 362 / 428 / 890, spread over it 351 / 356 / 353; 516 k x 4 spread
+// 2,146 / 2,033 / 2,145).
+static void set_staged_items(gw_plan p, BinGeom& g, int64_t nvis) {
+    if (p->tuning.item_max > 0) return;
+    g.item_max = (int)std::min<int64_t>(std::max<int64_t>(nvis / (4 * p->num_sms), 128), kItemMax);
+}
+// Visibilities below which the gather kernels are taken instead of the staged one
+// on bins g: that one reads the regions of all tiles however few records they
+// have, a gather every tap through L1/L2, so the line is where the points of the
+// regions are the taps (of mean S^2).  Calls, us, staged / gather, 4 polarisations,
+// by points a tap: support 7-127, 8192^2 64-point tiles, 48 k visibilities (2.2)
+// 1,965 / 1,359, 129 k (0.8) 2,689 / 2,523; 4096^2, 4 k (6.7) 418 / 337, 16 k (1.7)
+// 575 / 614, 48 k (0.6) 800 / 973; support 7-33, 8192^2, 16 k (14) 452 / 108; support
+// 7-63, 4096^2 16 k (4) 278 / 177, 48 k (1.3) 362 / 295, 129 k (0.5) 474 / 563.  At least
+// 8,192: fewer make few items where they are concentrated (4 k of support 7-127 in a
+// sixteenth of 1200^2 363 / 146, spread 165 / 196).
+static int64_t staged_few(gw_plan p, const BinGeom& g) {
+    const double edge = (1 << g.su) + 2.0 * p->hmax;
+    return std::max<int64_t>((int64_t)(edge * edge * g.ntu * g.ntv / p->mean_s2), 8192);
+}
 // Taps of nvis visibilities on planes of the mean S^2, in those of one
 // polarisation: each further one costs half of the first.
 static double direct_taps(gw_plan p, int64_t nvis) {
@@ -951,7 +974,8 @@ static double direct_taps(gw_plan p, int64_t nvis) {
 // 132 / 79; 8192^2 x 4, 20 k 519 / 90; support 5, 60 k x 1 81 / 56; beyond the line
 // support 7-63, 16 k x 4 112 / 150 (before the kernel kept four taps in flight).
 static bool direct_size(gw_plan p, int64_t nvis) {
-    return nvis <= kDirectDegridVis && direct_taps(p, nvis) <= kDirectDegridTaps;
+    return (nvis <= kDirectDegridVis && direct_taps(p, nvis) <= kDirectDegridTaps) ||
+           (staged_banded(p->hmax, p->desc.npol) && nvis < staged_few(p, staged_geom(p, nvis)));
 }
 // Direct (unbinned) gridding of a chunk of nvis visibilities: forced by the
 // tuning, or automatic for small inputs.  The direct gridder's time grows with
@@ -1697,7 +1721,8 @@ gw_status gw_degrid_vis(gw_plan p, const double* uvw_m, const double* freq_hz, i
             e = cudaMemsetAsync(out, 0, vb * nr * nchan * npol, s);
             if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
             const bool staged = p->tuning.degrid_kernel != 2;
-            const BinGeom& geom = staged ? staged_geom(p, nr * nchan) : p->geom_degrid;
+            BinGeom geom = staged ? staged_geom(p, nr * nchan) : p->geom_degrid;
+            if (staged) set_staged_items(p, geom, nr * nchan);
             st = index_and_bin(p, uvw_m + 3 * r0, freq_hz, nr, nchan, geom, s);
             if (st != GW_OK) return st;
             a.rec = p->sc.rec;

@@ -115,6 +115,17 @@ def test_sparse_inputs_take_large_tiles(gw, npol, n, n_ant, n_times, smin, smax)
     check(gw, obs, bands=smax > 17, degrid_kernel=1)
 
 
+# wide supports, whose regions are served in bands: few visibilities take the
+# direct kernel (here up to 8,192), and concentrated ones short items
+@pytest.mark.parametrize("scale", [1.0, 0.1])
+@pytest.mark.parametrize("n_times,n", [(96, 400), (272, 400), (274, 400), (100, 1600)])
+def test_few_visibilities_of_wide_supports(gw, n_times, n, scale):
+    obs = syn.small_case(n_ant=6, n_times=n_times, n_chan=2, npol=4, grid_n=n, s_min=9, s_max=101,
+                         n_w=4, beta=2, diameter_m=2.5 * n, seed=33)
+    obs.uvw_m[:, :2] *= scale
+    check(gw, drop_some(obs), bands=True)
+
+
 # one launch for small calls against the staged kernel: the same sums in the
 # same order, at supports around a warp's 32 taps and every polarisation count
 @pytest.mark.parametrize("npol,n,smin,smax,n_w", [
