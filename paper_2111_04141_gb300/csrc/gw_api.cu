@@ -963,6 +963,19 @@ static int64_t staged_few(gw_plan p, const BinGeom& g) {
     const double edge = (1 << g.su) + 2.0 * p->hmax;
     return std::max<int64_t>((int64_t)(edge * edge * g.ntu * g.ntv / p->mean_s2), 8192);
 }
+// Bins of the staged degridder where only an upper bound of the visibilities is
+// known.  In bands 64 points serve any density (32 where those are too few
+// tiles): 129 k x 4, support 7-127, 8192^2 4.1 / 2.6 / 1.8 ms with 32 / 64 / 128, 516 k
+// x 4 on 1200^2 2.0 / 2.2 / 2.6 ms.  Items are of a length that suits few and many.
+static BinGeom devcount_geom(gw_plan p, int64_t nmax) {
+    const bool banded = staged_banded(p->hmax, p->desc.npol);
+    const BinGeom& g64 = p->geom_staged64;
+    BinGeom g = !banded ? staged_geom(p, nmax)
+                        : (g64.ntu * g64.ntv >= kStagedMinTiles ? g64 : p->geom_degrid);
+    if (p->tuning.item_max == 0) g.item_max = banded ? 256 : 512;
+    return g;
+}
+
 // Taps of nvis visibilities on planes of the mean S^2, in those of one
 // polarisation: each further one costs half of the first.
 static double direct_taps(gw_plan p, int64_t nvis) {
@@ -1923,7 +1936,7 @@ gw_status gw_degrid_vis_devcount(gw_plan p, const double* uvw_m, const double* f
     const int64_t nmax = max_nrow * (int64_t)nchan;
     launch_zero_vis(vis_out, vk, nmax, npol, dc, s);
     const bool staged = p->tuning.degrid_kernel != 2;
-    const BinGeom& geom = staged ? p->geom_staged : p->geom_degrid;
+    const BinGeom geom = staged ? devcount_geom(p, nmax) : p->geom_degrid;
     const IndexBins ib = index_bins(p, geom);
     const bool counted = launch_index(uvw_m, freq_hz, max_nrow, nchan, p->ip, p->sc.rec,
                                       p->sc.dropped, s, d_nrow, &ib);
@@ -1951,10 +1964,15 @@ gw_status gw_degrid_vis_devcount(gw_plan p, const double* uvw_m, const double* f
     a.queue = p->sc.counters;
     a.ntiles_u = geom.ntu;
     a.tile_shift = geom.su;
-    if (staged)
-        launch_degrid_staged(a, p->hmax, p->num_sms, s);
-    else
-        launch_degrid(a, nmax, p->num_sms, s);
+    int64_t few = 0;
+    if (p->tuning.degrid_kernel == 0) {
+        // the count on the device says which of the kernels works
+        few = staged_few(p, geom);
+        a.row_count = d_nrow;
+        a.few_rows = (few + nchan - 1) / nchan;
+    }
+    if (!staged || few > 0) launch_degrid(a, few > 0 ? std::min(nmax, few) : nmax, p->num_sms, s);
+    if (staged && max_nrow >= a.few_rows) launch_degrid_staged(a, p->hmax, p->num_sms, s);
     e = cudaGetLastError();
     return e == cudaSuccess ? GW_OK : cuda_fail(e, "degrid launch");
 }

@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(kThreads) k_degrid(DegridArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    if (a.row_count && *a.row_count >= a.few_rows) return;
     const uint32_t n = *a.n_entries;
     const int hb = a.beta / 2;
     for (int64_t e = warp0; e < n; e += nwarps) {
@@ -312,6 +313,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
     constexpr int NPR = NPOL / 2;
     extern __shared__ __align__(16) float4 reg[];
     __shared__ StagedChunk s_ch[2];
+    if (a.row_count && *a.row_count < a.few_rows) return;
     uint4* meta0;
     {
         const int pm = cap + kStagedPad;

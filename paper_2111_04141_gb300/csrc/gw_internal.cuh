@@ -547,6 +547,10 @@ struct DegridArgs {
     uint32_t* queue = nullptr;
     int ntiles_u = 0;
     int tile_shift = 4;         // centre tiles of 2^tile_shift points a side
+    // with row_count, k_degrid works on fewer than few_rows rows and the staged
+    // kernel on as many and more
+    const int64_t* row_count = nullptr;
+    int64_t few_rows = 0;
     // debug bounds checks (0: unknown, not checked)
     int64_t table_elems = 0;    // elements of `table`, slack included
     int64_t vis_count = 0;      // visibilities of vis_out

@@ -126,6 +126,30 @@ def test_few_visibilities_of_wide_supports(gw, n_times, n, scale):
     check(gw, drop_some(obs), bands=True)
 
 
+# a row count on the device: rows beyond it stay as they were, whichever kernel
+# serves the count (the gather below 8,192 visibilities or more)
+@pytest.mark.parametrize("npol,smin,smax", [(4, 9, 101), (4, 7, 33), (1, 5, 5)])
+def test_device_counts(gw, npol, smin, smax):
+    obs = syn.small_case(n_ant=10, n_times=110, n_chan=2, npol=npol, grid_n=500, s_min=smin, s_max=smax,
+                         n_w=4, beta=2, diameter_m=1200.0, seed=35)
+    prm = Params(**obs.plan_kwargs())
+    rng = np.random.default_rng(3)
+    shape = (npol, 500, 500)
+    grid = (rng.normal(size=shape) + 1j * rng.normal(size=shape)).astype(np.complex64)
+    ref = Oracle(prm).degrid(obs.uvw_m, obs.freq_hz, grid.astype(np.complex128))
+    ref = ref.reshape(obs.nrow, obs.nchan, npol)
+    uvw, freq = torch.from_numpy(obs.uvw_m).to(DEV), torch.from_numpy(obs.freq_hz).to(DEV)
+    g = torch.from_numpy(grid).to(DEV)
+    with gw.Plan.from_observation(obs) as plan:
+        for rows in (0, 1, 100, 4095, 4096, obs.nrow):
+            out = torch.full(ref.shape, 7.0, dtype=torch.complex64, device=DEV)
+            plan.degrid_devcount(uvw, freq, torch.tensor([rows], dtype=torch.int64, device=DEV), g, out)
+            plan.device_status()
+            v = out.cpu().numpy().astype(np.complex128)
+            assert np.all(v[rows:] == 7.0)
+            assert np.linalg.norm(v[:rows] - ref[:rows]) <= TOL * np.linalg.norm(ref[:rows])
+
+
 # one launch for small calls against the staged kernel: the same sums in the
 # same order, at supports around a warp's 32 taps and every polarisation count
 @pytest.mark.parametrize("npol,n,smin,smax,n_w", [
