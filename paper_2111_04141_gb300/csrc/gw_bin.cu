@@ -372,10 +372,9 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
                 Scratch& sc, cudaStream_t s, DevCount dc, bool counted) {
     const int ntiles = bin_count(g);
     if (!counted) cudaMemsetAsync(sc.count, 0, sizeof(uint32_t) * ntiles, s);
-    // per-CTA shared histograms when the bins fit and every CTA has at
-    // least ntiles pairs of a record and a bin (zeroing and flushing its histogram stays a small
-    // part of its work) with enough of them for kBinSmBlocksMin CTAs; smaller
-    // inputs keep the global-atomic kernels, which spread over all SMs
+    // per-CTA shared histograms where zeroing and flushing one stays a small
+    // part of a CTA's work (bin_sm_blocks); sparser inputs keep the
+    // global-atomic kernels, which spread over all SMs
     int sm_blocks = 0;
     const size_t hsm = sizeof(uint32_t) * (size_t)((ntiles + 3) / 4 * 4);
     if (bin_in_shared(nvis, g)) {

@@ -134,12 +134,11 @@ bool launch_index(const double* uvw, const double* freq, int64_t nrow, int nchan
                        bins->sc->cursor, bins->sc->work};
         mode = 1;
         if (bin_in_shared(nvis, bins->g)) {
-            // a CTA per ntiles pairs at least, as in the binner; where that
-            // leaves SMs idle and a thread more than one record, the FP64 work
-            // would wait for it: the counters themselves for moderate numbers
-            // of centre bins (255 k records over 4,096: 43 us for both stages
-            // against 50 counted apart), else counted apart (footprint bins
-            // contend more: 30 k over 512, 36 us with the counters, 29 in CTAs)
+            // the binner's CTAs; where those (more bins than kBinSmFewBins, or
+            // few records a bin) leave SMs idle and a thread more than one
+            // record, the FP64 work would wait for them: the counters
+            // themselves for moderate numbers of centre bins, else counted
+            // apart (footprint bins contend more)
             const size_t hsm = sizeof(uint32_t) * (size_t)((ntiles + 3) / 4 * 4);
             int per_sm = 0;
             if (tables + hsm <= kIndexSmemMax &&

@@ -348,18 +348,29 @@ __device__ __forceinline__ void each_bin(const gw_index_rec& r, const BinGeom& g
 // Histograms in shared memory: CTAs of kBinSmThreads threads.
 constexpr int kBinSmThreads = 1024;
 constexpr int kBinSmTilesMax = 49152;     // 192 KB of u32 counters
-// CTAs that get at least as many (record, bin) pairs as there are bins, and the
-// fewest of them worth it.  255 k pairs over 16,384 bins (15 CTAs) bin in 115 us
-// with shared histograms and 55 us with global atomics, 1.2 M over 32,768 (38
-// CTAs) in 290 and 120; 63 k over 512 (124 CTAs) in 24 and 39, 218 k over 1,568
-// (139 CTAs; 41 k records of supports to 109) in 30 and 109
-// together with the index stage.
+// CTAs of a kernel over nvis records: a CTA clears and flushes a counter per bin,
+// so it gets at least as many (record, bin) pairs as there are bins, and the
+// histograms are worth it from kBinSmBlocksMin CTAs (255 k pairs over 16,384 bins
+// in 15 CTAs 115 us, with global atomics 55, 1.2 M over 32,768 in 38 CTAs 290 and
+// 120).  Up to kBinSmFewBins bins that costs a CTA no more than 512 records do, and
+// global atomics contend where the records are concentrated, so there 8 records a
+// bin will do.  Index and bin stages, us, with global / shared counters, records
+// spread in a disk, in a spiral with a dense core, in a hundredth of the grid: 252 k
+// over 2,116 centre bins 48 / 36, 76 / 36, 95 / 30, 50 k over 4,096 31 / 33, 36 / 32,
+// 40 / 27, 24 k over 4,096 (5.9 a bin) 28 / 31, 30 / 30, 30 / 25; 252 k over 8,192
+// footprint bins 50 / 47, 79 / 46, 130 / 38, 50 k (6.2 a bin) 32 / 40, 39 / 40, 44 / 33.
 constexpr int kBinSmBlocksMin = 48;
+constexpr int kBinSmFewBins = 16384;
+inline bool bin_few(int64_t nvis, const BinGeom& g) {
+    return bin_count(g) <= kBinSmFewBins && nvis >= 8LL * bin_count(g);
+}
 inline int64_t bin_sm_blocks(int64_t nvis, const BinGeom& g) {
-    return (int64_t)((double)nvis * g.per_vis / bin_count(g));
+    const int64_t by_bins = (int64_t)((double)nvis * g.per_vis / bin_count(g));
+    return bin_few(nvis, g) ? std::max(by_bins, nvis / 512) : by_bins;
 }
 inline bool bin_in_shared(int64_t nvis, const BinGeom& g) {
-    return bin_count(g) <= kBinSmTilesMax && bin_sm_blocks(nvis, g) >= kBinSmBlocksMin;
+    return bin_count(g) <= kBinSmTilesMax &&
+           (bin_few(nvis, g) ? nvis >= 4096 : bin_sm_blocks(nvis, g) >= kBinSmBlocksMin);
 }
 
 // Cursors of the bins, by all CTAs of a kernel ahead of the scatter.
