@@ -874,6 +874,7 @@ static void set_grid_items(gw_plan p, BinGeom& g, int64_t nvis) {
     const double pairs = (double)nvis * g.per_vis;
     g.item_max = pairs >= 1020.0 * 8 * p->num_sms ? 1020 : (pairs >= 510.0 * 2.5 * p->num_sms ? 510 : 255);
     g.item_limit = 8u * (uint32_t)g.item_max;
+    g.item_grow = g.item_max == 255 ? 2 : (g.item_max == 510 ? 1 : 0);   // up to kItemLong
 }
 static BinGeom grid_geom(gw_plan p, int groups, int64_t nvis) {
     BinGeom g = p->geom_grid;

@@ -293,21 +293,23 @@ struct BinGeom {
     int group_planes = 1;  // planes per layer: 1 for w-stacking layers, more for plane groups
     float per_vis = 1.f;   // bins that a record of the mean plane meets
     uint32_t item_limit = 0xffffffffu;   // bins of more entries get longer items (ItemRule)
+    uint32_t item_grow = 0;
 };
-// Work items of a bin of c entries: runs of at most `len`; of twice as many, at
-// most kItemLong, in a bin of more than `limit` entries, and four times in one of
-// more than twice that.
+// Work items of a bin of c entries: runs of at most `len`; of twice as many in a
+// bin of more than `limit` entries and four times in one of more than twice that,
+// doubled `grow` times at most.
 struct ItemRule {
-    uint32_t len, limit;
-    __host__ __device__ explicit ItemRule(const BinGeom& g) : len(g.item_max), limit(g.item_limit) {}
-    __host__ __device__ uint32_t size(uint32_t c) const {
-        const int k = (c > limit) + (c / 2 > limit);
-        const uint32_t n = len << k;
-        return k > 0 && n > (uint32_t)kItemLong ? (uint32_t)kItemLong : n;
+    uint32_t len, limit, grow;
+    __host__ __device__ explicit ItemRule(const BinGeom& g)
+        : len(g.item_max), limit(g.item_limit), grow(g.item_grow) {}
+    __host__ __device__ uint32_t doublings(uint32_t c) const {
+        const uint32_t k = (c > limit) + (c / 2 > limit);
+        return k < grow ? k : grow;
     }
+    __host__ __device__ uint32_t size(uint32_t c) const { return len << doublings(c); }
     __host__ __device__ uint32_t items(uint32_t c) const {
-        const uint32_t n = size(c);
-        return (c + n - 1) / n;
+        const uint32_t k = doublings(c);     // (one divisor for all bins)
+        return ((c + len - 1) / len + (1u << k) - 1) >> k;
     }
 };
 inline int bin_count(const BinGeom& g) {
