@@ -183,7 +183,8 @@ struct gw_plan_s {
     std::vector<int64_t> pplane_off;
     int64_t* d_pplane_off = nullptr;
     // pair tables: FP32 complex kernels of at most kPairPolMax polarisations
-    // (instead of ptable), or tables and visibilities of one 16-bit kind
+    // (instead of ptable), or tables and visibilities of one 16-bit kind with
+    // kMmaPolMin polarisations and more
     void* pairs = nullptr;
     std::vector<int64_t> pair_off;
     int64_t* d_pair_off = nullptr;
@@ -610,7 +611,8 @@ gw_status gw_plan_create(const gw_plan_desc* desc, void* cuda_stream, gw_plan* o
         GW_ALLOC(pt, (size_t)p->pplane_off[P]);
         p->ptable = pt;
     }
-    if (pairs_only || (desc->table_dtype != GW_C64 && desc->vis_dtype == desc->table_dtype)) {
+    if (pairs_only || (desc->table_dtype != GW_C64 && desc->vis_dtype == desc->table_dtype &&
+                       desc->npol >= kMmaPolMin)) {
         p->pair_off.assign(1, 1);
         for (int q = 0; q < P; ++q)
             p->pair_off.push_back(p->pair_off[q] + pair_table_pairs(p->support[q], beta));

@@ -59,8 +59,11 @@
 //   visibilities of any kind are widened to FP32 when staged; all
 //   accumulation is FP32.  With an error grid the commit is compensated
 //   (commit_compensated).
-// * Where tables and visibilities are of one 16-bit kind and no weights are
-//   given, the compute warps are MmaWarp instead of FmaWarp: the same
+// * Where tables and visibilities are of one 16-bit kind, with two and more
+//   polarisations and no weights, the compute warps are MmaWarp instead of
+//   FmaWarp (kernels, us, of 1.41 M visibilities, support 7-83, 2348^2, 1 / 2 / 3 / 4
+//   polarisations: 1,473 / 1,443 / 1,476 / 1,451 against 1,394 / 1,666 / 2,012 /
+//   2,436; seven other shapes alike): the same
 //   producers, tiles and hand-over, the products on the tensor cores.  An
 //   FP32 warp issues 32 packed FMAs (two issue slots each) and about 40 other
 //   instructions for an entry of 128 points and 4 polarisations; the tensor
@@ -453,7 +456,7 @@ struct PairEntries {
         lo = (int64_t)(uint32_t)(e.x + (uint32_t)(j0 * Q + max(0, -pc)));
         hi = (int64_t)(uint32_t)(e.x + (uint32_t)(j1 * Q + min(kBlockU / 2 - 1, Q - 1 - pc)));
     }
-};;
+};
 
 // A pair of the FP32 table, zero where `on` is false: one predicated load.  (A
 // conditional one became a branch: 1 polarisation 2.94 ms, so 2.82.  With two
@@ -576,7 +579,12 @@ struct PairWarp {
 // block row: rows of A the row's 16 points, K index the records' (re, im)
 // kernel values as stored, columns of B the components (re, im) of the
 // polarisations.  Its FP32 sums are added to the lane's accumulators with
-// ordinary (rounded) additions.  Lane (g, t) = (lane / 4, lane % 4) loads
+// ordinary (rounded) additions.  The additions inside a product are not rounded
+// to nearest one by one: they lose 3e-8 of the sum, always downwards, but replace
+// sixteen roundings by one.  Errors against 64 bits on the stored values, here /
+// FmaWarp, bfloat16, items of 1,024: 96 k x 4, 256^2, support 7-31 1.33 / 2.10 e-7,
+// coherent 0.77 / 0.80 e-7; 29 k x 4, 1024^2, support 7-63 0.98 / 1.86 e-7, coherent 0.84 /
+// 1.15 e-7; float16 alike.  Lane (g, t) = (lane / 4, lane % 4) loads
 // column pair g of records t and t + 4 and holds polarisation t of points 2 g,
 // 2 g + 1; pairs come from the pair tables (layout at pair_table_pairs).
 template <int TK>
@@ -950,7 +958,7 @@ void launch_t(const GridArgs& a, int num_sms, cudaStream_t s) {
     if constexpr (TK == GW_C64 && NPOL <= kPairPolMax) {
         launch_sp<NPOL, 0, TK, true>(a, num_sms, s);       // such plans have pair tables only
     } else {
-        if constexpr (TK == GW_BF16X2 || TK == GW_F16X2) {
+        if constexpr ((TK == GW_BF16X2 || TK == GW_F16X2) && NPOL >= kMmaPolMin) {
             if (a.pair_table && a.vis_kind == TK && !a.weight) {
                 launch_sp<NPOL, 0, TK, true>(a, num_sms, s);
                 return;

@@ -537,6 +537,7 @@ inline int64_t pair_table_pairs(int S, int beta) {
     return (int64_t)beta * beta * S * (S + 1);
 }
 constexpr int kPairPolMax = 2;
+constexpr int kMmaPolMin = 2;      // polarisations of the 16-bit tensor-core gridder
 // tab and pairs hold elements of kind `kind` (8 bytes for GW_C64, else 4).
 void launch_pair_tables(const void* tab, int kind, const int64_t* plane_off,
                         const int64_t* pair_off, const int* support, int P, int beta, void* pairs,
