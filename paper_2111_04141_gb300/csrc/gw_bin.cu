@@ -381,9 +381,12 @@ void launch_bin(const gw_index_rec* rec, int64_t nvis, const BinGeom& g, int P, 
         int dev = 0, nsm = 0, c_sm = 0, s_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_count_sm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm);
-        cudaFuncSetAttribute(k_scatter_sm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm);
-        cudaFuncSetAttribute(k_scatter_sm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm);
+        // (the most that any call needs: another thread may be between its
+        // setting and its launch)
+        const int most = (int)sizeof(uint32_t) * kBinSmTilesMax;
+        cudaFuncSetAttribute(k_count_sm, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        cudaFuncSetAttribute(k_scatter_sm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        cudaFuncSetAttribute(k_scatter_sm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c_sm, k_count_sm, kBinSmThreads, hsm);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
             &s_sm, ntiles <= kScanFusedMax ? k_scatter_sm<true> : k_scatter_sm<false>, kBinSmThreads, hsm);

@@ -663,8 +663,12 @@ void launch_staged_g(const DegridArgs& a, int hmax, size_t cap, size_t part, int
                      cudaStream_t s) {
     const size_t smem = (cap + kStagedPad) * NPOL * sizeof(float2) +
                         2 * kStagedMeta * sizeof(uint4) + part;
+    // (the most that any call needs: another thread may be between its setting
+    // and its launch)
+    constexpr size_t most = kStagedSmemMax + kStagedPad * NPOL * sizeof(float2) +
+                            2 * kStagedMeta * sizeof(uint4);
     cudaFuncSetAttribute(k_degrid_staged<NPOL, TK, GEN>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     k_degrid_staged<NPOL, TK, GEN><<<num_sms, kStagedThreads, smem, s>>>(a, hmax, (int)cap);
     note_launch();
 }

@@ -1,4 +1,4 @@
-"""Calls given another stream than the current one: arrays that the call
+"""Streams and threads.  Calls given another stream than the current one: arrays that the call
 allocates (and clears) on the current stream, and the imaging chains, whose
 transforms torch.fft runs on the current stream, are ordered between the two.
 The current stream is held up ahead of each call (a bounded device-side delay
@@ -112,3 +112,39 @@ def test_imaging_on_another_stream(gw, chain):
                 assert torch.linalg.vector_norm(got - want) <= 1e-6 * torch.linalg.vector_norm(want)
             else:
                 assert close(got, want)
+
+
+def test_threads_with_plans_of_different_sizes(gw):
+    """Two threads, each with its plan and stream, launch the same kernels with
+    different amounts of shared memory: neither's launch may be refused."""
+    import threading
+    plans, failures = [], []
+    for smax, n in ((5, 256), (71, 700)):
+        obs = syn.small_case(n_ant=12, n_times=80, n_chan=1, npol=2, grid_n=n, s_min=5, s_max=smax,
+                             n_w=3, beta=2, diameter_m=1500.0, seed=53)
+        uvw, freq, vis = (torch.from_numpy(a).to(DEV) for a in (obs.uvw_m, obs.freq_hz, obs.vis))
+        plan = gw.Plan.from_observation(obs)
+        plan.set_tuning(grid_kernel=1, degrid_kernel=1)
+        plans.append((plan, uvw, freq, vis, plan.grid(uvw, freq, vis)))
+    torch.cuda.synchronize()
+
+    def work(plan, uvw, freq, vis, model):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                first = plan.degrid(uvw, freq, model)
+                for _ in range(400):
+                    plan.grid(uvw, freq, vis)
+                    v = plan.degrid(uvw, freq, model)
+                torch.cuda.current_stream().synchronize()
+                assert torch.linalg.vector_norm(v - first) <= 1e-5 * torch.linalg.vector_norm(first)
+        except Exception as e:                       # reported by the main thread
+            failures.append(e)
+
+    threads = [threading.Thread(target=work, args=p) for p in plans]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for p in plans:
+        p[0].close()
+    assert not failures, failures
