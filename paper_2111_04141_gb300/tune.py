@@ -4,7 +4,10 @@ timing candidates on a sample job (CUDA events on the launching stream).
 The candidates are the plan tunables (gw_tuning): records per work item,
 which trades SM load balance on small or sparse jobs against commit
 traffic, and the degridding kernel (shared-memory staged tiles or global
-gather).  The best configuration is kept in a dict (and, optionally, a JSON
+gather), each with the plan's own choice by the size of the call (0), which a
+tuned plan would otherwise lose for jobs of other sizes than the sample's.
+Item sizes are multiples of the 255 records that every gridder stages at a
+time.  The best configuration is kept in a dict (and, optionally, a JSON
 file) keyed by the setup's name or by ``plan_key(plan)``: the plan
 parameters the timings depend on and the device's SM count.
 """
@@ -14,8 +17,8 @@ import json
 import os
 from typing import Dict, Iterable, Optional
 
-ITEM_CANDIDATES = (256, 512, 1024, 2048, 4096)
-DEGRID_CANDIDATES = (1, 2)
+ITEM_CANDIDATES = (0, 255, 510, 1020, 2040, 4080)
+DEGRID_CANDIDATES = (0, 1, 2)
 
 
 def _time(fn, stream, reps: int) -> float:

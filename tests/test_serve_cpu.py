@@ -258,3 +258,12 @@ def test_tuning_cache_keys_by_plan_parameters_and_persists(tmp_path):
     c.put(k, {"item_max": 2048, "degrid_kernel": 1, "grid_kernel": 0, "compress_min_gain": 0})
     assert TuningCache(path).get(k)["item_max"] == 2048
     assert TuningCache(path).get("other") is None
+
+
+def test_autotuner_offers_the_plans_own_choice():
+    """0 (chosen by the size of each call) is a candidate of both tunables, first
+    so that it keeps a tie; the other item sizes are whole batches of the gridders."""
+    from paper_2111_04141_gb300.tune import DEGRID_CANDIDATES, ITEM_CANDIDATES
+    assert ITEM_CANDIDATES[0] == 0 and DEGRID_CANDIDATES[0] == 0
+    assert set(DEGRID_CANDIDATES) == {0, 1, 2}
+    assert all(i % 255 == 0 for i in ITEM_CANDIDATES)
