@@ -1,9 +1,9 @@
 """The debug build (libgw_debug.so, GW_DEBUG_BOUNDS): its kernels check their
 indices against their buffers, record a failed check in the plan's device
 status word and skip the access.  On valid inputs no check may fire, and the
-results must be those of the release build: gridding (binned and direct),
-degridding (staged and gather) and the banded read-back, against the FP64
-oracle.  Run in a child process, which loads the debug library."""
+results must be those of the release build: gridding (binned, direct and on
+the 16-bit pair tables), degridding (direct, staged and gather) and the banded
+read-back, against the FP64 oracle.  Run in a child process, which loads the debug library."""
 import os
 import subprocess
 import sys
@@ -43,7 +43,7 @@ for npol, smax in ((4, 21), (3, 13), (1, 31)):
             g = plan.grid(uvw, freq, vis).cpu().numpy().astype(np.complex128)
             plan.device_status()
             assert rel(g, ref) <= 1e-5, (npol, gk, rel(g, ref))
-        for dk in (1, 2):
+        for dk in (0, 1, 2):                     # direct (small calls), staged, gather
             plan.set_tuning(**dict(plan.get_tuning(), degrid_kernel=dk))
             v = plan.degrid(uvw, freq, torch.from_numpy(g0).to(dev)).cpu().numpy()
             plan.device_status()
@@ -55,6 +55,14 @@ for npol, smax in ((4, 21), (3, 13), (1, 31)):
         plan.grid_devcount_readback(uvw, freq, d_nrow, vis, out, host, n_bands=3)
         plan.device_status()
         assert rel(host.numpy().astype(np.complex128), ref) <= 1e-5
+    if npol == 4:                                # the tensor-core gridder's pair tables
+        from paper_2111_04141_gb300.plan import to_storage
+        v16 = to_storage(torch.from_numpy(obs.vis), "bf16").to(dev)
+        with gw.Plan.from_observation(obs, table_dtype="bf16", vis_dtype="bf16") as plan:
+            plan.set_tuning(grid_kernel=1)
+            g = plan.grid(uvw, freq, v16).cpu().numpy().astype(np.complex128)
+            plan.device_status()
+            assert rel(g, ref) <= 5e-3, rel(g, ref)     # bfloat16 storage
 print("debug-bounds ok")
 """
 

@@ -150,8 +150,10 @@ def test_device_counts(gw, npol, smin, smax):
             assert np.linalg.norm(v[:rows] - ref[:rows]) <= TOL * np.linalg.norm(ref[:rows])
 
 
-# one launch for small calls against the staged kernel: the same sums in the
-# same order, at supports around a warp's 32 taps and every polarisation count
+# one launch for small calls against the staged kernel, both over a warp's
+# flattened taps, at supports around its 32 lanes and every polarisation count.
+# They fold the lanes' sums alike except for 3 polarisations and where bands cut
+# a sum: a few roundings of 2^-24, 3e-7 of the root mean square
 @pytest.mark.parametrize("npol,n,smin,smax,n_w", [
     (1, 130, 1, 1, 1), (2, 98, 5, 7, 2), (3, 142, 31, 33, 3), (4, 300, 5, 65, 4), (1, 600, 41, 255, 3)])
 def test_direct_equals_staged(gw, npol, n, smin, smax, n_w):
@@ -163,4 +165,4 @@ def test_direct_equals_staged(gw, npol, n, smin, smax, n_w):
     direct, dropped, _ = degrid(gw, obs, grid, True, degrid_kernel=0)
     staged, again, _ = degrid(gw, obs, grid, True, degrid_kernel=1)
     assert dropped == again
-    assert np.linalg.norm(direct - staged) <= 2 * TOL * np.linalg.norm(staged)
+    assert np.linalg.norm(direct - staged) <= 3e-7 * np.linalg.norm(staged)
