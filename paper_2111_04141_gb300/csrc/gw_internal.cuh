@@ -355,16 +355,16 @@ constexpr int kBinSmTilesMax = 49152;     // 192 KB of u32 counters
 // histograms are worth it from kBinSmBlocksMin CTAs (255 k pairs over 16,384 bins
 // in 15 CTAs 115 us, with global atomics 55, 1.2 M over 32,768 in 38 CTAs 290 and
 // 120).  Up to kBinSmFewBins bins that costs a CTA no more than 512 records do, and
-// global atomics contend where the records are concentrated, so there 8 records a
+// global atomics contend where the records are concentrated, so there 16 pairs a
 // bin will do.  Index and bin stages, us, with global / shared counters, records
 // spread in a disk, in a spiral with a dense core, in a hundredth of the grid: 252 k
-// over 2,116 centre bins 48 / 36, 76 / 36, 95 / 30, 50 k over 4,096 31 / 33, 36 / 32,
-// 40 / 27, 24 k over 4,096 (5.9 a bin) 28 / 31, 30 / 30, 30 / 25; 252 k over 8,192
-// footprint bins 50 / 47, 79 / 46, 130 / 38, 50 k (6.2 a bin) 32 / 40, 39 / 40, 44 / 33.
+// over 2,116 centre bins 48 / 36, 76 / 36, 95 / 30, 50 k over 4,096 (12
+// a bin) 31 / 33, 36 / 32, 40 / 27; 252 k over 8,192 footprint bins (43) 50 / 47, 79 / 46,
+// 130 / 38, 50 k (9) 32 / 40, 39 / 40, 44 / 33.
 constexpr int kBinSmBlocksMin = 48;
 constexpr int kBinSmFewBins = 16384;
 inline bool bin_few(int64_t nvis, const BinGeom& g) {
-    return bin_count(g) <= kBinSmFewBins && nvis >= 8LL * bin_count(g);
+    return bin_count(g) <= kBinSmFewBins && (double)nvis * g.per_vis >= 16.0 * bin_count(g);
 }
 inline int64_t bin_sm_blocks(int64_t nvis, const BinGeom& g) {
     const int64_t by_bins = (int64_t)((double)nvis * g.per_vis / bin_count(g));

@@ -25,13 +25,13 @@ def gw():
 
 
 # records and bins: 76,000 over 128 (shared, several records a thread), 30,400
-# over 512 (shared, few CTAs), 152,000 over 2,048 (counted by the binner, or with
-# centre bins the bins' counters), 7,600 over 2,048 (the bins' counters),
-# channels past the cached factors, and more bins than one kernel scans and
-# scatters (8,192), shared
+# over 512 (shared, few CTAs), 152,000, 30,400 (with footprints 19 pairs a bin,
+# shared; with centres 7), 15,200 (10 and 4, the bins' counters) and 7,600 over
+# 2,048 or 4,096, channels past the cached factors, and more bins than one kernel
+# scans and scatters (8,192), with centres more than 16,384
 @pytest.mark.parametrize("n,n_ant,n_times,n_chan,n_w", [
-    (512, 20, 100, 4, 5), (1024, 20, 40, 4, 1), (2048, 20, 200, 4, 3), (2048, 20, 10, 4, 7),
-    (512, 4, 3, 1500, 2), (4222, 20, 700, 4, 3)])
+    (512, 20, 100, 4, 5), (1024, 20, 40, 4, 1), (2048, 20, 200, 4, 3), (2048, 20, 40, 4, 3),
+    (2048, 20, 20, 4, 3), (2048, 20, 10, 4, 7), (512, 4, 3, 1500, 2), (4222, 20, 700, 4, 3)])
 @pytest.mark.parametrize("mode", [0, 1])
 def test_every_bin_holds_its_records(gw, n, n_ant, n_times, n_chan, n_w, mode):
     obs = syn.small_case(n_ant=n_ant, n_times=n_times, n_chan=n_chan, npol=1, grid_n=n, s_min=5,
