@@ -267,3 +267,23 @@ def test_autotuner_offers_the_plans_own_choice():
     assert ITEM_CANDIDATES[0] == 0 and DEGRID_CANDIDATES[0] == 0
     assert set(DEGRID_CANDIDATES) == {0, 1, 2}
     assert all(i % 255 == 0 for i in ITEM_CANDIDATES)
+
+
+@pytest.mark.parametrize("fast,want", [(0.98, (0, 0)), (0.9, (510, 1))])
+def test_autotuner_keeps_the_plans_own_choice_in_a_tie(monkeypatch, fast, want):
+    """Another candidate within the scatter of the timings does not replace it."""
+    import torch
+    from paper_2111_04141_gb300 import tune
+
+    class Plan:
+        device = None
+
+        def set_tuning(self, item_max=0, degrid_kernel=0, **rest):
+            self.now = (item_max, degrid_kernel)
+
+    plan = Plan()
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device=None: None)
+    monkeypatch.setattr(tune, "_time", lambda fn, stream, reps: fast if plan.now == (510, 1) else 1.0)
+    res = tune.tune_plan(plan, None, None, torch.zeros(1), None)
+    assert (res["tuning"]["item_max"], res["tuning"]["degrid_kernel"]) == want == plan.now
+    assert res["ms"] == (1.0 if want == (0, 0) else fast)
