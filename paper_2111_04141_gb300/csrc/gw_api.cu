@@ -987,8 +987,9 @@ static double direct_taps(gw_plan p, int64_t nvis) {
 // Direct (unbinned) degridding of small inputs.  Calls, us, staged / direct
 // (support 7-33, mean S^2 456, unless named): 1024^2, 16 k visibilities x 1 72 / 29,
 // x 4 82 / 40, uv within a tenth of the grid x 4 118 / 39, 60 k x 1 93 / 79; 4096^2 x 1, 60 k
-// 132 / 79; 8192^2 x 4, 20 k 519 / 90; support 5, 60 k x 1 81 / 56; beyond the line
-// support 7-63, 16 k x 4 112 / 150 (before the kernel kept four taps in flight).
+// 132 / 79; 8192^2 x 4, 20 k 519 / 90; support 5, 60 k x 1 81 / 56.  Beyond the line, on
+// 1024^2: support 7-33, 48 k x 4 105 / 89, 129 k x 1 124 / 152, x 4 155 / 203; 7-63, 16 k x 4
+// 103 / 68, 48 k x 4 149 / 165; 7-127, 16 k x 1 154 / 127, 48 k x 1 225 / 275.
 static bool direct_size(gw_plan p, int64_t nvis) {
     return (nvis <= kDirectDegridVis && direct_taps(p, nvis) <= kDirectDegridTaps) ||
            (staged_banded(p->hmax, p->desc.npol) && nvis < staged_few(p, staged_geom(p, nvis)));

@@ -8,8 +8,9 @@
 // Three kernels:
 // * k_degrid_staged (used by gw_degrid_vis): one CTA of 32 warps per SM
 //   serves chunks of work items (at most 1,024 records centred in one tile of
-//   16 x 16 points, or 32 x 32 to 128 x 128 for sparse inputs).  Warps 0-3
-//   load the records' metadata (id, kernel slice, centre, support) into one of two shared buffers, the next chunk's while all
+//   16 x 16 points, or 32 x 32 to 128 x 128 for sparse inputs and wide
+//   supports).  Warps 0-3 load the records' metadata (id, kernel slice, centre,
+//   support) into one of two shared buffers, the next chunk's while all
 //   warps compute the current one.  The CTA stages the tile's grid region
 //   (the tile plus the chunk's largest half-support on every side) in
 //   shared memory once, as polarisation pairs, at a row pitch padded to the
@@ -33,7 +34,8 @@
 //   taps share a region 5.2.)  The L1 data pipe bounds it (90 % on the 4-pol
 //   w-projection batch, 8.94 ms: 16-byte loads of staged points); before
 //   its instructions were cut 32 warps of 64 registers beat 24 of 80 there,
-//   9.34 against 9.52 ms, and 3.28 against 3.63 in bands.
+//   9.34 against 9.52 ms, and 3.28 against 3.63 in bands, although some variants
+//   spill (FP32 x 4: 88 bytes stored, 52 loaded).
 // * k_degrid_direct (small calls): one launch, index records included; the same
 //   per-record warp, reading the grid through L1/L2.
 // * k_degrid (the allocation-free entry point, and degrid_kernel = 2): the same
@@ -336,11 +338,11 @@ __global__ void __launch_bounds__(kStagedThreads) k_degrid_staged(DegridArgs a, 
     int next_c0 = 0;
 
     // The loader warps (0-3) pick the next chunk and load its records'
-    // metadata (id, kernel slice offset, centre relative to the tile,
-    // support | conj << 16) into buffer `buf`, records wider than h_max / 2
+    // metadata (id, kernel slice offset, centre relative to the tile, the word
+    // of kMetaSupport) into buffer `buf`, records wider than h_max / 2
     // first: warps claim records in this order, so the long ones start early
     // and the short ones even out the end of the chunk.  Each loader thread
-    // issues the loads of its (up to 8) records together.
+    // issues the loads of its (up to 8) records kLoaderBatch at a time.
     auto load_chunk = [&](const int buf) {
         StagedChunk& c = s_ch[buf];
         if (threadIdx.x == 0) {

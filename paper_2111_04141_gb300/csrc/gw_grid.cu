@@ -87,8 +87,9 @@ __global__ void k_weight_vis(const void* __restrict__ vis, int kind, const float
 // whose lane 0 computes the visibility's index record (the same bit-exact
 // FP64 sequence as the index stage) and broadcasts it, then spreads it over
 // the flattened S x S taps of its (unpadded) kernel slice with one global
-// vector atomic per tap and polarisation.  One launch per call instead of
-// the binned path's seven, which is what small jobs pay for.  Counts the
+// vector atomic per tap and polarisation.  One launch per call instead of the
+// binned path's three or four kernels, each of which waits for the one before:
+// that is what small jobs pay for.  Counts the
 // dropped visibilities and accumulates the work counters the binner would
 // (valid records, sum of S^2).
 constexpr int kDirectChanCache = 256;   // channel factors kept in shared memory

@@ -459,9 +459,10 @@ struct PairEntries {
 };
 
 // A pair of the FP32 table, zero where `on` is false: one predicated load.  (A
-// conditional one became a branch: 1 polarisation 2.94 ms, so 2.82.  With two
-// polarisations, and in FmaWarp, the conditional loads schedule better: 1.57
-// against 1.59 ms and 8.23 against 8.79.)
+// conditional one became a branch: 4.2 M visibilities x 1, support 31, 2.94 ms, so
+// 2.82.  With two polarisations, and in FmaWarp, the conditional loads schedule
+// better: the same x 2 3.887 against 3.957 ms (eight runs each, all within 0.005 of
+// that) and the 4096^2 batch 8.23 against 8.79.)
 __device__ __forceinline__ float4 load_pair(const float4* __restrict__ p, bool on) {
     float4 v;
     asm("{.reg .pred q; setp.ne.u32 q, %5, 0;\n"

@@ -3,6 +3,7 @@ slot affinity, latency statistics, and the serving-stream generator."""
 import math
 
 import numpy as np
+import pytest
 
 import synthetic as syn
 from paper_2111_04141_gb300.serve import Job, Scheduler, latency_stats
