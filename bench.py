@@ -40,8 +40,8 @@ FFMA_PER_SM_PER_CLK = 128
 
 # DRAM traffic of the gridding kernel from one ncu capture, valid only for the
 # kernel source it was taken on (sha256 of gw_grid_kernel.cuh); null otherwise.
-GRID_TRAFFIC = {"sha256": "7f1d6b08e8ace1744f53a0b6c51b489ff5bf98e59b2c4261b42e85713275b78b",
-                "bytes_per_launch": 0.963154e9 + 0.264228e9,
+GRID_TRAFFIC = {"sha256": "087b4ff4f8c99d6a300db14a178f4322f0c90b3b7b8f4f8fbde08d5ba46ccb94",
+                "bytes_per_launch": 0.963227e9 + 0.263536e9,
                 "capture": "profiles/k_grid_wproj4096.md"}
 
 
