@@ -1968,15 +1968,16 @@ gw_status gw_degrid_vis_devcount(gw_plan p, const double* uvw_m, const double* f
     a.queue = p->sc.counters;
     a.ntiles_u = geom.ntu;
     a.tile_shift = geom.su;
-    int64_t few = 0;
-    if (p->tuning.degrid_kernel == 0) {
-        // the count on the device says which of the kernels works
-        few = staged_few(p, geom);
+    // few visibilities: the gather; where the bound allows few and many, both
+    // are launched and the count on the device says which of them works
+    const int64_t few_rows = p->tuning.degrid_kernel == 0 ? (staged_few(p, geom) + nchan - 1) / nchan
+                                                          : (staged ? 0 : INT64_MAX);
+    if (few_rows > 0 && max_nrow >= few_rows) {
         a.row_count = d_nrow;
-        a.few_rows = (few + nchan - 1) / nchan;
+        a.few_rows = few_rows;
     }
-    if (!staged || few > 0) launch_degrid(a, few > 0 ? std::min(nmax, few) : nmax, p->num_sms, s);
-    if (staged && max_nrow >= a.few_rows) launch_degrid_staged(a, p->hmax, p->num_sms, s);
+    if (few_rows > 0) launch_degrid(a, std::min(max_nrow, few_rows) * nchan, p->num_sms, s);
+    if (max_nrow >= few_rows) launch_degrid_staged(a, p->hmax, p->num_sms, s);
     e = cudaGetLastError();
     return e == cudaSuccess ? GW_OK : cuda_fail(e, "degrid launch");
 }

@@ -141,7 +141,7 @@ def test_device_counts(gw, npol, smin, smax):
     uvw, freq = torch.from_numpy(obs.uvw_m).to(DEV), torch.from_numpy(obs.freq_hz).to(DEV)
     g = torch.from_numpy(grid).to(DEV)
     with gw.Plan.from_observation(obs) as plan:
-        for rows in (0, 1, 100, 4095, 4096, obs.nrow):
+        for rows in (0, 1, 100, 4095, 4096, obs.nrow, obs.nrow + 7):     # (at most all)
             out = torch.full(ref.shape, 7.0, dtype=torch.complex64, device=DEV)
             plan.degrid_devcount(uvw, freq, torch.tensor([rows], dtype=torch.int64, device=DEV), g, out)
             plan.device_status()
