@@ -132,13 +132,15 @@ typedef struct {
 typedef struct {
     int32_t item_max;       /* records per gridding / staged-degridding work item:
                                0 = automatic (gridding: 1020, and in gw_grid_vis,
-                               _fresh, _host and _compensated 255 or 510 for small calls,
-                               in tiles of few records; staged degridding: 128 to 1024
-                               by the size of the call, 256 or 512 in
-                               gw_degrid_vis_devcount), else 64 .. 2^20 (smaller items spread small jobs over more
-                               SMs, larger ones commit less often) */
-    int32_t degrid_kernel;  /* 0 = automatic (small chunks directly, in one launch, else
-                               staged; gw_degrid_vis_devcount: the gather for few
+                               _fresh, _host and _compensated 255 or 510 for small
+                               calls, in tiles of few records; staged degridding: 128
+                               to 1024 by the size of the call, 256 or 512 in
+                               gw_degrid_vis_devcount), else 64 .. 2^20 (smaller items
+                               spread small jobs over more SMs, larger ones commit less
+                               often) */
+    int32_t degrid_kernel;  /* 0 = automatic (small chunks, and few visibilities of wide
+                               supports, directly in one launch, else staged;
+                               gw_degrid_vis_devcount: the gather for few
                                visibilities, else staged),
                                1 = shared-memory staged, 2 = global gather */
     int32_t grid_kernel;    /* gw_grid_vis / _compensated: 0 = automatic (direct for chunks of
